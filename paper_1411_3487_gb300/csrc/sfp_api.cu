@@ -1291,7 +1291,7 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
             std::vector<double> w = g.tab.w;
             w[0] = g.tab.w0;
             rc = sfp::fused_create(&g.fused, M, g.C, g.tab.chi.data(), g.tab.phi.data(), g.tab.h.data(), w.data(),
-                                   (float*)g.R, b->stream, bf16, two);
+                                   g.tab.dm.data(), g.tab.g.data(), (float*)g.R, b->stream, bf16, two);
             if (rc) { destroy_impl(b); return rc; }
         }
         if (precision == SFP_FP64 && M <= kChainMaxBeads) {

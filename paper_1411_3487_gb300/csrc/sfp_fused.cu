@@ -2,6 +2,11 @@
 // the SFP_FP32 and SFP_MIXED_BF16 paths, M = 64, 128, 256 or 512 beads,
 // n_steps per launch.
 //
+// SFP_MIXED_BF16 chains of 64, 128 and 256 beads with bead noise take the lane
+// step (sfp_lanes.cuh: bonds and modes on the TMEM lanes), launched from here;
+// the kernels below serve the TF32 and two-pass splits, mode-keyed noise, and
+// 512 beads.
+//
 // The 128 TMEM lanes hold a tile's chain-axis rows: lane quarter q (rows
 // 32 q .. 32 q + 31) holds chains q cpq .. q cpq + cpq - 1 of the tile
 // (cpq <= 10 chains per quarter), chain k of the quarter in rows 32 q + 3 k +
@@ -75,6 +80,7 @@
 #include "../../include/sfp.h"
 #include "sfp_device.cuh"
 #include "sfp_fused.h"
+#include "sfp_lanes.cuh"
 #include "sfp_ptx.cuh"
 
 namespace sfp {
@@ -952,6 +958,19 @@ k_fused_step(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CU
     tmem_free<2 * NB>(tmem);
 }
 
+// One tile per CTA, bonds and modes on the TMEM lanes (sfp_lanes.cuh).
+template <int M>
+__global__ void __launch_bounds__(lanes::kThreads, 1)
+k_lane_step(const FusedArgs a, const lanes::LaneArgs la)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint32_t s_tmem;
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    tmem_alloc<lanes::Geo<M>::kCols>(&s_tmem);
+    const uint32_t tmem = s_tmem;
+    lanes::lane_tile<M>(a, la, blockIdx.x, smem, tmem);
+    tmem_free<lanes::Geo<M>::kCols>(tmem);
+}
 
 // The 512-bead step: tile `tile` on a cluster of two CTAs, CTA h (its rank)
 // holding bonds and modes 256 h .. 256 h + 255 (see the file's header).  The
@@ -1566,6 +1585,7 @@ k_fused_pair(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CU
 // the longest tiles start first and the short ones fill the tail.
 struct GroupSlot {
     CUtensorMap tmR, tmChiH, tmChiL, tmFH, tmFL;
+    lanes::LaneArgs la;
     FusedArgs a;
     int tiles;      // 0: the slot is unused
 };
@@ -1575,16 +1595,23 @@ struct GroupedArgs {
 };
 
 // A tile of one slot as a call of its own (not inlined), so that each length's
-// body gets its own register allocation.
-template <int NB, bool BF, bool TWO>
-__device__ __noinline__ bool grouped_tile(const GroupSlot& g, int tile, uint8_t* smem, uint32_t tmem)
+// body gets its own register allocation.  smem_raw: the CTA's dynamic shared
+// memory; each body aligns it as it needs (the lane step, which uses almost all
+// of it, to 128 bytes only).
+__device__ __forceinline__ uint8_t* align_up(uint8_t* p, uintptr_t to)
 {
-    return fused_tile<NB, BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, smem, tmem);
+    return (uint8_t*)(((uintptr_t)p + to - 1) & ~(to - 1));
+}
+template <int NB, bool BF, bool TWO>
+__device__ __noinline__ bool grouped_tile(const GroupSlot& g, int tile, uint8_t* smem_raw, uint32_t tmem)
+{
+    if constexpr (BF && !TWO) return lanes::lane_tile<NB>(g.a, g.la, tile, align_up(smem_raw, 128), tmem);
+    else return fused_tile<NB, BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, align_up(smem_raw, 1024), tmem);
 }
 template <bool BF, bool TWO>
-__device__ __noinline__ bool grouped_pair(const GroupSlot& g, int tile, uint8_t* smem, uint32_t tmem)
+__device__ __noinline__ bool grouped_pair(const GroupSlot& g, int tile, uint8_t* smem_raw, uint32_t tmem)
 {
-    return pair_tile<BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, smem, tmem);
+    return pair_tile<BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, align_up(smem_raw, 1024), tmem);
 }
 
 template <bool BF, bool TWO>
@@ -1597,20 +1624,19 @@ k_fused_grouped(const __grid_constant__ GroupedArgs P)
     }
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t s_tmem;
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     tmem_alloc<512>(&s_tmem);
     const uint32_t tmem = s_tmem;
     const int k = (int)(blockIdx.x >> 1);
     const int np = P.g[0].tiles;
     bool ok = true;
     if (k < np) {
-        ok = grouped_pair<BF, TWO>(P.g[0], k, smem, tmem);
+        ok = grouped_pair<BF, TWO>(P.g[0], k, smem_raw, tmem);
     } else {
         const int item = 2 * (k - np) + (int)cluster_rank();
         const int n1 = P.g[1].tiles, n2 = n1 + P.g[2].tiles, n3 = n2 + P.g[3].tiles;
-        if (item < n1) ok = grouped_tile<256, BF, TWO>(P.g[1], item, smem, tmem);
-        else if (item < n2) ok = grouped_tile<128, BF, TWO>(P.g[2], item - n1, smem, tmem);
-        else if (item < n3) ok = grouped_tile<64, BF, TWO>(P.g[3], item - n2, smem, tmem);
+        if (item < n1) ok = grouped_tile<256, BF, TWO>(P.g[1], item, smem_raw, tmem);
+        else if (item < n2) ok = grouped_tile<128, BF, TWO>(P.g[2], item - n1, smem_raw, tmem);
+        else if (item < n3) ok = grouped_tile<64, BF, TWO>(P.g[3], item - n2, smem_raw, tmem);
     }
     fence_before();
     __syncthreads();
@@ -1628,17 +1654,24 @@ struct FusedPlan {
     float* w32 = nullptr;       // w_p with w_0 (FP32), for the mode-keyed epilogue
     float* zbuf = nullptr;      // mode-keyed noise of two steps [2][C][3][M]
     bool mz = false;            // mode-keyed noise on
+    uint8_t* lane_tab = nullptr;   // lane step (BF16, three passes, 64 .. 256 beads): table blocks
+    float4* lane_c = nullptr;      // ... and per-mode constants
     CUtensorMap tmR, tmChiH, tmChiL, tmFH, tmFL;
 };
 
-// Chains per tile: a multiple of 4 (one share per TMEM lane quarter), 4..kChains.
-static int round_tile(int cpt) { return std::min(kChains, std::max(4, (cpt + 3) / 4 * 4)); }
+// Chains per tile: a multiple of 4 (one share per TMEM lane quarter), 4..most.
+static int round_tile(int cpt, int most) { return std::min(most, std::max(4, (cpt + 3) / 4 * 4)); }
+// Most chains per tile of a plan's step.
+static int most_chains(const FusedPlan* p) { return p->lane_tab ? lanes::kMaxChains : kChains; }
 
 bool fused_supported(int M) { return M == 64 || M == 128 || M == 256 || M == 512; }
 
 // Dynamic shared memory of the grouped kernel: that of its largest tile.
-static int grouped_smem(bool bf16)
+static int grouped_smem(bool bf16, bool two)
 {
+    if (bf16 && !two)
+        return std::max({FSmem<256, true, false>::kBytes, lanes::Geo<256>::kBytes, lanes::Geo<128>::kBytes,
+                         lanes::Geo<64>::kBytes});
     return bf16 ? std::max({FSmem<256, true, true>::kBytes, FSmem<128, true, true>::kBytes, FSmem<64, true, true>::kBytes,
                             FSmem<256, true, false>::kBytes})
                 : std::max({FSmem<256, false, false>::kBytes, FSmem<128, false, false>::kBytes,
@@ -1651,6 +1684,63 @@ static cudaError_t set_smem()
     return cudaFuncSetAttribute(k_fused_step<NB, BF, TWO, MZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 FSmem<NB, BF, kRS<NB, BF, MZ>>::kBytes);
 }
+template <int M>
+static cudaError_t set_smem_lane()
+{
+    return cudaFuncSetAttribute(k_lane_step<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, lanes::Geo<M>::kBytes);
+}
+
+// Table blocks of the lane step (lanes::kBlkBytes each, in the order a step takes
+// them) and its per-mode constants; see sfp_lanes.cuh for the layout, the mirror
+// symmetry at 256 beads and the symmetric table at 128.
+template <int M>
+static int lane_tables(FusedPlan* p, const double* chi, const double* phi, const double* h, const double* w,
+                       const double* dm, const double* g, cudaStream_t stream)
+{
+    using G = lanes::Geo<M>;
+    const double pi = 3.14159265358979323846;
+    std::vector<float4> lc(M);
+    std::vector<double> es(M, 1.0);
+    for (int q = 0; q < M; ++q) {
+        double cs = 1.0;
+        if (G::kScaled) {
+            // chi_{n,p} = c_p sin(pi n p / M): R is scaled by c_p, the increment by h_p c_p
+            cs = -2.0 * std::sqrt(2.0 / M) * std::sin(0.5 * pi * q / M);
+            es[q] = h[q] * cs;
+        }
+        lc[q] = make_float4((float)dm[q], (float)g[q], (float)cs, (float)es[q]);
+    }
+    auto table = [&](int t, int e, int row, int k) -> double {     // t: 0 inverse, 1 noise, 2 forward
+        const int r = M == 64 ? row & 63 : row;
+        if (G::kScaled && t != 1) return std::sin(pi * (double)((r * k) % (2 * M)) / M);
+        const int mode = G::NP * (t == 0 ? k : r) + e, n = t == 0 ? r : k;
+        if (t == 1) return w[mode] * phi[(size_t)n * M + mode];
+        double c = chi[(size_t)n * M + mode];
+        if (G::kFold && n == 0) c = e ? chi[(size_t)(M / 2) * M + mode] * (t == 2 ? 0.5 : 1.0) : 0.0;
+        return t == 2 ? h[mode] * c : c;
+    };
+    std::vector<uint16_t> img((size_t)G::BLK_TAB * lanes::kBlkBytes / 2);
+    for (int b = 0; b < G::BLK_TAB; ++b) {
+        const int t = b / G::BLK, kc = (b % G::BLK) / G::NP, e = (b % G::BLK) % G::NP;
+        uint16_t* d = img.data() + (size_t)b * lanes::kBlkBytes / 2;
+        for (int k = 0; k < 32; ++k)
+            for (int row = 0; row < 128; ++row) {
+                const double x = table(t, e, row, 32 * kc + k);
+                const size_t o = (size_t)(k >> 4) * 2048 + ((k >> 3) & 1) * 1024 + (row >> 3) * 64 + (row & 7) * 8 + (k & 7);
+                d[o] = bf16_round_host((float)x);
+                d[4096 + o] = bf16_round_host((float)(x - (double)bf16_to_float_host(d[o])));
+            }
+    }
+    if (cudaMalloc((void**)&p->lane_tab, img.size() * 2) != cudaSuccess ||
+        cudaMalloc((void**)&p->lane_c, lc.size() * sizeof(float4)) != cudaSuccess)
+        return report(SFP_ENOMEM, "lane-step table allocation failed");
+    if (cudaMemcpyAsync(p->lane_tab, img.data(), img.size() * 2, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+        cudaMemcpyAsync(p->lane_c, lc.data(), lc.size() * sizeof(float4), cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+        cudaStreamSynchronize(stream) != cudaSuccess || set_smem_lane<M>() != cudaSuccess)
+        return report(SFP_ECUDA, "lane-step set-up failed");
+    return SFP_OK;
+}
+
 template <bool BF, bool TWO = false>
 static cudaError_t set_smem_pair()
 {
@@ -1659,7 +1749,7 @@ static cudaError_t set_smem_pair()
 }
 
 int fused_create(FusedPlan** out, int M, int C, const double* chi, const double* phi, const double* h,
-                 const double* w, float* R, cudaStream_t stream, bool bf16, bool two)
+                 const double* w, const double* dm, const double* g, float* R, cudaStream_t stream, bool bf16, bool two)
 {
     *out = nullptr;
     if (!fused_supported(M)) return report(SFP_ENOTSUP, "the fused step needs M in {64, 128, 256, 512}");
@@ -1673,12 +1763,22 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
     // SMs), then the chains spread evenly over the tiles of those waves: chains
     // per tile = ceil(C / (units x waves)) rounded up to a multiple of 4
     // (fused_set_tile changes it)
+    if (bf16 && !two && M <= 256) {
+        const int rc = M == 256 ? lane_tables<256>(p, chi, phi, h, w, dm, g, stream)
+                     : M == 128 ? lane_tables<128>(p, chi, phi, h, w, dm, g, stream)
+                                : lane_tables<64>(p, chi, phi, h, w, dm, g, stream);
+        if (rc) {
+            fused_destroy(p);
+            return rc;
+        }
+    }
+    const int most = most_chains(p);
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 148;
     const int units = M == 512 ? sms / 2 : sms;
-    const int waves = std::max(1, (C + units * kChains - 1) / (units * kChains));
-    p->cpt = round_tile((C + units * waves - 1) / (units * waves));
+    const int waves = std::max(1, (C + units * most - 1) / (units * most));
+    p->cpt = round_tile((C + units * waves - 1) / (units * waves), most);
     const size_t mm = (size_t)M * M;
     // chi [n][p] (row n = 0 and column p = 0 are zero) and F [2M][M]:
     // F[p][n] = h_p chi[n][p] (Eq. f2 weight on DeltaH = chi^T v, Eq. e11),
@@ -1745,8 +1845,7 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
         e = M == 512 ? set_smem_pair<true, true>() : M == 256 ? set_smem<256, true, true>() :
             M == 128 ? set_smem<128, true, true>() : set_smem<64, true, true>();
     else if (bf16)
-        e = M == 512 ? set_smem_pair<true>() : M == 256 ? set_smem<256, true>() :
-            M == 128 ? set_smem<128, true>() : set_smem<64, true>();
+        e = M == 512 ? set_smem_pair<true>() : cudaSuccess;   // the lane step's own set-up: lane_tables
     else
         e = M == 512 ? set_smem_pair<false>() : M == 256 ? set_smem<256, false>() :
             M == 128 ? set_smem<128, false>() : set_smem<64, false>();
@@ -1766,7 +1865,7 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(p->two ? k_fused_grouped<true, true> : bf16 ? k_fused_grouped<true, false>
                                                                              : k_fused_grouped<false, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, grouped_smem(bf16));
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, grouped_smem(bf16, p->two));
     if (e != cudaSuccess) {
         fused_destroy(p);
         return report(SFP_ECUDA, "cudaFuncSetAttribute (fused step) failed");
@@ -1784,6 +1883,14 @@ int fused_step(FusedPlan* p, const FusedArgs& args, cudaStream_t stream)
     a.zbuf = p->zbuf;
     a.w = p->w32;
     if (p->mz && (p->two || p->M > 256)) return report(SFP_ENOTSUP, "mode-keyed noise: M <= 256, three passes");
+    if (p->lane_tab && !p->mz) {
+        const lanes::LaneArgs la{p->lane_tab, p->lane_c};
+        if (p->M == 256) k_lane_step<256><<<grid, lanes::kThreads, lanes::Geo<256>::kBytes, stream>>>(a, la);
+        else if (p->M == 128) k_lane_step<128><<<grid, lanes::kThreads, lanes::Geo<128>::kBytes, stream>>>(a, la);
+        else k_lane_step<64><<<grid, lanes::kThreads, lanes::Geo<64>::kBytes, stream>>>(a, la);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? SFP_OK : report(SFP_ECUDA, cudaGetErrorString(e));
+    }
 #define SFP_FUSED_LAUNCH(NBV, BFV)                                                                   \
     if (p->mz)                                                                                       \
         k_fused_step<NBV, BFV, false, true><<<grid, kThreads, FSmem<NBV, BFV, kRS<NBV, BFV, true>>::kBytes, stream>>>( \
@@ -1791,8 +1898,8 @@ int fused_step(FusedPlan* p, const FusedArgs& args, cudaStream_t stream)
     else if (p->two)                                                                                 \
         k_fused_step<NBV, BFV, BFV><<<grid, kThreads, FSmem<NBV, BFV, kRS<NBV, BFV>>::kBytes, stream>>>(         \
             p->tmR, p->tmChiH, p->tmChiL, p->tmFH, p->tmFL, a);                                      \
-    else                                                                                             \
-        k_fused_step<NBV, BFV><<<grid, kThreads, FSmem<NBV, BFV, kRS<NBV, BFV>>::kBytes, stream>>>(              \
+    else if constexpr (!BFV)                                                                         \
+        k_fused_step<NBV, false><<<grid, kThreads, FSmem<NBV, false, false>::kBytes, stream>>>(                  \
             p->tmR, p->tmChiH, p->tmChiL, p->tmFH, p->tmFL, a)
     cudaError_t e = cudaSuccess;
     switch (p->M * 2 + (p->bf16 ? 1 : 0)) {
@@ -1849,6 +1956,7 @@ int fused_step_grouped(FusedPlan* const* plans, const FusedArgs* args, int n, cu
             return report(SFP_EINVAL, "grouped step: one plan each of 64, 128, 256, 512 beads, one arithmetic");
         GroupSlot& g = P.g[slot];
         g.tmR = p->tmR; g.tmChiH = p->tmChiH; g.tmChiL = p->tmChiL; g.tmFH = p->tmFH; g.tmFL = p->tmFL;
+        g.la = lanes::LaneArgs{p->lane_tab, p->lane_c};
         g.a = args[i];
         if (args[i].C < 1 || args[i].C > p->C) return report(SFP_EINVAL, "grouped step: chain count outside the plan");
         g.tiles = (args[i].C + p->cpt - 1) / p->cpt;
@@ -1858,7 +1966,7 @@ int fused_step_grouped(FusedPlan* const* plans, const FusedArgs* args, int n, cu
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2u * (unsigned)(P.g[0].tiles + (small + 1) / 2));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = grouped_smem(bf);
+    cfg.dynamicSmemBytes = grouped_smem(bf, two);
     cfg.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1882,13 +1990,16 @@ size_t fused_bytes(const FusedPlan* p)
 {
     if (!p) return 0;
     return (size_t)6 * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float) +
-           (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0);
+           (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0) +
+           (p->lane_tab ? (size_t)(p->M == 256 ? lanes::Geo<256>::BLK_TAB : p->M == 128 ? lanes::Geo<128>::BLK_TAB
+                                                                                     : lanes::Geo<64>::BLK_TAB) *
+                                  lanes::kBlkBytes + (size_t)p->M * sizeof(float4) : 0);
 }
 
 int fused_set_tile(FusedPlan* p, int cpt)
 {
     if (cpt < 1 || cpt > kChains) return report(SFP_EINVAL, "chains per tile must be 1..40");
-    cpt = round_tile(cpt);
+    cpt = round_tile(cpt, most_chains(p));
     CUtensorMap m;
     const int rc = make_map_2d(&m, p->R, 3 * p->C, p->M, 3 * (cpt / 4));
     if (rc) return rc;
@@ -1917,6 +2028,8 @@ void fused_destroy(FusedPlan* p)
     for (void* t : p->tab)
         if (t) cudaFree(t);
     if (p->w32) cudaFree(p->w32);
+    if (p->lane_tab) cudaFree(p->lane_tab);
+    if (p->lane_c) cudaFree(p->lane_c);
     if (p->zbuf) cudaFree(p->zbuf);
     delete p;
 }
