@@ -36,7 +36,7 @@
 // and writes its own modes, 256 contiguous bytes per warp.
 //
 // Measured (GB300, 400-step calls, 4096 x 256 bp, 28 chains per tile): 22.8 us a
-// step with the chains' axes on the TMEM lanes (fused_tile), 16.6 us here; 50 x
+// step with the chains' axes on the TMEM lanes (fused_tile), 12.9 us here; 50 x
 // 128 bp, 8 steps with the call around them: 146 -> 97 us; 4096 x 64 bp, 400 steps
 // and 21 samples: 4.75 -> 3.71 ms.
 #pragma once
@@ -86,6 +86,14 @@ struct Geo {
     static constexpr uint32_t kCols = M == 64 ? 256 : 512;
     static_assert(kBytes <= 227 * 1024, "shared memory of one CTA");
 };
+
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 
 // Shared-memory matrix descriptor without swizzle (core matrices of 8 x 16 bytes).
 __device__ __forceinline__ uint64_t ndesc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
@@ -167,7 +175,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
     uint64_t* never = bars + 23;        // nothing arrives here (the stall test)
     volatile int* abort_flag = (volatile int*)(bars + 24);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp: uniform
     const int c0 = tile * a.cpt;
     const int Ct = min(a.cpt, a.C - c0);
 
@@ -217,7 +225,8 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 int src = 0;
                 for (int it = 0; it < total; ++it) {
                     const int s = it % G::ST;
-                    if (!mbar_wait(&empty[s], ((it / G::ST) & 1) ^ 1, a.err, abort_flag)) { ok = false; break; }
+                    ok = mbar_wait(&empty[s], ((it / G::ST) & 1) ^ 1, a.err, abort_flag);
+                    if (!ok) break;
                     mbar_expect_tx(&full[s], kBlkBytes);
                     bulk_load(tabs + s * kBlkBytes, la.tab + (size_t)src * kBlkBytes, kBlkBytes, &full[s]);
                     if (++src == G::BLK_STEP) src = 0;
@@ -235,70 +244,81 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t id_z = idesc_bf16(128, kRowsN);              // B K-major
-            constexpr uint32_t id_x = id_z | (1u << 16);                    // B rows-major
-            bool ok = true;
-            if (a.stall_test) ok = mbar_wait(never, 0, a.err, abort_flag);
-            if constexpr (!G::kStream) ok = ok && mbar_wait(tab_full, 0, a.err, abort_flag);
-            const uint32_t tab0 = smem_u32(tabs), x0 = smem_u32(X), z0 = smem_u32(Z);
-            int it = 0;                                     // streamed blocks taken
-            // the six MMAs of each of the block's two K steps: table hi/lo x operand hi/lo
-            auto block = [&](int resident, uint32_t d, uint64_t b_hi, uint64_t b_lo, uint32_t bstep, uint32_t idesc,
-                             bool first) {
-                const int s = G::kStream ? it % G::ST : resident;
-                if constexpr (G::kStream) ok = ok && mbar_wait(&full[s], (it / G::ST) & 1, a.err, abort_flag);
-                if (ok) {
-                    fence_after();
-                    const uint64_t ad = ndesc(tab0 + s * kBlkBytes, kALbo, kASbo);
+        // ---------------- MMA issuer.  The whole warp runs the loops and the waits,
+        // one elected lane issues: with everything but the issue itself uniform over
+        // the warp, descriptors live in uniform registers and an MMA costs a few
+        // instructions (a single-lane loop took 740 cycles for the six MMAs of a
+        // block, beside 16 busy warps; their run time is 288).
+        constexpr uint32_t id_z = idesc_bf16(128, kRowsN);              // B K-major
+        constexpr uint32_t id_x = id_z | (1u << 16);                    // B rows-major
+        const bool leader = elect_one();
+        bool ok = true;
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            ok = __all_sync(0xffffffffu, ok && mbar_wait(bar, parity, a.err, abort_flag));
+            fence_after();
+        };
+        if (a.stall_test) wait(never, 0);
+        if constexpr (!G::kStream) wait(tab_full, 0);
+        const uint64_t tab0 = ndesc(smem_u32(tabs), kALbo, kASbo);
+        const uint64_t x0 = ndesc(smem_u32(X), 128, kXSbo), z0 = ndesc(smem_u32(Z), kZLbo, 128);
+        int slot = 0;                                   // ring slot and phase of the next streamed block
+        uint32_t phase = 0;
+        // the six MMAs of a block's two K steps, table hi/lo x operand hi/lo; b: the
+        // operand's hi part (the lo part b_lo further), bstep: its next K step
+        auto block = [&](int resident, uint32_t d, uint64_t b, uint32_t b_lo, uint32_t bstep, uint32_t idesc, bool first) {
+            const int s = G::kStream ? slot : resident;
+            if constexpr (G::kStream) wait(&full[s], phase);
+            if (leader && ok) {
+                const uint64_t ad = tab0 + (uint64_t)(s * (kBlkBytes / 16));
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {
-                        const uint64_t ah = ad + (uint64_t)(kk * 4096 / 16), al = ah + (uint64_t)(8192 / 16);
-                        const uint64_t bh = b_hi + (uint64_t)(kk * (bstep / 16)), bl = b_lo + (uint64_t)(kk * (bstep / 16));
-                        mma_bf16(d, al, bh, idesc, (first && kk == 0) ? 0u : 1u);
-                        mma_bf16(d, ah, bl, idesc, 1u);
-                        mma_bf16(d, ah, bh, idesc, 1u);
-                    }
-                    if constexpr (G::kStream) mma_commit(&empty[s]);
+                for (int kk = 0; kk < 2; ++kk) {
+                    const uint64_t ah = ad + kk * (4096 / 16), al = ah + 8192 / 16;
+                    const uint64_t bh = b + kk * (bstep / 16), bl = bh + b_lo / 16;
+                    mma_bf16(d, al, bh, idesc, (first && kk == 0) ? 0u : 1u);
+                    mma_bf16(d, ah, bl, idesc, 1u);
+                    mma_bf16(d, ah, bh, idesc, 1u);
                 }
-                ++it;
-            };
-            // a contraction of operand X (modes or bond forces) into D
-            auto with_x = [&](int res0, uint32_t d0, bool first) {
-#pragma unroll 1
-                for (int b = 0; b < G::BLK; ++b) {
-                    const int e = b % NP, kc = b / NP;
-                    const uint64_t xh = ndesc(x0 + e * 2 * kXPart + kc * 4 * 128, 128, kXSbo);
-                    block(res0 + b, d0 + e * kRowsN, xh, xh + kXPart / 16, 256, id_x, first && kc == 0);
-                }
-            };
-            const uint32_t d_u = tmem, d_inc = tmem + NP * kRowsN, d_z = G::kScaled ? d_inc + kRowsN : d_inc;
-            int chunk = 0;
-#pragma unroll 1
-            for (int sp = 0; sp < a.n_steps; ++sp) {
-                ok = ok && mbar_wait(r_ready, sp & 1, a.err, abort_flag);
-                if (ok) fence_after();
-                with_x(0, d_u, true);
-                if (ok) mma_commit(u_done);
-#pragma unroll 1
-                for (int ch = 0; ch < G::NCH; ++ch, ++chunk) {
-                    ok = ok && mbar_wait(n_ready, chunk & 1, a.err, abort_flag);
-                    if (ok) fence_after();
-#pragma unroll 1
-                    for (int b = 0; b < G::BLK / G::NCH; ++b) {
-                        const int e = b % NP, kc = b / NP;          // K block of the chunk
-                        const uint64_t zh = ndesc(z0 + e * 2 * kZPart + kc * 4 * kZLbo, kZLbo, 128);
-                        block(G::BLK + ch * (G::BLK / G::NCH) + b, d_z + e * kRowsN, zh, zh + kZPart / 16, 2 * kZLbo,
-                              id_z, ch == 0 && kc == 0);
-                    }
-                    if (ok) mma_commit(n_free);
-                }
-                ok = ok && mbar_wait(v_ready, sp & 1, a.err, abort_flag);
-                if (ok) fence_after();
-                with_x(G::kScaled ? 0 : 2 * G::BLK, d_inc, G::kScaled);
-                if (ok) mma_commit(inc_done);
+                if constexpr (G::kStream) mma_commit(&empty[s]);
             }
+            if constexpr (G::kStream) {
+                if (++slot == G::ST) {
+                    slot = 0;
+                    phase ^= 1u;
+                }
+            }
+        };
+        // a contraction of operand X (modes or bond forces) into d
+        auto with_x = [&](int res0, uint32_t d, bool first) {
+#pragma unroll 1
+            for (int kc = 0; kc < G::BLK / NP; ++kc)
+#pragma unroll
+                for (int e = 0; e < NP; ++e)
+                    block(res0 + kc * NP + e, d + e * kRowsN, x0 + (uint64_t)((e * 2 * kXPart + kc * 4 * 128) / 16), kXPart,
+                          256, id_x, first && kc == 0);
+        };
+        const uint32_t d_u = tmem, d_inc = tmem + NP * kRowsN, d_z = G::kScaled ? d_inc + kRowsN : d_inc;
+        int chunk = 0;
+#pragma unroll 1
+        for (int sp = 0; sp < a.n_steps && ok; ++sp) {
+            wait(r_ready, sp & 1);
+            with_x(0, d_u, true);
+            if (leader && ok) mma_commit(u_done);
+#pragma unroll 1
+            for (int ch = 0; ch < G::NCH; ++ch, ++chunk) {
+                wait(n_ready, chunk & 1);
+                constexpr int KC = G::BLK / G::NCH / NP;            // K blocks of a chunk
+#pragma unroll 1
+                for (int kc = 0; kc < KC; ++kc)
+#pragma unroll
+                    for (int e = 0; e < NP; ++e)
+                        block(G::BLK + (ch * KC + kc) * NP + e, d_z + e * kRowsN,
+                              z0 + (uint64_t)((e * 2 * kZPart + kc * 4 * kZLbo) / 16), kZPart, 2 * kZLbo, id_z,
+                              ch == 0 && kc == 0);
+                if (leader && ok) mma_commit(n_free);
+            }
+            wait(v_ready, sp & 1);
+            with_x(G::kScaled ? 0 : 2 * G::BLK, d_inc, G::kScaled);
+            if (leader && ok) mma_commit(inc_done);
         }
     } else if (warp < 2 + kWarps) {
         // ---------------- the working warps
