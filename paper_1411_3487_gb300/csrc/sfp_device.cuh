@@ -149,7 +149,8 @@ template <> struct Normals<float> {
         float ra, rb, sa, ca, sb, cb;
         box_radius2(w.x, w.z, ra, rb);
         box_angle2(w.y, w.w, sa, ca, sb, cb);
-        g[0] = ra * ca; g[1] = ra * sa; g[2] = rb * cb; g[3] = rb * sb;
+        // rounded here: a product contracted into a caller's sum would differ between kernels
+        g[0] = __fmul_rn(ra, ca); g[1] = __fmul_rn(ra, sa); g[2] = __fmul_rn(rb, cb); g[3] = __fmul_rn(rb, sb);
     }
 };
 template <> struct Normals<double> {

@@ -1721,14 +1721,14 @@ static int lane_tables(FusedPlan* p, const double* chi, const double* phi, const
     };
     std::vector<uint16_t> img((size_t)G::BLK_TAB * lanes::kBlkBytes / 2);
     for (int b = 0; b < G::BLK_TAB; ++b) {
-        const int t = b / G::BLK, kc = (b % G::BLK) / G::NP, e = (b % G::BLK) % G::NP;
+        const int t = b / G::BLK, k0 = 16 * ((b % G::BLK) / G::NP), e = (b % G::BLK) % G::NP;
         uint16_t* d = img.data() + (size_t)b * lanes::kBlkBytes / 2;
-        for (int k = 0; k < 32; ++k)
+        for (int k = 0; k < 16; ++k)
             for (int row = 0; row < 128; ++row) {
-                const double x = table(t, e, row, 32 * kc + k);
-                const size_t o = (size_t)(k >> 4) * 2048 + ((k >> 3) & 1) * 1024 + (row >> 3) * 64 + (row & 7) * 8 + (k & 7);
+                const double x = table(t, e, row, k0 + k);
+                const size_t o = (size_t)(k >> 3) * 1024 + (row >> 3) * 64 + (row & 7) * 8 + (k & 7);
                 d[o] = bf16_round_host((float)x);
-                d[4096 + o] = bf16_round_host((float)(x - (double)bf16_to_float_host(d[o])));
+                d[lanes::kBlkBytes / 4 + o] = bf16_round_host((float)(x - (double)bf16_to_float_host(d[o])));
             }
     }
     if (cudaMalloc((void**)&p->lane_tab, img.size() * 2) != cudaSuccess ||

@@ -23,22 +23,25 @@
 // themselves; at 64 beads lanes 64..127 repeat lanes 0..63, so that all four
 // TMEM lane quarters can work on the tile's chains.
 //
-// Roles (18 warps of work): warp 0 streams the tables (256 beads: 24 blocks of
-// 16 KB a step through a ring; 64 and 128 beads: resident, loaded once), warp 1
-// issues the MMAs, warps 2..17 do everything else: per step
-//   force:     bond vectors from D_u -> v -> operand X, then normals of the next
-//              step while the forward MMAs run
-//   epilogue:  R += -dm R + D_inc (+ shear) -> global and operand X, then more
-//              normals while the inverse MMAs run
-// All 16 warps run the same code at about the same time, and the normals, the
-// most arithmetic of a step and independent of the state, fill every wait for
-// the tensor pipe.  The state R stays in global memory (L2): each thread reads
-// and writes its own modes, 256 contiguous bytes per warp.
+// Roles (20 warps): warp 0 streams the tables (256 beads: 48 blocks of 8 KB a step
+// through a ring; 64 and 128 beads: resident, loaded once); warp 1 issues the MMAs
+// (256 beads: of the even modes, warp 18 of the odd ones, whose accumulators are
+// others); warps 2..9 (two per TMEM lane quarter) form the force, D_u -> v -> operand
+// X, and update the modes, R += -dm R + D_inc (+ shear) -> operand X; warps 10..17
+// draw the normals, the most arithmetic of a step and independent of the state, into
+// the two buffers of the noise operand; warp 19 keeps the FP64 centre of mass.  The
+// chain of a step, inverse MMAs - force - forward MMAs - update, then leaves most
+// issue slots to the normals.  The state stays in TMEM for the launch; at 256 beads
+// three of eight batches of chains find no room there and live in global memory (L2),
+// read and written by the thread that owns the modes.
 //
-// Measured (GB300, 400-step calls, 4096 x 256 bp, 28 chains per tile): 22.8 us a
-// step with the chains' axes on the TMEM lanes (fused_tile), 12.9 us here; 50 x
-// 128 bp, 8 steps with the call around them: 146 -> 97 us; 4096 x 64 bp, 400 steps
-// and 21 samples: 4.75 -> 3.71 ms.
+// What bounds it (256 beads, 28 chains): about 38 K warp instructions a step at two
+// per cycle, 168 warps' worth of Philox calls more than half of them; a chain of 5.3
+// us a step with one chain per tile (inverse and forward MMAs 3000 cycles each, force,
+// update and four hand-overs).  State and D live in 504 of the 512 TMEM columns.
+// Measured (GB300, us a step in a 400-step call, the four-role kernel of sfp_fused.cu
+// before -> here): 4096 x 256 bp 22.7 -> 9.1, 8 x 256 bp 19.1 -> 5.3, 4096 x 128 bp
+// 10.3 -> 4.3, 50 x 128 bp 9.5 -> 2.7, 4096 x 64 bp 7.3 -> 2.3, 8 x 64 bp 5.9 -> 1.5.
 #pragma once
 #include <cstdint>
 #include <cuda_bf16.h>
@@ -54,36 +57,43 @@ using namespace ptx;
 
 constexpr int kRowsN = 96;                      // MMA N: 32 chain slots x 3 axes
 constexpr int kMaxChains = 32;
-constexpr int kWarps = 16;                      // working warps (2 .. 17)
-constexpr int kThreads = 32 * (2 + kWarps);
-constexpr int kBlkBytes = 16384;                // a table block: [hi, lo][2 K steps][2 k groups][16 row groups][8][8]
+constexpr int kWork = 8, kNoise = 8;            // force / update warps (2 .. 9), noise warps (10 .. 17)
+constexpr int kThreads = 32 * (4 + kWork + kNoise);
+constexpr int kBlkBytes = 8192;                 // a table block (one K step of 16): [hi, lo][2 k groups][16 row groups][8][8]
 constexpr int kALbo = 2048, kASbo = 128;        // table blocks: K-major core matrices
 constexpr int kXSbo = 2048;                     // operand X: rows-major (MN-major) core matrices, [12 row groups][16 k groups]
 constexpr int kXPart = 12 * kXSbo;              // one parity and part (hi or lo): 24 KB
-constexpr int kZLbo = 12 * 128 + 16;            // noise operand: K-major core matrices, k groups 16 bytes apart in the banks
-constexpr int kZPart = 8 * kZLbo;               // K = 64
+constexpr int kZLbo = 12 * 128 + 32;            // noise operand: K-major core matrices, k groups 32 bytes apart in the banks
+constexpr int kZPart = 4 * kZLbo;               // K = 32
 
+// Rows of N: four chains (batch b = chain / 4 of the tile) hold rows 24 (b / 2) +
+// 8 axis + 4 (b & 1) + chain % 4, so that a thread's four values of an axis are 8
+// contiguous bytes of operand X.
 template <int M>
 struct Geo {
     static constexpr bool kFold = M == 256;
     static constexpr int NP = kFold ? 2 : 1;            // parities
     static constexpr int KP = M / NP;                   // K of one parity's contraction
-    static constexpr int NG = M == 64 ? 8 : 4;          // chain groups (working warps of a lane)
-    static constexpr int SLOTS = kMaxChains / NG;       // chain slots of a group
     static constexpr bool kStream = M == 256;           // tables through a ring, else resident
     static constexpr bool kScaled = M == 128;           // one symmetric table sin(pi n p / M) for both directions
-    static constexpr int BLK = NP * KP / 32;            // table blocks of one contraction
+    static constexpr int NCH = KP / 32;                 // noise chunks (K = 32 per parity) of a step
+    static constexpr int BLK = NP * KP / 16;            // table blocks of one contraction
     static constexpr int BLK_STEP = 3 * BLK;            // ... of a step (streamed)
     static constexpr int BLK_TAB = kScaled ? 2 * BLK : 3 * BLK;   // ... in the table image
-    static constexpr int ST = kStream ? 5 : BLK_TAB;    // blocks in shared memory
-    static constexpr int NCH = M == 64 ? 1 : 2;         // noise chunks (K = 64 per parity) of a step
+    // blocks in shared memory: all, or a ring; a ring slot always serves the same
+    // parity, whose MMA warp so sees every phase of its barrier
+    static constexpr int ST = kStream ? 10 : BLK_TAB;
+    static_assert(!kStream || ST % NP == 0, "ring slots per parity");
     static constexpr int XB = NP * 2 * kXPart;
-    static constexpr int ZB = NP * 2 * kZPart;
+    static constexpr int ZB = NP * 2 * kZPart;          // one buffer of the noise operand
     static constexpr int kMisc = 1664;
-    static constexpr int kBytes = ST * kBlkBytes + XB + ZB + kMisc + 128;
+    static constexpr int kBytes = ST * kBlkBytes + XB + 2 * ZB + kMisc + 128;
     // TMEM columns: D_u and D_inc, 96 each per parity; with the symmetric table, whose
-    // increment h_p c_p scales after the contraction, the noise in a third accumulator
-    static constexpr uint32_t kCols = M == 64 ? 256 : 512;
+    // increment h_p c_p scales after the contraction, the noise in a third accumulator;
+    // then the state R of the first TB batches
+    static constexpr uint32_t kCols = 512;
+    static constexpr int kRCol = (2 * NP + (kScaled ? 1 : 0)) * kRowsN;
+    static constexpr int TB = (512 - kRCol) / (12 * NP) < 8 ? (512 - kRCol) / (12 * NP) : 8;
     static_assert(kBytes <= 227 * 1024, "shared memory of one CTA");
 };
 
@@ -123,23 +133,40 @@ __device__ __forceinline__ void tmem_wait12(float (&a)[3][4])
                  :: "memory");
 }
 
-// Four values as BF16 hi and lo parts (round to nearest even), value i in halfword i.
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const float (&v)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};"
+                 ::"r"(taddr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Two values as BF16 hi and lo parts (round to nearest even), value i in halfword i.
+__device__ __forceinline__ void split2(f32x2 x, uint32_t& hi, uint32_t& lo)
+{
+    float a, b;
+    unpack2(x, a, b);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
+    unpack2(sub2(x, pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xFFFF0000u))), a, b);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b), "f"(a));
+}
 __device__ __forceinline__ void split4(const float (&x)[4], uint2& hi, uint2& lo)
 {
-    uint32_t h[2], l[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h[i]) : "f"(x[2 * i + 1]), "f"(x[2 * i]));
-        const float a = x[2 * i] - __uint_as_float(h[i] << 16);
-        const float b = x[2 * i + 1] - __uint_as_float(h[i] & 0xFFFF0000u);
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l[i]) : "f"(b), "f"(a));
-    }
-    hi = make_uint2(h[0], h[1]);
-    lo = make_uint2(l[0], l[1]);
+    split2(pack2(x[0], x[1]), hi.x, lo.x);
+    split2(pack2(x[2], x[3]), hi.y, lo.y);
+}
+
+// 1/|u| of two bonds; |u|^2 of a bond that exists is far from the denormals.
+__device__ __forceinline__ f32x2 rsqrt2(f32x2 t)
+{
+    float a, b;
+    unpack2(t, a, b);
+    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(a));
+    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(b));
+    return pack2(a, b);
 }
 
 struct LaneArgs {
-    const uint8_t* tab;     // table blocks in the order a step takes them (chi, w phi, h chi); 128 beads: sin, w phi
+    const uint8_t* tab;     // table blocks chi, w phi, h chi (128 beads: sin, w phi), K blocks in order, even modes first
     const float4* lane_c;   // per mode p: 1 - e^{-zeta dtau}, shear weight, operand scale, increment scale
 };
 
@@ -155,25 +182,25 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
     uint8_t* tabs = smem;
     uint8_t* X = smem + G::ST * kBlkBytes;
     uint8_t* Z = X + G::XB;
-    uint8_t* misc = Z + G::ZB;
+    uint8_t* misc = Z + 2 * G::ZB;
     int64_t* s_step = (int64_t*)misc;               // [32]
     double* s_shear = (double*)(misc + 256);        // [32]
     uint32_t* s_job = (uint32_t*)(misc + 512);      // [32]
     int* s_left = (int*)(misc + 640);               // [32] steps this chain still takes in this launch
-    float* s_d0 = (float*)(misc + 768);             // [32][3] noise increments of the centre of mass
+    float* s_d0 = (float*)(misc + 768);             // [3][32] noise increments of the centre of mass
     uint64_t* bars = (uint64_t*)(misc + 1152);
     float* s_shf = (float*)(misc + 1408);           // [32]
-    uint64_t* full = bars;              // table block landed (1 + tx)
-    uint64_t* empty = bars + 8;         // MMAs done with the block (commit)
-    uint64_t* tab_full = bars + 16;     // resident tables landed
-    uint64_t* r_ready = bars + 17;      // operand X holds the modes (every working warp)
-    uint64_t* v_ready = bars + 18;      // operand X holds the bond forces
-    uint64_t* n_ready = bars + 19;      // noise operand written
-    uint64_t* n_free = bars + 20;       // MMAs done with the noise operand (commit)
-    uint64_t* u_done = bars + 21;       // inverse MMAs done (commit)
-    uint64_t* inc_done = bars + 22;     // forward MMAs done (commit)
-    uint64_t* never = bars + 23;        // nothing arrives here (the stall test)
-    volatile int* abort_flag = (volatile int*)(bars + 24);
+    uint64_t* full = bars;              // ring slot: table block landed (1 + tx)
+    uint64_t* empty = bars + 10;        // ... MMAs done with it (commit)
+    uint64_t* tab_full = bars + 20;     // resident tables landed
+    uint64_t* r_ready = bars + 21;      // operand X holds the modes, D_inc has been read (every work warp)
+    uint64_t* v_ready = bars + 22;      // operand X holds the bond forces (every work warp; warp 19: s_d0 has been read)
+    uint64_t* n_ready = bars + 23;      // noise buffer b written (every noise warp)
+    uint64_t* n_free = bars + 25;       // MMAs done with noise buffer b (a commit per parity)
+    uint64_t* u_done = bars + 27;       // inverse MMAs done (a commit per parity)
+    uint64_t* inc_done = bars + 28;     // noise and forward MMAs done (a commit per parity)
+    uint64_t* never = bars + 29;        // nothing arrives here (the stall test)
+    volatile int* abort_flag = (volatile int*)(bars + 30);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp: uniform
     const int c0 = tile * a.cpt;
@@ -186,12 +213,14 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 mbar_init(&empty[s], 1);
             }
         mbar_init(tab_full, 1);
-        mbar_init(r_ready, kWarps);
-        mbar_init(v_ready, kWarps);
-        mbar_init(n_ready, kWarps);
-        mbar_init(n_free, 1);
-        mbar_init(u_done, 1);
-        mbar_init(inc_done, 1);
+        mbar_init(r_ready, kWork);
+        mbar_init(v_ready, kWork + 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&n_ready[b], kNoise);
+            mbar_init(&n_free[b], NP);
+        }
+        mbar_init(u_done, NP);
+        mbar_init(inc_done, NP);
         mbar_init(never, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -208,49 +237,62 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         s_shf[i] = (float)s_shear[i];
     }
     // rows and K indices that nothing writes stay zero
-    for (int i = threadIdx.x; i < (G::XB + G::ZB) / 16; i += blockDim.x)
+    for (int i = threadIdx.x; i < (G::XB + 2 * G::ZB) / 16; i += blockDim.x)
         reinterpret_cast<uint4*>(X)[i] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async();
     fence_before();
     __syncthreads();
     fence_after();
     const bool has_shear = __syncthreads_or(threadIdx.x < Ct && s_shear[threadIdx.x] != 0.0) != 0;
+    // no chain of the tile is sheared or reaches its stop step in this launch
+    const bool steady = __syncthreads_and(!has_shear && (threadIdx.x >= Ct || s_left[threadIdx.x] == a.n_steps)) != 0;
 
     if (warp == 0) {
-        // ---------------- table blocks
-        if (lane == 0) {
+        // ---------------- table blocks (the whole warp runs the loop, one lane issues:
+        // see the MMA issuer)
+        const bool leader = elect_one();
+        if constexpr (G::kStream) {
+            const int total = a.n_steps * G::BLK_STEP;
             bool ok = true;
-            if constexpr (G::kStream) {
-                const int total = a.n_steps * G::BLK_STEP;
-                int src = 0;
-                for (int it = 0; it < total; ++it) {
-                    const int s = it % G::ST;
-                    ok = mbar_wait(&empty[s], ((it / G::ST) & 1) ^ 1, a.err, abort_flag);
-                    if (!ok) break;
+            int s = 0, src = 0;
+            uint32_t phase = 1;
+#pragma unroll 1
+            for (int it = 0; it < total; ++it) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], phase, a.err, abort_flag));
+                if (!ok) break;
+                if (leader) {
                     mbar_expect_tx(&full[s], kBlkBytes);
-                    bulk_load(tabs + s * kBlkBytes, la.tab + (size_t)src * kBlkBytes, kBlkBytes, &full[s]);
-                    if (++src == G::BLK_STEP) src = 0;
+                    bulk_load(tabs + s * kBlkBytes, la.tab + src * kBlkBytes, kBlkBytes, &full[s]);
                 }
-                // the last commit of every ring slot has landed before the tile ends
-                for (int s = 0; s < G::ST && s < total && ok; ++s) {
-                    const int last = s + G::ST * ((total - 1 - s) / G::ST);
-                    ok = mbar_wait(&empty[s], (last / G::ST) & 1, a.err, abort_flag);
+                if (++src == G::BLK_STEP) src = 0;
+                if (++s == G::ST) {
+                    s = 0;
+                    phase ^= 1u;
                 }
-            } else {
+            }
+            // the last commit of every ring slot has landed before the tile ends
+            for (int k = 0; k < G::ST && k < total && ok; ++k) {
+                const int last = k + G::ST * ((total - 1 - k) / G::ST);
+                ok = mbar_wait(&empty[k], (last / G::ST) & 1, a.err, abort_flag);
+            }
+        } else {
+            if (leader) {
                 mbar_expect_tx(tab_full, G::BLK_TAB * kBlkBytes);
                 for (int k = 0; k < G::BLK_TAB; ++k)
-                    bulk_load(tabs + k * kBlkBytes, la.tab + (size_t)k * kBlkBytes, kBlkBytes, tab_full);
-                mbar_wait(tab_full, 0, a.err, abort_flag);
+                    bulk_load(tabs + k * kBlkBytes, la.tab + k * kBlkBytes, kBlkBytes, tab_full);
             }
+            mbar_wait(tab_full, 0, a.err, abort_flag);
         }
-    } else if (warp == 1) {
+    } else if (warp == 1 || (NP == 2 && warp == 18)) {
+        const int e = warp == 1 ? 0 : NP - 1;           // this warp's parity
         // ---------------- MMA issuer.  The whole warp runs the loops and the waits,
         // one elected lane issues: with everything but the issue itself uniform over
         // the warp, descriptors live in uniform registers and an MMA costs a few
         // instructions (a single-lane loop took 740 cycles for the six MMAs of a
         // block, beside 16 busy warps; their run time is 288).
-        constexpr uint32_t id_z = idesc_bf16(128, kRowsN);              // B K-major
-        constexpr uint32_t id_x = id_z | (1u << 16);                    // B rows-major
+        // N: the rows of the batches in use (24 per two batches), a multiple of 16
+        const uint32_t id_z = idesc_bf16(128, (24 * ((Ct + 7) >> 3) + 15) & ~15);       // B K-major
+        const uint32_t id_x = id_z | (1u << 16);                                        // B rows-major
         const bool leader = elect_one();
         bool ok = true;
         auto wait = [&](uint64_t* bar, uint32_t parity) {
@@ -260,43 +302,39 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         if (a.stall_test) wait(never, 0);
         if constexpr (!G::kStream) wait(tab_full, 0);
         const uint64_t tab0 = ndesc(smem_u32(tabs), kALbo, kASbo);
-        const uint64_t x0 = ndesc(smem_u32(X), 128, kXSbo), z0 = ndesc(smem_u32(Z), kZLbo, 128);
-        int slot = 0;                                   // ring slot and phase of the next streamed block
+        const uint64_t x0 = ndesc(smem_u32(X) + e * 2 * kXPart, 128, kXSbo), z0 = ndesc(smem_u32(Z) + e * 2 * kZPart, kZLbo, 128);
+        int slot = e;                                   // ring slot and phase of this parity's next streamed block
         uint32_t phase = 0;
-        // the six MMAs of a block's two K steps, table hi/lo x operand hi/lo; b: the
-        // operand's hi part (the lo part b_lo further), bstep: its next K step
-        auto block = [&](int resident, uint32_t d, uint64_t b, uint32_t b_lo, uint32_t bstep, uint32_t idesc, bool first) {
+        // the three MMAs of a block, table hi/lo x operand hi/lo; b: the operand's hi
+        // part (the lo part b_lo further)
+        auto block = [&](int resident, uint32_t d, uint64_t b, uint32_t b_lo, uint32_t idesc, bool first) {
             const int s = G::kStream ? slot : resident;
             if constexpr (G::kStream) wait(&full[s], phase);
             if (leader && ok) {
-                const uint64_t ad = tab0 + (uint64_t)(s * (kBlkBytes / 16));
-#pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    const uint64_t ah = ad + kk * (4096 / 16), al = ah + 8192 / 16;
-                    const uint64_t bh = b + kk * (bstep / 16), bl = bh + b_lo / 16;
-                    mma_bf16(d, al, bh, idesc, (first && kk == 0) ? 0u : 1u);
-                    mma_bf16(d, ah, bl, idesc, 1u);
-                    mma_bf16(d, ah, bh, idesc, 1u);
-                }
+                const uint64_t ah = tab0 + (uint64_t)(s * (kBlkBytes / 16)), al = ah + kBlkBytes / 32, bl = b + b_lo / 16;
+                mma_bf16(d, al, b, idesc, first ? 0u : 1u);
+                mma_bf16(d, ah, bl, idesc, 1u);
+                mma_bf16(d, ah, b, idesc, 1u);
                 if constexpr (G::kStream) mma_commit(&empty[s]);
             }
             if constexpr (G::kStream) {
-                if (++slot == G::ST) {
-                    slot = 0;
+                slot += NP;                             // the other parity's block lies between
+                if (slot >= G::ST) {
+                    slot -= G::ST;
                     phase ^= 1u;
                 }
             }
         };
+        // unrolled where slots are constants; at 256 beads the loops stay small, for the
+        // instruction cache (32 KB of code in the four roles' loops: 10.3 us a step, 9.1 below that)
+        constexpr int kUnroll = G::kStream ? 1 : 8;
         // a contraction of operand X (modes or bond forces) into d
         auto with_x = [&](int res0, uint32_t d, bool first) {
-#pragma unroll 1
-            for (int kc = 0; kc < G::BLK / NP; ++kc)
-#pragma unroll
-                for (int e = 0; e < NP; ++e)
-                    block(res0 + kc * NP + e, d + e * kRowsN, x0 + (uint64_t)((e * 2 * kXPart + kc * 4 * 128) / 16), kXPart,
-                          256, id_x, first && kc == 0);
+#pragma unroll(kUnroll)
+            for (int k = 0; k < G::KP / 16; ++k)
+                block(res0 + k, d, x0 + (uint64_t)(k * (2 * 128 / 16)), kXPart, id_x, first && k == 0);
         };
-        const uint32_t d_u = tmem, d_inc = tmem + NP * kRowsN, d_z = G::kScaled ? d_inc + kRowsN : d_inc;
+        const uint32_t d_u = tmem + e * kRowsN, d_inc = d_u + NP * kRowsN, d_z = G::kScaled ? d_inc + kRowsN : d_inc;
         int chunk = 0;
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps && ok; ++sp) {
@@ -305,113 +343,306 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             if (leader && ok) mma_commit(u_done);
 #pragma unroll 1
             for (int ch = 0; ch < G::NCH; ++ch, ++chunk) {
-                wait(n_ready, chunk & 1);
-                constexpr int KC = G::BLK / G::NCH / NP;            // K blocks of a chunk
-#pragma unroll 1
-                for (int kc = 0; kc < KC; ++kc)
+                const int b = chunk & 1;
+                wait(&n_ready[b], (chunk >> 1) & 1);
 #pragma unroll
-                    for (int e = 0; e < NP; ++e)
-                        block(G::BLK + (ch * KC + kc) * NP + e, d_z + e * kRowsN,
-                              z0 + (uint64_t)((e * 2 * kZPart + kc * 4 * kZLbo) / 16), kZPart, 2 * kZLbo, id_z,
-                              ch == 0 && kc == 0);
-                if (leader && ok) mma_commit(n_free);
+                for (int k = 0; k < 2; ++k)
+                    block(G::BLK + 2 * ch + k, d_z, z0 + (uint64_t)(b * (G::ZB / 16) + k * (2 * kZLbo / 16)), kZPart, id_z,
+                          ch == 0 && k == 0);
+                if (leader && ok) mma_commit(&n_free[b]);
             }
             wait(v_ready, sp & 1);
             with_x(G::kScaled ? 0 : 2 * G::BLK, d_inc, G::kScaled);
             if (leader && ok) mma_commit(inc_done);
         }
-    } else if (warp < 2 + kWarps) {
-        // ---------------- the working warps
+    } else if (warp >= 2 && warp < 2 + kWork) {
+        // ---------------- force and update
         const int q = warp & 3;                                 // TMEM lane quarter
-        const int g = ((warp - 2) >> 2) + (M == 64 ? 4 * (q >> 1) : 0);   // chain group
         const int j = (32 * q + lane) & (M == 64 ? 63 : 127);   // bond (pair) and mode (pair) index
-        const bool lane0 = (32 * q & (M == 64 ? 63 : 127)) == 0;   // this warp holds mode 0
-        const int ks = (a.cpt + G::NG - 1) / G::NG;             // chain slots in use per group
-        const int cl0 = g * ks;                                 // this group's first chain of the tile
-        const int ns = max(0, min(ks, Ct - cl0));               // ... and its live chains
-        // first row of the group: 24 rows (3 axes x 8 slots) per 4 or 8 groups
-        const int pos0 = M == 64 ? 4 * (g >> 2) : 0;
-        const int row0 = 24 * (g & 3) + pos0;
-        const uint32_t tq = (uint32_t)(32 * q) << 16;
-        const uint32_t d_u = tmem + tq + (uint32_t)row0, d_inc = d_u + NP * kRowsN;
-        // this thread's 8 bytes of operand X: parity e, part, axis
-        uint8_t* xw = X + 3 * (g & 3) * kXSbo + j * 16 + pos0 * 2;
+        // the tile's batches of four chains: this warp takes b0, b0 + bs, ... of its lanes
+        const int b0 = ((warp - 2) >> 2) + (M == 64 ? 2 * (q >> 1) : 0), bs = M == 64 ? 4 : 2;
+        const int nb = (Ct + 3) >> 2;
+        const bool own0 = (32 * q & (M == 64 ? 63 : 127)) == 0 && lane == 0;   // this thread holds mode 0
+        const uint32_t d_u = tmem + ((uint32_t)(32 * q) << 16), d_inc = d_u + NP * kRowsN;
+        auto col = [](int b) { return 24 * (b >> 1) + 4 * (b & 1); };          // the batch's first row
+        uint8_t* xw = X + j * 16;
         float dm[NP], gw[NP], cs[NP], es[NP];
 #pragma unroll
         for (int e = 0; e < NP; ++e) {
             const float4 c = la.lane_c[NP * j + e];
             dm[e] = c.x; gw[e] = c.y; cs[e] = c.z; es[e] = c.w;
         }
-        bool ok = true, finite = true;
-        // the centre of mass (FP64): lane 3 s + axis of a warp that holds mode 0
-        const int ms = lane / 3, ma = lane - 3 * ms;
-        const bool cm_mine = lane0 && ms < ns;
-        double cm = cm_mine ? a.com[3 * (size_t)(c0 + cl0 + ms) + ma] : 0.0;
-
+        bool ok = true;
         auto arrive = [&](uint64_t* bar) {
             fence_before();
             fence_proxy_async();
             __syncwarp();
             if (lane == 0 && ok) mbar_arrive(bar);
         };
-        auto put_x = [&](const float (&x)[3][4], int e, int sb) {
-#pragma unroll
-            for (int ax = 0; ax < 3; ++ax) {
-                uint2 h, l;
-                split4(x[ax], h, l);
-                uint8_t* w = xw + e * 2 * kXPart + ax * kXSbo + sb * 2;
-                *reinterpret_cast<uint2*>(w) = h;
-                *reinterpret_cast<uint2*>(w + kXPart) = l;
-            }
+        auto store_x = [&](uint2 hi, uint2 lo, int e, int ax, int b) {
+            uint8_t* w = xw + e * 2 * kXPart + (3 * (b >> 1) + ax) * kXSbo + (b & 1) * 8;
+            *reinterpret_cast<uint2*>(w) = hi;
+            *reinterpret_cast<uint2*>(w + kXPart) = lo;
         };
-        // the modes (2 j, 2 j + 1) or j of four chains, [parity][axis][chain]
-        auto load_r = [&](float (&r)[NP][3][4], int sb) {
+        // the modes (2 j, 2 j + 1) or j of a batch in global memory and in TMEM,
+        // [parity][axis][chain]; chains past the tile's last are zero
+        float* Rj = a.R + (size_t)3 * c0 * M + NP * j;
+        auto load_r = [&](float (&r)[NP][3][4], int b) {
+            const float* p = Rj + (size_t)(12 * b) * M;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i) {
+                const bool live = 4 * b + i < Ct;
 #pragma unroll
                 for (int ax = 0; ax < 3; ++ax) {
-                    const float* p = a.R + (size_t)(3 * (c0 + cl0 + sb + i) + ax) * M + NP * j;
                     if constexpr (NP == 2) {
-                        const float2 x = sb + i < ns ? *reinterpret_cast<const float2*>(p) : make_float2(0.f, 0.f);
+                        const float2 x = live ? *reinterpret_cast<const float2*>(p + (3 * i + ax) * M) : make_float2(0.f, 0.f);
                         r[0][ax][i] = x.x;
                         r[NP - 1][ax][i] = x.y;
                     } else {
-                        r[0][ax][i] = sb + i < ns ? *p : 0.f;
+                        r[0][ax][i] = live ? p[(3 * i + ax) * M] : 0.f;
                     }
-                }
-        };
-        auto put_r = [&](const float (&r)[NP][3][4], int sb) {
-#pragma unroll
-            for (int e = 0; e < NP; ++e) {
-                if constexpr (G::kScaled) {
-                    float x[3][4];
-#pragma unroll
-                    for (int ax = 0; ax < 3; ++ax)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) x[ax][i] = cs[e] * r[e][ax][i];
-                    put_x(x, e, sb);
-                } else {
-                    put_x(r[e], e, sb);
                 }
             }
         };
+        auto store_r = [&](const float (&r)[NP][3][4], int b) {
+            float* p = Rj + (size_t)(12 * b) * M;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (4 * b + i < Ct)
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) {
+                        if constexpr (NP == 2)
+                            *reinterpret_cast<float2*>(p + (3 * i + ax) * M) = make_float2(r[0][ax][i], r[NP - 1][ax][i]);
+                        else
+                            p[(3 * i + ax) * M] = r[0][ax][i];
+                    }
+        };
+        const uint32_t r_col = d_u + G::kRCol;
+        auto fetch_r = [&](float (&r)[NP][3][4], int b) {       // before a tmem_wait12
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(r_col + (b * NP + e) * 12 + 4 * ax, r[e][ax]);
+        };
+        auto keep_r = [&](const float (&r)[NP][3][4], int b) {
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) tmem_st4(r_col + (b * NP + e) * 12 + 4 * ax, r[e][ax]);
+        };
+        auto put_r = [&](const float (&r)[NP][3][4], int b) {
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) {
+                    uint2 h, l;
+                    if constexpr (G::kScaled) {
+                        const float x[4] = {cs[e] * r[e][ax][0], cs[e] * r[e][ax][1], cs[e] * r[e][ax][2], cs[e] * r[e][ax][3]};
+                        split4(x, h, l);
+                    } else {
+                        split4(r[e][ax], h, l);
+                    }
+                    store_x(h, l, e, ax, b);
+                }
+        };
+        // bond vectors -> residual force v (Eq. e11) of a batch, two chains at a time
+        // (packed FP32)
+        auto force4 = [&](int b) {
+            float u[NP][3][4];
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + e * kRowsN + 8 * ax + col(b), u[e][ax]);
+#pragma unroll
+            for (int e = 0; e < NP; ++e) tmem_wait12(u[e]);
+            uint2 xh[NP][3], xl[NP][3];
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+                f32x2 w[NP][3];
+#pragma unroll
+                for (int e = 0; e < NP; ++e)
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) w[e][ax] = pack2(u[e][ax][i], u[e][ax][i + 1]);
+                if constexpr (NP == 2) {
+                    f32x2 p[3], m[3];     // bonds j and M - j
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) {
+                        p[ax] = add2(w[NP - 1][ax], w[0][ax]);
+                        m[ax] = sub2(w[NP - 1][ax], w[0][ax]);
+                    }
+                    const f32x2 fp = add2(rsqrt2(fma2(p[0], p[0], fma2(p[1], p[1], mul2(p[2], p[2])))), both2(-a.c12nu));
+                    const f32x2 fm = add2(rsqrt2(fma2(m[0], m[0], fma2(m[1], m[1], mul2(m[2], m[2])))), both2(-a.c12nu));
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) {
+                        const f32x2 vm = mul2(m[ax], fm);
+                        w[0][ax] = fma2(p[ax], fp, mul2(vm, both2(-1.0f)));      // even modes
+                        w[NP - 1][ax] = fma2(p[ax], fp, vm);                     // odd modes
+                    }
+                } else {
+                    const f32x2 f = add2(rsqrt2(fma2(w[0][0], w[0][0], fma2(w[0][1], w[0][1], mul2(w[0][2], w[0][2])))),
+                                         both2(-a.c12nu));
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) w[0][ax] = j >= 1 ? mul2(w[0][ax], f) : 0ull;   // v_0 = 0
+                }
+#pragma unroll
+                for (int e = 0; e < NP; ++e)
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) {
+                        if (i == 0) split2(w[e][ax], xh[e][ax].x, xl[e][ax].x);
+                        else split2(w[e][ax], xh[e][ax].y, xl[e][ax].y);
+                    }
+            }
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) store_x(xh[e][ax], xl[e][ax], e, ax, b);
+        };
+        // update (Eqs. d3, btum) of a batch whose modes are in r (tm: in TMEM)
+        auto update4 = [&](float (&r)[NP][3][4], int b, int sp, bool tm, bool plain) {
+            float d[NP][3][4];
+            if (tm) fetch_r(r, b);
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + e * kRowsN + 8 * ax + col(b), d[e][ax]);
+            if constexpr (G::kScaled) {
+                float dz[3][4];
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + kRowsN + 8 * ax + col(b), dz[ax]);
+                tmem_wait12(d[0]);
+                tmem_wait12(dz);
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) d[0][ax][i] = fmaf(es[0], d[0][ax][i], dz[ax][i]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < NP; ++e) tmem_wait12(d[e]);
+            }
+            if (tm) {
+#pragma unroll
+                for (int e = 0; e < NP; ++e) tmem_wait12(r[e]);
+            }
+            if (own0) {
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax)
+                    *reinterpret_cast<float4*>(s_d0 + 32 * ax + 4 * b) = make_float4(d[0][ax][0], d[0][ax][1], d[0][ax][2], d[0][ax][3]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (plain || sp < s_left[4 * b + i]) {      // a chain at its stop step stays as it is
+#pragma unroll
+                    for (int e = 0; e < NP; ++e) {
+                        const float ry = r[e][1][i];
+#pragma unroll
+                        for (int ax = 0; ax < 3; ++ax) r[e][ax][i] += fmaf(-dm[e], r[e][ax][i], d[e][ax][i]);
+                        if (!plain) r[e][0][i] = fmaf(__fmul_rn(s_shf[4 * b + i], gw[e]), ry, r[e][0][i]);
+                    }
+                }
+            }
+            put_r(r, b);
+            if (tm) keep_r(r, b);
+            else store_r(r, b);
+        };
 
-        // Normals of a noise chunk (Eq. b5): 64 K indices of step sp, chunk ch.  A
-        // lane draws four consecutive beads of a chain (three Philox calls) and,
-        // with the mirror symmetry, their four mirror images, and writes the sums
-        // and differences as 8 bytes of a row of the noise operand: 16 lanes fill
-        // a chain's row.  The chunk's items go to the warps in turn, starting one
-        // warp group further from chunk to chunk.
-        auto noise = [&](int sp, int ch, int chunk) {
-            const int items = (Ct + 1) >> 1;                    // two chains per item
-            const int item = (warp - 2 + 8 * chunk) & (kWarps - 1);
-            const int cl = 2 * item + (lane >> 4), t = lane & 15;
-            const bool mine = item < items && cl < Ct;
-            uint2 hi[NP][3], lo[NP][3];
-            if (mine) {
-                const uint32_t job = s_job[cl];
-                const int64_t st = s_step[cl] + sp;
-                const uint32_t b4 = (uint32_t)(16 * ch + t);    // beads 4 b4 ...
+        // operand X of the first step
+#pragma unroll 1
+        for (int b = b0; b < nb; b += bs) {
+            float r[NP][3][4];
+            load_r(r, b);
+            if (own0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) r[0][0][i] = r[0][1][i] = r[0][2][i] = 0.f;
+            }
+            put_r(r, b);
+            if (b < G::TB) keep_r(r, b);
+        }
+        tmem_wait_st();
+        arrive(r_ready);
+#pragma unroll 1
+        for (int sp = 0; sp < a.n_steps; ++sp) {
+            ok = ok && mbar_wait(u_done, sp & 1, a.err, abort_flag);
+            fence_after();
+#pragma unroll 1
+            for (int b = b0; b < nb; b += bs) force4(b);
+            arrive(v_ready);
+            // a batch whose modes are in global memory is updated last; they come from L2
+            // while the forward MMAs run
+            float rg[NP][3][4];
+            const int bg = b0 + bs * ((G::TB - b0 + bs - 1) / bs);      // this warp's first one
+            if (G::TB < 8 && bg < nb) load_r(rg, bg);
+            ok = ok && mbar_wait(inc_done, sp & 1, a.err, abort_flag);
+            fence_after();
+#pragma unroll 1
+            for (int b = b0; b < min(nb, G::TB); b += bs) {
+                float r[NP][3][4];
+                if (steady) update4(r, b, sp, true, true);
+                else update4(r, b, sp, true, false);
+            }
+            if constexpr (G::TB < 8) {
+#pragma unroll 1
+                for (int b = bg; b < nb; b += bs) {
+                    if (b != bg) load_r(rg, b);
+                    update4(rg, b, sp, false, steady);
+                }
+            }
+            tmem_wait_st();
+            arrive(r_ready);
+        }
+        // the state back to global memory; mode 0, whose table columns are zero, has only
+        // summed up its noise (the centre of mass is warp 19's).  A non-finite mode stays
+        // non-finite: looked at once per launch.
+        bool finite = true;
+#pragma unroll 1
+        for (int b = b0; b < nb; b += bs) {
+            float r[NP][3][4];
+            if (b < G::TB) {
+                fetch_r(r, b);
+#pragma unroll
+                for (int e = 0; e < NP; ++e) tmem_wait12(r[e]);
+            } else {
+                load_r(r, b);
+            }
+            if (own0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) r[0][0][i] = r[0][1][i] = r[0][2][i] = 0.f;
+            }
+            if (ok) store_r(r, b);
+#pragma unroll
+            for (int e = 0; e < NP; ++e)
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) finite = finite && (4 * b + i >= Ct || isfinite(r[e][ax][i]));
+        }
+        if (!finite) atomicOr(a.err, 1);
+    } else if (warp >= 2 + kWork && warp < 2 + kWork + kNoise) {
+        // ---------------- normals (Eq. b5), drawn ahead of the step, 32 K indices of
+        // each parity at a time, into two buffers in turn.  A lane draws four
+        // consecutive beads of a chain (three Philox calls) and, with the mirror
+        // symmetry, their four mirror images, and writes the sums and differences as
+        // 8 bytes of a row of the noise operand: 8 lanes fill a chain's row, a warp
+        // takes four chains (a batch).
+        const int nw = warp - 2 - kWork;
+        const int t = lane & 7;
+        bool ok = true;
+        const int chunks = a.n_steps * G::NCH;
+        static_assert(G::NCH % 2 == 0, "chunks in pairs");
+        // Both chunks of a pair are drawn before either is written, so that the second
+        // half of a step's normals waits in registers for the first half's MMAs.
+#pragma unroll 1
+        for (int chunk = 0; chunk < chunks; chunk += 2) {
+            const int sp = chunk / G::NCH, ch = chunk - G::NCH * sp;
+            uint2 hi[2][NP][3], lo[2][NP][3];
+            // with fewer batches than warps, a chunk's batches go to other warps than the last one's
+            const int cl[2] = {4 * ((nw + 5 * chunk) & (kNoise - 1)) + (lane >> 3),
+                               4 * ((nw + 5 * chunk + 5) & (kNoise - 1)) + (lane >> 3)};
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (cl[k] >= Ct) continue;
+                const uint32_t job = s_job[cl[k]];
+                const int64_t st = s_step[cl[k]] + sp;
+                const uint32_t b4 = (uint32_t)(8 * (ch + k) + t);       // beads 4 b4 ...
                 float z[3][4];
                 bead_quad_normals<float>(a.seed, job, st, b4, 0u, z);
                 if constexpr (NP == 2) {
@@ -425,183 +656,62 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                             s[i] = z[ax][i] + y[ax][3 - i];
                             d[i] = z[ax][i] - y[ax][3 - i];
                         }
-                        split4(s, hi[0][ax], lo[0][ax]);
-                        split4(d, hi[NP - 1][ax], lo[NP - 1][ax]);
+                        split4(s, hi[k][0][ax], lo[k][0][ax]);
+                        split4(d, hi[k][NP - 1][ax], lo[k][NP - 1][ax]);
                     }
                 } else {
 #pragma unroll
-                    for (int ax = 0; ax < 3; ++ax) split4(z[ax], hi[0][ax], lo[0][ax]);
+                    for (int ax = 0; ax < 3; ++ax) split4(z[ax], hi[k][0][ax], lo[k][0][ax]);
                 }
             }
-            // the previous chunk's MMAs have read the operand
-            if (chunk > 0) ok = ok && mbar_wait(n_free, (chunk - 1) & 1, a.err, abort_flag);
-            if (mine && ok) {
-                const int cg = cl / ks, cs_ = cl - cg * ks;
-                uint8_t* w = Z + (t >> 1) * kZLbo + 3 * (cg & 3) * 128 + ((M == 64 ? 4 * (cg >> 2) : 0) + cs_) * 16 + (t & 1) * 8;
 #pragma unroll
-                for (int e = 0; e < NP; ++e)
-#pragma unroll
-                    for (int ax = 0; ax < 3; ++ax) {
-                        *reinterpret_cast<uint2*>(w + e * 2 * kZPart + ax * 128) = hi[e][ax];
-                        *reinterpret_cast<uint2*>(w + e * 2 * kZPart + kZPart + ax * 128) = lo[e][ax];
-                    }
-            }
-            arrive(n_ready);
-        };
-
-        // operand X of the first step
-        for (int sb = 0; sb < ns; sb += 4) {
-            float r[NP][3][4];
-            load_r(r, sb);
-            put_r(r, sb);
-        }
-        arrive(r_ready);
-        int chunk = 0;
-        if constexpr (G::NCH == 2) noise(0, 0, chunk++);
-        // phases of half a step: even ones form the force, odd ones update the modes;
-        // each is followed by a chunk of normals drawn ahead
-#pragma unroll 1
-        for (int ph = -1; ph < 2 * a.n_steps; ++ph) {
-            const int sp = ph >> 1;
-            if (ph >= 0 && (ph & 1) == 0) {
-                // ---- bond vectors -> residual force v (Eq. e11)
-                ok = ok && mbar_wait(u_done, sp & 1, a.err, abort_flag);
-                fence_after();
-#pragma unroll 1
-                for (int sb = 0; sb < ns; sb += 4) {
-                    float u[NP][3][4];
+            for (int k = 0; k < 2; ++k) {
+                // the MMAs have read the chunk that this buffer held
+                if (chunk >= 2) ok = ok && mbar_wait(&n_free[k], ((chunk >> 1) - 1) & 1, a.err, abort_flag);
+                if (cl[k] < Ct && ok) {
+                    const int b = cl[k] >> 2;
+                    uint8_t* w = Z + k * G::ZB + (t >> 1) * kZLbo + 3 * (b >> 1) * 128 + (4 * (b & 1) + (cl[k] & 3)) * 16 + (t & 1) * 8;
 #pragma unroll
                     for (int e = 0; e < NP; ++e)
-#pragma unroll
-                        for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + e * kRowsN + 8 * ax + sb, u[e][ax]);
-#pragma unroll
-                    for (int e = 0; e < NP; ++e) tmem_wait12(u[e]);
-                    if constexpr (NP == 2) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float p[3], m[3];     // bonds j and M - j
-#pragma unroll
-                            for (int ax = 0; ax < 3; ++ax) {
-                                p[ax] = u[NP - 1][ax][i] + u[0][ax][i];
-                                m[ax] = u[NP - 1][ax][i] - u[0][ax][i];
-                            }
-                            const float fp = rsqrtf(fmaf(p[0], p[0], fmaf(p[1], p[1], p[2] * p[2]))) - a.c12nu;
-                            const float fm = rsqrtf(fmaf(m[0], m[0], fmaf(m[1], m[1], m[2] * m[2]))) - a.c12nu;
-#pragma unroll
-                            for (int ax = 0; ax < 3; ++ax) {
-                                const float vm = m[ax] * fm;
-                                u[0][ax][i] = fmaf(p[ax], fp, -vm);          // even modes
-                                u[NP - 1][ax][i] = fmaf(p[ax], fp, vm);      // odd modes
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float f = rsqrtf(fmaf(u[0][0][i], u[0][0][i], fmaf(u[0][1][i], u[0][1][i], u[0][2][i] * u[0][2][i]))) -
-                                      a.c12nu;
-#pragma unroll
-                            for (int ax = 0; ax < 3; ++ax) u[0][ax][i] = j >= 1 ? u[0][ax][i] * f : 0.f;   // v_0 = 0
-                        }
-                    }
-#pragma unroll
-                    for (int e = 0; e < NP; ++e) put_x(u[e], e, sb);
-                }
-                arrive(v_ready);
-            } else if (ph >= 0) {
-                // ---- update (Eqs. d3, btum)
-                float r[NP][3][4];
-                if (ns > 0) load_r(r, 0);
-                ok = ok && mbar_wait(inc_done, sp & 1, a.err, abort_flag);
-                fence_after();
-                const bool last = sp == a.n_steps - 1;
-#pragma unroll 1
-                for (int sb = 0; sb < ns; sb += 4) {
-                    float d[NP][3][4];
-#pragma unroll
-                    for (int e = 0; e < NP; ++e)
-#pragma unroll
-                        for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + e * kRowsN + 8 * ax + sb, d[e][ax]);
-                    float dz[3][4];
-                    if constexpr (G::kScaled) {
-#pragma unroll
-                        for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + kRowsN + 8 * ax + sb, dz[ax]);
-                    }
-                    if (sb > 0) load_r(r, sb);
-#pragma unroll
-                    for (int e = 0; e < NP; ++e) tmem_wait12(d[e]);
-                    if constexpr (G::kScaled) {
-                        tmem_wait12(dz);
-#pragma unroll
-                        for (int ax = 0; ax < 3; ++ax)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) d[0][ax][i] = fmaf(es[0], d[0][ax][i], dz[ax][i]);
-                    }
-                    if (lane0 && lane == 0) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (sb + i < ns)
-#pragma unroll
-                                for (int ax = 0; ax < 3; ++ax) s_d0[3 * (cl0 + sb + i) + ax] = d[0][ax][i];
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (sb + i >= ns) break;
-                        if (sp < s_left[cl0 + sb + i]) {        // a chain at its stop step stays as it is
-                            const float sh = has_shear ? s_shf[cl0 + sb + i] : 0.f;
-#pragma unroll
-                            for (int e = 0; e < NP; ++e) {
-                                const float ry = r[e][1][i];
-#pragma unroll
-                                for (int ax = 0; ax < 3; ++ax) {
-                                    const float x = r[e][ax][i];
-                                    r[e][ax][i] = x + fmaf(-dm[e], x, d[e][ax][i]);
-                                }
-                                if (has_shear) r[e][0][i] += sh * gw[e] * ry;
-                            }
-                        }
-                        if (lane0 && lane == 0) r[0][0][i] = r[0][1][i] = r[0][2][i] = 0.f;   // the centre of mass is cm
 #pragma unroll
                         for (int ax = 0; ax < 3; ++ax) {
-                            float* p = a.R + (size_t)(3 * (c0 + cl0 + sb + i) + ax) * M + NP * j;
-                            if constexpr (NP == 2)
-                                *reinterpret_cast<float2*>(p) = make_float2(r[0][ax][i], r[NP - 1][ax][i]);
-                            else
-                                *p = r[0][ax][i];
+                            *reinterpret_cast<uint2*>(w + e * 2 * kZPart + ax * 128) = hi[k][e][ax];
+                            *reinterpret_cast<uint2*>(w + e * 2 * kZPart + kZPart + ax * 128) = lo[k][e][ax];
                         }
-                        // a non-finite mode stays non-finite: looked at once per launch
-                        if (last) {
-#pragma unroll
-                            for (int e = 0; e < NP; ++e)
-#pragma unroll
-                                for (int ax = 0; ax < 3; ++ax) finite = finite && isfinite(r[e][ax][i]);
-                        }
-                    }
-                    if (!last) put_r(r, sb);
                 }
-                if (!last) arrive(r_ready);
-                if (lane0) {
-                    // centre of mass (p = 0 of Eq. d3 with zeta_0 = 0) in FP64
-                    __syncwarp();
-                    const double ycm = has_shear ? __shfl_down_sync(0xffffffffu, cm, 1) : 0.0;
-                    if (cm_mine && sp < s_left[cl0 + ms]) {
-                        double x = (double)s_d0[3 * (cl0 + ms) + ma] * a.inv_sqrtM;
-                        if (has_shear && ma == 0) x += s_shear[cl0 + ms] * a.dtau * ycm;
-                        cm += x;
-                    }
-                    __syncwarp();
-                }
-            }
-            // normals drawn ahead: chunk 0 of step s + 1 after the force of step s, the
-            // last chunk of step s + 1 after the update of step s
-            const int zs = (ph + 2) >> 1;
-            if (zs < a.n_steps) {
-                if (G::NCH == 2) noise(zs, (ph & 1) ? 1 : 0, chunk++);
-                else if (ph & 1) noise(zs, 0, chunk++);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0 && ok) mbar_arrive(&n_ready[k]);
             }
         }
-        if (ok && cm_mine) a.com[3 * (size_t)(c0 + cl0 + ms) + ma] = cm;
-        if (ok && lane0 && lane < ns) a.step[c0 + cl0 + lane] = s_step[cl0 + lane] + s_left[cl0 + lane];
-        if (!finite) atomicOr(a.err, 1);
+    } else if (warp == 19) {
+        // ---------------- the centre of mass (p = 0 of Eq. d3 with zeta_0 = 0) in
+        // FP64, a chain per lane, and the step counters
+        bool ok = true;
+        const bool live = lane < Ct;
+        double cm[3] = {0.0, 0.0, 0.0};
+        double* cg = a.com + 3 * (size_t)(c0 + lane);
+        if (live)
+            for (int ax = 0; ax < 3; ++ax) cm[ax] = cg[ax];
+        const double sh = __dmul_rn(s_shear[lane], a.dtau);
+        if (lane == 0) mbar_arrive(v_ready);
+        ok = mbar_wait(r_ready, 0, a.err, abort_flag);      // every phase in turn
+#pragma unroll 1
+        for (int sp = 0; sp < a.n_steps; ++sp) {
+            ok = ok && mbar_wait(r_ready, (sp + 1) & 1, a.err, abort_flag);
+            if (ok && live && sp < s_left[lane]) {
+                const double ycm = cm[1];
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) cm[ax] = fma((double)s_d0[32 * ax + lane], a.inv_sqrtM, cm[ax]);
+                if (has_shear) cm[0] = fma(sh, ycm, cm[0]);
+            }
+            __syncwarp();
+            if (lane == 0 && ok && sp + 1 < a.n_steps) mbar_arrive(v_ready);
+        }
+        if (ok && live) {
+            for (int ax = 0; ax < 3; ++ax) cg[ax] = cm[ax];
+            a.step[c0 + lane] = s_step[lane] + s_left[lane];
+        }
     }
     fence_before();
     __syncthreads();
