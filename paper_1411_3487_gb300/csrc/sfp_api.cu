@@ -305,23 +305,39 @@ int upload_typed(sfp_batch* b, void* dst, const std::vector<double>& src)
 
 unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// One or two FP32 products (n of them) of the same shape in one launch of k_gemm_f32.
+// 64 x 64 tiles, and 32 x 32 ones where 64 x 64 would not give every SM a block
+// (measured, us: 600 x 128 x 128, 20 blocks, 10.3 and 6.3; 150 x 1000 x 1000 51 and
+// 31; 6003 x 100 x 100, 188 blocks, 10.4 both; 12288 x 256 x 256 45 and 64; 128 x 128
+// tiles of 8 x 8 outputs per thread: 59, and never ahead up to 49152 x 512 x 512).
+cudaError_t gemm_f32(cudaStream_t st, const sfp::GemmF32& g, int n, int J, int Nc, int K)
+{
+    bool vec = K % 4 == 0;
+    for (int z = 0; z < n; ++z)
+        vec = vec && ((uintptr_t)g.in[z] | (uintptr_t)g.b[z] | (uintptr_t)g.out[z]) % 16 == 0;
+    if ((int64_t)nblk(Nc, 64) * nblk(J, 64) * n >= 152) {
+        const dim3 grid(nblk(Nc, 64), nblk(J, 64), (unsigned)n);
+        if (vec) sfp::k_gemm_f32<64, 64, 8, 4, true><<<grid, 128, 0, st>>>(g, J, Nc, K);
+        else sfp::k_gemm_f32<64, 64, 8, 4, false><<<grid, 128, 0, st>>>(g, J, Nc, K);
+    } else {
+        const dim3 grid(nblk(Nc, 32), nblk(J, 32), (unsigned)n);
+        if (vec) sfp::k_gemm_f32<32, 32, 4, 4, true><<<grid, 64, 0, st>>>(g, J, Nc, K);
+        else sfp::k_gemm_f32<32, 32, 4, 4, false><<<grid, 64, 0, st>>>(g, J, Nc, K);
+    }
+    return cudaGetLastError();
+}
+
 template <typename T>
 int launch_gemm(sfp_batch* b, const T* In, const T* B, T* Out, int J, int Nc, int K)
 {
     if constexpr (sizeof(T) == 4) {
-        if (Nc >= 128) {
-            dim3 grid(nblk(Nc, 128), nblk(J, 128));
-            sfp::k_gemm_nt<float, 128, 128, 8, 8, 8><<<grid, 256, 0, b->cur>>>(In, B, Out, J, Nc, K);
-        } else {
-            dim3 grid(nblk(Nc, 64), nblk(J, 64));
-            sfp::k_gemm_nt<float, 64, 64, 8, 4, 4><<<grid, 256, 0, b->cur>>>(In, B, Out, J, Nc, K);
-        }
+        CUDA_TRY(gemm_f32(b->cur, sfp::GemmF32{{In, nullptr}, {B, nullptr}, {Out, nullptr}}, 1, J, Nc, K));
     } else {
         dim3 grid(nblk(Nc, 64), nblk(J, 64));
         sfp::k_gemm_nt<double, 64, 64, 8, 4, 4><<<grid, 256, 0, b->cur>>>(In, B, Out, J, Nc, K);
+        CUDA_TRY(cudaGetLastError());
     }
     b->launches++;
-    CUDA_TRY(cudaGetLastError());
     return SFP_OK;
 }
 
@@ -357,6 +373,19 @@ cudaError_t launch_noise(cudaStream_t st, T* z, int C, int M, uint32_t seed, con
 {
     const unsigned grid = nblk((int64_t)C * ((3 * M + 3) / 4), 256);
     sfp::k_noise<T><<<grid, 256, 0, st>>>(z, C, M, seed, job, step, tag);
+    return cudaGetLastError();
+}
+
+// Both in one launch (CUDA-core transforms).
+template <typename T>
+cudaError_t launch_force_noise(cudaStream_t st, const T* u, T* v, T* z, int C, int M, T c12nu, uint32_t seed,
+                               const uint32_t* job, const int64_t* step, uint32_t tag = 0u)
+{
+    const unsigned nf = nblk((int64_t)C * ((M + 3) / 4), 256), nz = nblk((int64_t)C * ((3 * M + 3) / 4), 256);
+    if (sizeof(T) == 4 && M % 4 == 0)
+        sfp::k_force_noise<T, true><<<nf + nz, 256, 0, st>>>(u, v, C, M, c12nu, nf, z, seed, job, step, tag);
+    else
+        sfp::k_force_noise<T, false><<<nf + nz, 256, 0, st>>>(u, v, C, M, c12nu, nf, z, seed, job, step, tag);
     return cudaGetLastError();
 }
 
@@ -642,9 +671,10 @@ int step_group(sfp_batch* b, Group& g)
     T* yz = (T*)g.yz;
     int rc;
     if ((rc = mark(b, 0))) return rc;
-    // a3: the bead noise depends on the step counters alone, so it runs on a
-    // stream of its own beside a1 and a2 (serially while stages are timed)
-    const bool side = !b->timing;
+    // a3: the bead noise depends on the step counters alone, so beside tensor-core
+    // transforms it runs on a stream of its own beside a1 and a2; beside CUDA-core
+    // transforms it shares a2's launch; while stages are timed, both in line
+    const bool side = !b->timing && g.tc, merged = !b->timing && !g.tc;
     // mode-keyed noise: Z drawn straight into the mode-space buffer, and the
     // forward transform forms DeltaH alone
     const bool mk = b->noise == SFP_NOISE_MODES;
@@ -664,20 +694,28 @@ int step_group(sfp_batch* b, Group& g)
     if (g.tc) b->launches++;
     if ((rc = mark(b, 1))) return rc;
     // a2: residual bond force v (Eq. e11)
-    CUDA_TRY(launch_force<T>(b->cur, r, fz, C, M, (T)(1.0 - 2.0 * b->dv.nu)));
+    if (merged)
+        CUDA_TRY(launch_force_noise<T>(b->cur, r, fz, znoise, C, M, (T)(1.0 - 2.0 * b->dv.nu), b->seed, g.job, g.step, ntag));
+    else
+        CUDA_TRY(launch_force<T>(b->cur, r, fz, C, M, (T)(1.0 - 2.0 * b->dv.nu)));
     b->launches++;
     if ((rc = mark(b, 2))) return rc;
     if (side) {
         CUDA_TRY(cudaStreamWaitEvent(b->cur, g.njoin, 0));
-    } else {
+    } else if (!merged) {
         CUDA_TRY(launch_noise<T>(b->cur, znoise, C, M, b->seed, g.job, g.step, ntag));
         b->launches++;
     }
     if ((rc = mark(b, 3))) return rc;
     // a4: DeltaH = chi^T v (Eq. e11), Z = phi^T z (Eq. c4): the forward transform
     if (g.tc) rc = sfp::tc_transform(g.tc, mk ? 2 : 1, b->cur);
-    else if (!(rc = launch_gemm<T>(b, fz, (const T*)g.chiT, yz, 3 * C, M, M)) && !mk)
+    else if constexpr (sizeof(T) == 4) {
+        CUDA_TRY(gemm_f32(b->cur, sfp::GemmF32{{fz, fz + n}, {(const T*)g.chiT, (const T*)g.phiT}, {yz, yz + n}}, mk ? 1 : 2,
+                          3 * C, M, M));
+        b->launches++;
+    } else if (!(rc = launch_gemm<T>(b, fz, (const T*)g.chiT, yz, 3 * C, M, M)) && !mk) {
         rc = launch_gemm<T>(b, fz + n, (const T*)g.phiT, yz + n, 3 * C, M, M);
+    }
     if (rc) return rc;
     if (g.tc) b->launches++;
     if ((rc = mark(b, 4))) return rc;
@@ -1062,19 +1100,6 @@ __global__ void k_noalloc_prep(float* R, int64_t* step, uint32_t* job, double* s
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-template <typename T>
-cudaError_t gemm_on(cudaStream_t st, const T* In, const T* B, T* Out, int J, int Nc, int K)
-{
-    if (Nc >= 128) {
-        dim3 grid(nblk(Nc, 128), nblk(J, 128));
-        sfp::k_gemm_nt<T, 128, 128, 8, 8, 8><<<grid, 256, 0, st>>>(In, B, Out, J, Nc, K);
-    } else {
-        dim3 grid(nblk(Nc, 64), nblk(J, 64));
-        sfp::k_gemm_nt<T, 64, 64, 8, 4, 4><<<grid, 256, 0, st>>>(In, B, Out, J, Nc, K);
-    }
-    return cudaGetLastError();
-}
 
 // sfp_set_modes body for host element type S (double or float).
 template <typename S>
@@ -2058,11 +2083,9 @@ int sfp_step_noalloc(const sfp_params* params, const sfp_chain_desc* chain, int3
     const double w0 = std::sqrt(2.0 * dv.Tstar * dtau);
     int* bad = (int*)(base + o_bad);   // written by the update kernel, not reported here
     for (int64_t s = 0; s < n_steps; ++s) {
-        CUDA_TRY(gemm_on<float>(st, modes_dev, chi, r, 3 * C, M, M));
-        CUDA_TRY(launch_force<float>(st, r, fz, C, M, c12));
-        CUDA_TRY(launch_noise<float>(st, fz + n, C, M, (uint32_t)seed, job, step));
-        CUDA_TRY(gemm_on<float>(st, fz, chiT, yz, 3 * C, M, M));
-        CUDA_TRY(gemm_on<float>(st, fz + n, phiT, yz + n, 3 * C, M, M));
+        CUDA_TRY(gemm_f32(st, sfp::GemmF32{{modes_dev, nullptr}, {chi, nullptr}, {r, nullptr}}, 1, 3 * C, M, M));
+        CUDA_TRY(launch_force_noise<float>(st, r, fz, fz + n, C, M, c12, (uint32_t)seed, job, step));
+        CUDA_TRY(gemm_f32(st, sfp::GemmF32{{fz, fz + n}, {chiT, phiT}, {yz, yz + n}}, 2, 3 * C, M, M));
         CUDA_TRY(launch_mode_update<float>(st, modes_dev, yz, yz + n, com_dev, step, dm, h, w, g, shear, C, M, w0,
                                            dtau, bad, nullptr));
     }

@@ -70,6 +70,144 @@ k_gemm_nt(const T* __restrict__ In, const T* __restrict__ B, T* __restrict__ Out
 }
 
 // ---------------------------------------------------------------------------
+// The same product in FP32 (the plain path, and every length that the tensor-core
+// kernels do not take): Out_z[j][i] = sum_k In_z[j][k] B_z[i][k], blockIdx.z picks the
+// product (the forward transform's two are one launch).  Block tile BM x BN, K chunks
+// of 16 in two shared-memory buffers (the next chunk's loads are in registers while
+// one is multiplied), TM x TN outputs per thread as TM / 2 pairs of rows
+// (fma.rn.f32x2); every output sums k in ascending order.  VEC: K % 4 == 0 and
+// 16-byte-aligned operands (float4 loads and stores).
+// Bound by FP32 issue on large shapes (48 of 80 TFLOP/s at 49152 x 512 x 512, 36 at
+// 12288 x 256 x 256), by the latency of one block per SM on small ones (19 us for
+// 3072 x 256 x 256, inverse).  With k_gemm_nt's 128 x 128 tiles (scalar loads, one
+// buffer, 48 blocks on 152 SMs) a step of 1024 x 256 beads took 287 us, here 57; 2001
+// x 100 beads 83 and 37, 4096 x 256 beads 396 and 142, 50 x 1000 beads 1099 and 107.
+// ---------------------------------------------------------------------------
+struct GemmF32 {
+    const float* in[2];
+    const float* b[2];
+    float* out[2];
+};
+
+template <int BM, int BN, int TM, int TN, bool VEC>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+k_gemm_f32(const GemmF32 g, int J, int N, int K)
+{
+    constexpr int NT = (BM / TM) * (BN / TN), BK = 16;
+    constexpr int LA = BM + 4, LB = BN + 4;                     // row pitches of the k-major tiles
+    constexpr int QA = BM * BK / 4 / NT, QB = BN * BK / 4 / NT; // float4 loads per thread and chunk
+    static_assert(QA * NT * 4 == BM * BK && QB * NT * 4 == BN * BK && TM % 4 == 0 && TN % 4 == 0, "tile split");
+    __shared__ __align__(16) float As[2][BK][LA];
+    __shared__ __align__(16) float Bs[2][BK][LB];
+    const float* __restrict__ In = blockIdx.z ? g.in[1] : g.in[0];
+    const float* __restrict__ B = blockIdx.z ? g.b[1] : g.b[0];
+    float* __restrict__ Out = blockIdx.z ? g.out[1] : g.out[0];
+    const int tid = threadIdx.x, tx = tid % (BN / TN), ty = tid / (BN / TN);
+    const int j0 = blockIdx.y * BM, i0 = blockIdx.x * BN;
+    float4 ra[QA], rb[QB];
+    auto fetch4 = [&](const float* __restrict__ p, int row, int rows, int k) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < rows) {
+            const float* q = p + (size_t)row * K + k;
+            if constexpr (VEC) {
+                if (k < K) x = *reinterpret_cast<const float4*>(q);
+            } else {
+                if (k < K) x.x = q[0];
+                if (k + 1 < K) x.y = q[1];
+                if (k + 2 < K) x.z = q[2];
+                if (k + 3 < K) x.w = q[3];
+            }
+        }
+        return x;
+    };
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < QA; ++q) {
+            const int e = tid + NT * q;
+            ra[q] = fetch4(In, j0 + (e >> 2), J, k0 + 4 * (e & 3));
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int e = tid + NT * q;
+            rb[q] = fetch4(B, i0 + (e >> 2), N, k0 + 4 * (e & 3));
+        }
+    };
+    auto put = [&](int buf) {
+#pragma unroll
+        for (int q = 0; q < QA; ++q) {
+            const int e = tid + NT * q, m = e >> 2, k = 4 * (e & 3);
+            As[buf][k][m] = ra[q].x; As[buf][k + 1][m] = ra[q].y; As[buf][k + 2][m] = ra[q].z; As[buf][k + 3][m] = ra[q].w;
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int e = tid + NT * q, m = e >> 2, k = 4 * (e & 3);
+            Bs[buf][k][m] = rb[q].x; Bs[buf][k + 1][m] = rb[q].y; Bs[buf][k + 2][m] = rb[q].z; Bs[buf][k + 3][m] = rb[q].w;
+        }
+    };
+    f32x2 acc[TM / 2][TN];
+#pragma unroll
+    for (int x = 0; x < TM / 2; ++x)
+#pragma unroll
+        for (int y = 0; y < TN; ++y) acc[x][y] = 0ull;
+    fetch(0);
+    put(0);
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = 0; k0 < K; k0 += BK) {
+        const bool more = k0 + BK < K;
+        if (more) fetch(k0 + BK);
+#pragma unroll
+        for (int kk = 0; kk < BK; ++kk) {
+            f32x2 a[TM / 2], b[TN];
+#pragma unroll
+            for (int x = 0; x < TM / 4; ++x) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][ty * TM + 4 * x]);
+                a[2 * x] = v.x;
+                a[2 * x + 1] = v.y;
+            }
+#pragma unroll
+            for (int y = 0; y < TN / 4; ++y) {
+                const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * TN + 4 * y]);
+                b[4 * y] = both2(v.x); b[4 * y + 1] = both2(v.y); b[4 * y + 2] = both2(v.z); b[4 * y + 3] = both2(v.w);
+            }
+#pragma unroll
+            for (int x = 0; x < TM / 2; ++x)
+#pragma unroll
+                for (int y = 0; y < TN; ++y) acc[x][y] = fma2(a[x], b[y], acc[x][y]);
+        }
+        if (more) {
+            put(buf ^ 1);           // the other buffer's readers passed the last barrier
+            __syncthreads();
+            buf ^= 1;
+        }
+    }
+#pragma unroll
+    for (int x = 0; x < TM; ++x) {
+        const int gj = j0 + ty * TM + x;
+        if (gj >= J) continue;
+        float o[TN];
+#pragma unroll
+        for (int y = 0; y < TN; ++y) {
+            float lo, hi;
+            unpack2(acc[x / 2][y], lo, hi);
+            o[y] = x & 1 ? hi : lo;
+        }
+#pragma unroll
+        for (int y = 0; y < TN; y += 4) {
+            const int gi = i0 + tx * TN + y;
+            float* q = Out + (size_t)gj * N + gi;
+            if (VEC && N % 4 == 0) {
+                if (gi < N) *reinterpret_cast<float4*>(q) = make_float4(o[y], o[y + 1], o[y + 2], o[y + 3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (gi + i < N) q[i] = o[y + i];
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Residual bond force (Eqs. e4, e5, e11), from bond vectors:
 //   u_n = sum_p chi_{n,p} R_p (given, n >= 1; slot 0 holds 0),
 //   v_n = u_n (1/|u_n| - (1 - 2nu)) for n >= 1, v_0 = 0,
@@ -90,11 +228,9 @@ __device__ __forceinline__ void residual_v(const T u[3], bool ok, T c12nu, T v[3
 }
 
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(256)
-k_force(const T* __restrict__ ub, T* __restrict__ vb, int C, int M, T c12nu)
+__device__ __forceinline__ void force_quad(const T* __restrict__ ub, T* __restrict__ vb, int C, int M, T c12nu, int64_t t)
 {
     const int Q = (M + 3) >> 2;                    // bond quads per chain
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)C * Q) return;
     const int c = (int)(t / Q), n0 = 4 * (int)(t - (int64_t)c * Q);
     const size_t base = (size_t)c * 3 * M;
@@ -145,12 +281,10 @@ k_force(const T* __restrict__ ub, T* __restrict__ vb, int C, int M, T c12nu)
 // beside the inverse transform.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256)
-k_noise(T* __restrict__ z, int C, int M, uint32_t seed, const uint32_t* __restrict__ job,
-        const int64_t* __restrict__ step, uint32_t tag)
+__device__ __forceinline__ void noise_call(T* __restrict__ z, int C, int M, uint32_t seed, const uint32_t* __restrict__ job,
+                                           const int64_t* __restrict__ step, uint32_t tag, int64_t t)
 {
     const int K = (3 * M + 3) >> 2;                // Philox calls per chain and step
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)C * K) return;
     const int c = (int)(t / K), call = (int)(t - (int64_t)c * K);
     T g[4];
@@ -161,6 +295,35 @@ k_noise(T* __restrict__ z, int C, int M, uint32_t seed, const uint32_t* __restri
         const int k = 4 * call + e, n = k / 3;
         if (n < M) zc[(size_t)(k - 3 * n) * M + n] = g[e];
     }
+}
+
+// The two as kernels of their own (the tensor-core transforms, whose inverse leaves
+// the CUDA cores to the noise), and in one launch, the first nf blocks the force, the
+// others the noise (the CUDA-core transforms, beside which noise on a second stream
+// gains nothing: a step of 50 x 20 beads takes 20.9 us with the second stream's two
+// event waits and 16.7 here, one of 1024 x 256 beads 59.3 and 57.0).
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256)
+k_force(const T* __restrict__ ub, T* __restrict__ vb, int C, int M, T c12nu)
+{
+    force_quad<T, VEC>(ub, vb, C, M, c12nu, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_noise(T* __restrict__ z, int C, int M, uint32_t seed, const uint32_t* __restrict__ job,
+        const int64_t* __restrict__ step, uint32_t tag)
+{
+    noise_call<T>(z, C, M, seed, job, step, tag, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256)
+k_force_noise(const T* __restrict__ ub, T* __restrict__ vb, int C, int M, T c12nu, unsigned nf, T* __restrict__ z,
+              uint32_t seed, const uint32_t* __restrict__ job, const int64_t* __restrict__ step, uint32_t tag)
+{
+    if (blockIdx.x < nf) force_quad<T, VEC>(ub, vb, C, M, c12nu, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    else noise_call<T>(z, C, M, seed, job, step, tag, (int64_t)(blockIdx.x - nf) * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
