@@ -999,13 +999,43 @@ void scatter_group(const sfp_batch* b, const Group& g, const std::vector<E>& in,
         std::memcpy(packed + b->off[g.chains[i]], in.data() + i * blk, blk * sizeof(E));
 }
 
+// FP64 beads -> modes (DIR 0, Eq. c1) or modes -> beads (DIR 1) of a group, in halves
+// when the number of beads is even.
+template <int DIR>
+int phi_transform(sfp_batch* b, Group& g, const double* in, double* out)
+{
+    const double* tab = DIR == 0 ? g.phiT_d : g.phi_d;
+    if (g.M % 2) return launch_gemm<double>(b, in, tab, out, 3 * g.C, g.M, g.M);
+    const dim3 grid(nblk(g.M / 2, 32), nblk(3 * g.C, 64));
+    sfp::k_sym_gemm<DIR><<<grid, 256, 0, b->cur>>>(in, tab, out, 3 * g.C, g.M);
+    CUDA_TRY(cudaGetLastError());
+    b->launches++;
+    return SFP_OK;
+}
+
+// Equilibrium starts of a group into g.stage2 (positions; tabs: l0 | Ld | Lo).  Chains
+// per block: as many as give every SM one block, at most 32 (a warp takes their serial
+// parts), within the shared memory.
+cudaError_t launch_equilibrium(sfp_batch* b, Group& g, const double* tabs)
+{
+    const int N = g.M - 1;
+    const size_t per_chain = (size_t)sfp::eq_pitch(g.M) * sizeof(double);
+    const int per = (int)std::max<size_t>(1, std::min<size_t>({32, (size_t)(g.C + 151) / 152, (227 * 1024) / per_chain}));
+    const size_t smem = per * per_chain;
+    const cudaError_t e = cudaFuncSetAttribute(sfp::k_equilibrium, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    sfp::k_equilibrium<<<nblk(g.C, per), 256, smem, b->stream>>>(g.stage2, tabs, tabs + N, tabs + 2 * N, g.C, g.M, per,
+                                                                b->dv.Tstar, b->dv.nu, b->seed, g.job);
+    return cudaGetLastError();
+}
+
 // CoM-relative bead positions (FP64, scaled) of a group into g.stage2
 int positions_dev(sfp_batch* b, Group& g)
 {
     const int64_t n = (int64_t)g.C * 3 * g.M;
     int rc = to_double(b, g.R, g.stage, n);
     if (rc) return rc;
-    return launch_gemm<double>(b, g.stage, g.phi_d, g.stage2, 3 * g.C, g.M, g.M);
+    return phi_transform<1>(b, g, g.stage, g.stage2);
 }
 
 int destroy_impl(sfp_batch* b)
@@ -1439,7 +1469,7 @@ int sfp_set_positions(sfp_batch* b, const double* host, size_t n_doubles)
         gather_group(b, g, host, tmp);
         for (auto& x : tmp) x *= inv_d;
         CUDA_TRY(cudaMemcpyAsync(g.stage2, tmp.data(), tmp.size() * 8, cudaMemcpyHostToDevice, b->stream));
-        int rc = launch_gemm<double>(b, g.stage2, g.phiT_d, g.stage, 3 * g.C, g.M, g.M);
+        int rc = phi_transform<0>(b, g, g.stage2, g.stage);
         if (rc) return rc;
         if ((rc = load_modes_dev(b, g, g.stage))) return rc;
         CUDA_TRY(cudaStreamSynchronize(b->stream));
@@ -1459,27 +1489,17 @@ int sfp_init_equilibrium(sfp_batch* b, int64_t burn_in_steps)
         all.insert(all.end(), l0.begin(), l0.end());
         all.insert(all.end(), Ld.begin(), Ld.end());
         all.insert(all.end(), Lo.begin(), Lo.end());
-        const int N = g.M - 1;
-        // l0 | Ld | Lo live in the head of stage2's tail-free region: use yz scratch
         double* tabs = nullptr;
-        double* xs = nullptr;
         CUDA_TRY(cudaMalloc(&tabs, all.size() * 8));
-        cudaError_t e = cudaMalloc(&xs, (size_t)g.C * g.M * 8);
-        if (e != cudaSuccess) { cudaFree(tabs); return fail(SFP_ENOMEM, "init scratch: %s", cudaGetErrorString(e)); }
-        e = cudaMemcpyAsync(tabs, all.data(), all.size() * 8, cudaMemcpyHostToDevice, b->stream);
-        if (e == cudaSuccess) {
-            sfp::k_equilibrium<<<nblk(g.C, 64), 64, 0, b->stream>>>(g.stage2, xs, tabs, tabs + N, tabs + 2 * N,
-                                                                   g.C, g.M, b->dv.Tstar, b->dv.nu, b->seed, g.job);
-            e = cudaGetLastError();
-        }
+        cudaError_t e = cudaMemcpyAsync(tabs, all.data(), all.size() * 8, cudaMemcpyHostToDevice, b->stream);
+        if (e == cudaSuccess) e = launch_equilibrium(b, g, tabs);
         int rc = SFP_OK;
-        if (e == cudaSuccess) rc = launch_gemm<double>(b, g.stage2, g.phiT_d, g.stage, 3 * g.C, g.M, g.M);
+        if (e == cudaSuccess) rc = phi_transform<0>(b, g, g.stage2, g.stage);
         if (e == cudaSuccess && !rc) rc = load_modes_dev(b, g, g.stage);
         if (e == cudaSuccess && !rc) e = cudaMemsetAsync(g.com, 0, (size_t)g.C * 3 * 8, b->stream);
         if (e == cudaSuccess && !rc) e = cudaMemsetAsync(g.step, 0, (size_t)g.C * 8, b->stream);
         if (e == cudaSuccess && !rc) e = cudaStreamSynchronize(b->stream);
         cudaFree(tabs);
-        cudaFree(xs);
         if (rc) return rc;
         if (e != cudaSuccess) return fail(SFP_ECUDA, "init_equilibrium: %s", cudaGetErrorString(e));
     }
@@ -2153,7 +2173,7 @@ int sfp::internal_slots_start(sfp_batch* b, const int32_t* slots, const uint32_t
     CUDA_TRY(cudaMemcpyAsync(g.slot_stop, stops, (size_t)n * 8, cudaMemcpyHostToDevice, b->stream));
     CUDA_TRY(cudaMemcpyAsync(g.slot_shear, sh.data(), (size_t)n * 8, cudaMemcpyHostToDevice, b->stream));
     const int N = g.M - 1;
-    const size_t smem = (size_t)4 * g.M * 8;
+    const size_t smem = (size_t)sfp::eq_pitch(g.M) * 8;
     if (b->precision == SFP_FP64) {
         if (smem > 48 * 1024)
             CUDA_TRY(cudaFuncSetAttribute(sfp::k_init_slots<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

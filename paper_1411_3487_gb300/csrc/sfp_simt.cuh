@@ -70,6 +70,87 @@ k_gemm_nt(const T* __restrict__ In, const T* __restrict__ B, T* __restrict__ Out
 }
 
 // ---------------------------------------------------------------------------
+// The FP64 transforms between beads and modes of chains with an even number of beads,
+// in halves: phi_{n,p} is even (p even) or odd (p odd) under n -> M - 1 - n, so
+//   DIR 0 (B = phi^T [p][n]):  R_p = sum_{n < M/2} phi_{n,p} (r_n +- r_{M-1-n})
+//   DIR 1 (B = phi [n][p]):    r_n, r_{M-1-n} = E_n +- O_n, E and O the sums over the
+//                              even and the odd modes, n < M/2
+// take half the products of k_gemm_nt, which GB300's FP64 units bound: 4096 x 256
+// beads 1557 us there, 804 us here.  Block tile 64 rows x 32 outputs of each parity.
+// ---------------------------------------------------------------------------
+template <int DIR>
+__global__ void __launch_bounds__(256)
+k_sym_gemm(const double* __restrict__ In, const double* __restrict__ B, double* __restrict__ Out, int J, int M)
+{
+    constexpr int BM = 64, BN = 32, BK = 8;
+    __shared__ double As[2][BK][BM + 1];            // [parity]
+    __shared__ double Bs[2][BK][BN + 1];
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, H = M / 2;
+    const int j0 = blockIdx.y * BM, i0 = blockIdx.x * BN;
+    double acc[2][4][2] = {};
+    for (int k0 = 0; k0 < H; k0 += BK) {
+        for (int e = tid; e < BM * BK; e += 256) {
+            const int row = e / BK, kk = e % BK, j = j0 + row, k = k0 + kk;
+            double x = 0.0, y = 0.0;
+            if (j < J && k < H) {
+                const double* p = In + (size_t)j * M;
+                if constexpr (DIR == 0) {
+                    const double u = p[k], v = p[M - 1 - k];
+                    x = u + v;
+                    y = u - v;
+                } else {
+                    x = p[2 * k];
+                    y = p[2 * k + 1];
+                }
+            }
+            As[0][kk][row] = x;
+            As[1][kk][row] = y;
+        }
+        for (int e = tid; e < 2 * BN * BK; e += 256) {
+            const int par = e / (BN * BK), col = (e / BK) % BN, kk = e % BK, i = i0 + col, k = k0 + kk;
+            double x = 0.0;
+            if (i < H && k < H) x = DIR == 0 ? B[(size_t)(2 * i + par) * M + k] : B[(size_t)i * M + 2 * k + par];
+            Bs[par][kk][col] = x;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < BK; ++kk)
+#pragma unroll
+            for (int par = 0; par < 2; ++par) {
+                double a[4], b[2];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) a[x] = As[par][kk][ty + 16 * x];
+#pragma unroll
+                for (int y = 0; y < 2; ++y) b[y] = Bs[par][kk][tx + 16 * y];
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) acc[par][x][y] = fma(a[x], b[y], acc[par][x][y]);
+            }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const int j = j0 + ty + 16 * x;
+        if (j >= J) continue;
+        double* o = Out + (size_t)j * M;
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const int i = i0 + tx + 16 * y;
+            if (i >= H) continue;
+            const double e = acc[0][x][y], d = acc[1][x][y];
+            if constexpr (DIR == 0) {
+                o[2 * i] = e;
+                o[2 * i + 1] = d;
+            } else {
+                o[i] = e + d;
+                o[M - 1 - i] = e - d;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // The same product in FP32 (the plain path, and every length that the tensor-core
 // kernels do not take): Out_z[j][i] = sum_k In_z[j][k] B_z[i][k], blockIdx.z picks the
 // product (the forward transform's two are one launch).  Block tile BM x BN, K chunks
@@ -746,93 +827,128 @@ __global__ void k_advance_steps(int64_t* __restrict__ step, const int64_t* __res
 }
 
 // ---------------------------------------------------------------------------
-// Equilibrium start, one thread per chain, FP64 (Philox counter (0,0,k,1)):
+// Equilibrium start, FP64 (Philox counter (0,0,k,1)):
 //   l = l0 + sqrt(T*) L^-T eps   with (I - nu A) = L L^T  (Ld diag, Lo sub-diag)
 //   t_1 uniform on the sphere, t_n ~ von Mises-Fisher(t_{n-1}, nu l_{n-1} l_n / T*)
-//   r_n = sum_{k<=n} l_k t_k, centroid removed.   out: pos[c][3][M], scratch x[c][M]
+//   r_n = sum_{k<=n} l_k t_k, centroid removed.
+// A block samples n_ch chains in shared memory, eq_pitch(M) doubles per chain: bond
+// lengths [M], then turns and later positions [M][3]; the centroid ends in the first
+// three lengths' place.  Only what is a chain of dependences stays serial, one thread
+// per chain: the back substitution and the frame that each bond passes on to the next;
+// Philox, logarithms, exponentials and sines run a bead per thread.  Bound by FP64
+// issue (about 450 FP64 instructions per bead at 4 GFMA/s per SM).  One thread per
+// chain for everything, in strided global memory, took 2367 us for 4096 x 256 beads;
+// 845 us here.
 // ---------------------------------------------------------------------------
-// One chain's equilibrium start (positions p[3][M], scratch x[M]); p and x may
-// be global or shared memory.
-__device__ void sample_start(double* __restrict__ p, double* __restrict__ x,
-                             const double* __restrict__ l0, const double* __restrict__ Ld,
-                             const double* __restrict__ Lo, int M, double Tstar, double nu,
-                             uint32_t seed, uint32_t job)
+__host__ __device__ constexpr int eq_pitch(int M) { return 4 * M + 1; }   // odd: chains apart in the banks
+
+__device__ __forceinline__ void sample_starts(double* eq_smem, const double* __restrict__ l0, const double* __restrict__ Ld,
+                                              const double* __restrict__ Lo, int n_ch, int M, double Tstar, double nu,
+                                              uint32_t seed, const uint32_t* __restrict__ job)
 {
-    const int N = M - 1;
-    const uint2 key = make_uint2(seed, job);
-    // back substitution L^T x = eps, eps_i is the normal of bond i+1
-    for (int i = N - 1; i >= 0; --i) {
-        const uint4 wd = philox4x32_10(make_uint4(0u, 0u, (uint32_t)(i + 1), 1u), key);
+    const int N = M - 1, pitch = eq_pitch(M);
+    const double sT = sqrt(Tstar);
+    // eps_i, the normal of bond i + 1
+    for (int t = threadIdx.x; t < n_ch * N; t += blockDim.x) {
+        const int c = t / N, i = t - c * N;
+        const uint4 wd = philox4x32_10(make_uint4(0u, 0u, (uint32_t)(i + 1), 1u), make_uint2(seed, job[c]));
         double s, co;
         sincospi(2.0 * u01d(wd.y), &s, &co);
-        const double eps = sqrt(-2.0 * log(u01d(wd.x))) * co;
-        const double nxt = (i + 1 < N) ? Lo[i + 1] * x[i + 1] : 0.0;
-        x[i] = (eps - nxt) / Ld[i];
+        eq_smem[c * pitch + i] = sqrt(-2.0 * log(u01d(wd.x))) * co;
     }
-    double t[3];
-    {
-        const uint4 wd = philox4x32_10(make_uint4(0u, 0u, 0u, 1u), key);
-        const double ct = 2.0 * u01d(wd.x) - 1.0;
-        const double st = sqrt((1.0 - ct) * (1.0 + ct));
-        double sp, cp;
-        sincospi(2.0 * u01d(wd.y), &sp, &cp);
-        t[0] = st * cp; t[1] = st * sp; t[2] = ct;
+    __syncthreads();
+    // back substitution L^T x = eps, then the bond lengths l = l0 + sqrt(T*) x
+    if (threadIdx.x < n_ch) {
+        double* x = eq_smem + threadIdx.x * pitch;
+        double nxt = 0.0;
+        for (int i = N - 1; i >= 0; --i) {
+            const double v = (x[i] - nxt) / Ld[i];
+            x[i] = l0[i] + sT * v;
+            nxt = Lo[i] * v;
+        }
     }
-    const double sT = sqrt(Tstar);
-    double acc[3] = {0.0, 0.0, 0.0}, sum[3] = {0.0, 0.0, 0.0};
-    p[0] = p[M] = p[2 * M] = 0.0;
-    double lprev = 0.0;
-    for (int n = 1; n <= N; ++n) {
-        const double ln = l0[n - 1] + sT * x[n - 1];
-        if (n >= 2 && Tstar > 0.0) {
-            const uint4 wd = philox4x32_10(make_uint4(0u, 0u, (uint32_t)n, 1u), key);
-            const double kap = nu * lprev * ln / Tstar;
+    __syncthreads();
+    // turn of bond n against bond n - 1 (von Mises-Fisher): cosine, and sine times the
+    // cosine and sine of the angle about bond n - 1
+    for (int t = threadIdx.x; t < n_ch * (N - 1); t += blockDim.x) {
+        const int c = t / (N - 1), n = 2 + t - c * (N - 1);
+        const double* l = eq_smem + c * pitch;
+        double* a = eq_smem + c * pitch + M + 3 * n;
+        double ct = 1.0, ca = 0.0, sa = 0.0;
+        if (Tstar > 0.0) {
+            const uint4 wd = philox4x32_10(make_uint4(0u, 0u, (uint32_t)n, 1u), make_uint2(seed, job[c]));
+            const double kap = nu * l[n - 2] * l[n - 1] / Tstar;
             const double U = u01d(wd.z);
-            const double ct = 1.0 + log(U + (1.0 - U) * exp(-2.0 * kap)) / kap;
+            ct = 1.0 + log(U + (1.0 - U) * exp(-2.0 * kap)) / kap;
             const double st = sqrt(fmax(0.0, (1.0 - ct) * (1.0 + ct)));
             double sp, cp;
             sincospi(2.0 * u01d(wd.w), &sp, &cp);
-            // orthonormal pair perpendicular to t (Duff et al., JCGT 2017)
-            const double sg = copysign(1.0, t[2]);
-            const double a = -1.0 / (sg + t[2]);
-            const double bb = t[0] * t[1] * a;
-            const double e1[3] = {1.0 + sg * t[0] * t[0] * a, sg * bb, -sg * t[0]};
-            const double e2[3] = {bb, sg + t[1] * t[1] * a, -t[1]};
-            double tn[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) tn[k] = ct * t[k] + st * (cp * e1[k] + sp * e2[k]);
-            const double nn = sqrt(tn[0] * tn[0] + tn[1] * tn[1] + tn[2] * tn[2]);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] = tn[k] / nn;
+            ca = st * cp;
+            sa = st * sp;
         }
+        a[0] = ct; a[1] = ca; a[2] = sa;
+    }
+    __syncthreads();
+    // bond by bond along the chain; position n takes the place of turn n
+    if (threadIdx.x < n_ch) {
+        const double* l = eq_smem + threadIdx.x * pitch;
+        double* a = eq_smem + threadIdx.x * pitch + M;
+        const uint4 wd = philox4x32_10(make_uint4(0u, 0u, 0u, 1u), make_uint2(seed, job[threadIdx.x]));
+        const double z0 = 2.0 * u01d(wd.x) - 1.0;
+        const double st = sqrt((1.0 - z0) * (1.0 + z0));
+        double sp, cp;
+        sincospi(2.0 * u01d(wd.y), &sp, &cp);
+        double t[3] = {st * cp, st * sp, z0}, acc[3] = {0.0, 0.0, 0.0}, sum[3] = {0.0, 0.0, 0.0};
+        a[0] = a[1] = a[2] = 0.0;
+        for (int n = 1; n <= N; ++n) {
+            if (n >= 2 && Tstar > 0.0) {
+                // orthonormal pair perpendicular to t (Duff et al., JCGT 2017)
+                const double ct = a[3 * n], ca = a[3 * n + 1], sa = a[3 * n + 2];
+                const double sg = copysign(1.0, t[2]);
+                const double q = -1.0 / (sg + t[2]);
+                const double bb = t[0] * t[1] * q;
+                const double tn[3] = {ct * t[0] + ca * (1.0 + sg * t[0] * t[0] * q) + sa * bb,
+                                      ct * t[1] + ca * (sg * bb) + sa * (sg + t[1] * t[1] * q),
+                                      ct * t[2] - ca * (sg * t[0]) - sa * t[1]};
+                const double inv = rsqrt(tn[0] * tn[0] + tn[1] * tn[1] + tn[2] * tn[2]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            acc[k] += ln * t[k];
-            p[k * M + n] = acc[k];
-            sum[k] += acc[k];
+                for (int k = 0; k < 3; ++k) t[k] = tn[k] * inv;
+            }
+            const double ln = l[n - 1];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                acc[k] += ln * t[k];
+                a[3 * n + k] = acc[k];
+                sum[k] += acc[k];
+            }
         }
-        lprev = ln;
-    }
+        // the centroid in the place of the first bond lengths (N >= 2), read below
+        double* m = eq_smem + threadIdx.x * pitch;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const double m = sum[k] / M;
-        for (int n = 0; n < M; ++n) p[k * M + n] -= m;
+        for (int k = 0; k < 3; ++k) m[k] = sum[k] / M;
     }
+    __syncthreads();
 }
 
-__global__ void k_equilibrium(double* __restrict__ pos, double* __restrict__ xs,
-                              const double* __restrict__ l0, const double* __restrict__ Ld,
-                              const double* __restrict__ Lo, int C, int M, double Tstar,
-                              double nu, uint32_t seed, const uint32_t* __restrict__ job)
+// Starts of a batch, `per` chains per block.   out: pos[c][3][M]
+__global__ void __launch_bounds__(256)
+k_equilibrium(double* __restrict__ pos, const double* __restrict__ l0, const double* __restrict__ Ld,
+              const double* __restrict__ Lo, int C, int M, int per, double Tstar, double nu, uint32_t seed,
+              const uint32_t* __restrict__ job)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    sample_start(pos + (size_t)c * 3 * M, xs + (size_t)c * M, l0, Ld, Lo, M, Tstar, nu, seed, job[c]);
+    extern __shared__ double eq_smem[];
+    const int c0 = blockIdx.x * per, n_ch = min(per, C - c0);
+    sample_starts(eq_smem, l0, Ld, Lo, n_ch, M, Tstar, nu, seed, job + c0);
+    for (int t = threadIdx.x; t < n_ch * 3 * M; t += blockDim.x) {
+        const int c = t / (3 * M), e = t - c * 3 * M, k = e / M, n = e - k * M;
+        const double* q = eq_smem + c * eq_pitch(M);
+        pos[(size_t)(c0 + c) * 3 * M + e] = q[M + 3 * n + k] - q[k];
+    }
 }
 
 // Serving: start n chains in the slots slot[i] with job key jobv[i], stop step
-// stopv[i] and shear rate shv[i] (1/tau).  One block per slot: thread 0 draws the
-// equilibrium start into shared memory (3M + M doubles), then the block projects it
+// stopv[i] and shear rate shv[i] (1/tau).  One block per slot: it draws the
+// equilibrium start in shared memory (eq_pitch(M) doubles) and projects it
 // onto the modes R_p = sum_n phi_{n,p} r_n (Eq. c1, p >= 1; phi FP64 [n][p]); the
 // centre of mass is at the origin and the step counter 0.
 template <typename T>
@@ -845,11 +961,9 @@ __global__ void k_init_slots(T* __restrict__ R, double* __restrict__ com, int64_
                              int M, double Tstar, double nu, uint32_t seed)
 {
     extern __shared__ double sh_pos[];
-    double* xs = sh_pos + 3 * M;
     const int i = blockIdx.x;
     const int c = slot[i];
-    if (threadIdx.x == 0) sample_start(sh_pos, xs, l0, Ld, Lo, M, Tstar, nu, seed, jobv[i]);
-    __syncthreads();
+    sample_starts(sh_pos, l0, Ld, Lo, 1, M, Tstar, nu, seed, jobv + i);
     T* Rc = R + (size_t)c * 3 * M;
     for (int p = threadIdx.x; p < M; p += blockDim.x) {
         double s[3] = {0.0, 0.0, 0.0};
@@ -857,7 +971,7 @@ __global__ void k_init_slots(T* __restrict__ R, double* __restrict__ com, int64_
             for (int n = 0; n < M; ++n) {
                 const double f = phi[(size_t)n * M + p];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) s[a] += f * sh_pos[a * M + n];
+                for (int a = 0; a < 3; ++a) s[a] += f * (sh_pos[M + 3 * n + a] - sh_pos[a]);
             }
 #pragma unroll
         for (int a = 0; a < 3; ++a) Rc[(size_t)a * M + p] = (T)s[a];
