@@ -609,9 +609,9 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
     int rc;
     if ((rc = mark(b, 0))) return rc;
     const size_t smem = (size_t)9 * g.M * sizeof(double);
+    const auto chain_steps = g.M % 2 ? sfp::k_chain_steps<double, false> : sfp::k_chain_steps<double, true>;
     if (smem > 48 * 1024)
-        CUDA_TRY(cudaFuncSetAttribute(sfp::k_chain_steps<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+        CUDA_TRY(cudaFuncSetAttribute(chain_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const double c12 = 1.0 - 2.0 * b->dv.nu, w0cm = g.tab.w0 / std::sqrt((double)g.M);
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
@@ -647,7 +647,7 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
         }
     } else {
         const int threads = std::min(256, (g.M + 31) / 32 * 32);
-        sfp::k_chain_steps<double><<<g.C, threads, smem, b->cur>>>(
+        chain_steps<<<g.C, threads, smem, b->cur>>>(
             (double*)g.R, g.com, g.step, g.limited ? g.stop : nullptr, g.job, g.shear, (const double*)g.chiT,
             (const double*)g.chi, g.phi_d, (const double*)g.dm, (const double*)g.h, (const double*)g.w,
             (const double*)g.g, g.C, g.M, c12, w0cm, g.dtau, b->seed, (int)n_steps,
