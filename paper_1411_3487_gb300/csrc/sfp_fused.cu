@@ -2,10 +2,9 @@
 // the SFP_FP32 and SFP_MIXED_BF16 paths, M = 64, 128, 256 or 512 beads,
 // n_steps per launch.
 //
-// SFP_MIXED_BF16 chains of 64, 128 and 256 beads with bead noise take the lane
-// step (sfp_lanes.cuh: bonds and modes on the TMEM lanes), launched from here;
-// the kernels below serve the TF32 and two-pass splits, mode-keyed noise, and
-// 512 beads.
+// SFP_MIXED_BF16 chains with bead noise take the lane step (sfp_lanes.cuh: bonds
+// and modes on the TMEM lanes), launched from here; the kernels below serve the
+// TF32 and two-pass splits and mode-keyed noise.
 //
 // The 128 TMEM lanes hold a tile's chain-axis rows: lane quarter q (rows
 // 32 q .. 32 q + 31) holds chains q cpq .. q cpq + cpq - 1 of the tile
@@ -958,17 +957,23 @@ k_fused_step(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CU
     tmem_free<2 * NB>(tmem);
 }
 
-// One tile per CTA, bonds and modes on the TMEM lanes (sfp_lanes.cuh).
+// One tile per CTA (512 beads: per cluster of two), bonds and modes on the TMEM lanes
+// (sfp_lanes.cuh).
 template <int M>
 __global__ void __launch_bounds__(lanes::kThreads, 1)
 k_lane_step(const FusedArgs a, const lanes::LaneArgs la)
 {
+    if (lanes::Geo<M>::kPair && cluster_size() != 2u) {
+        // every access to the other CTA assumes a cluster of two
+        if (threadIdx.x == 0) atomicOr(a.err, 4);
+        return;
+    }
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t s_tmem;
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
     tmem_alloc<lanes::Geo<M>::kCols>(&s_tmem);
     const uint32_t tmem = s_tmem;
-    lanes::lane_tile<M>(a, la, blockIdx.x, smem, tmem);
+    lanes::lane_tile<M>(a, la, lanes::Geo<M>::kPair ? blockIdx.x >> 1 : blockIdx.x, smem, tmem);
     tmem_free<lanes::Geo<M>::kCols>(tmem);
 }
 
@@ -1611,7 +1616,8 @@ __device__ __noinline__ bool grouped_tile(const GroupSlot& g, int tile, uint8_t*
 template <bool BF, bool TWO>
 __device__ __noinline__ bool grouped_pair(const GroupSlot& g, int tile, uint8_t* smem_raw, uint32_t tmem)
 {
-    return pair_tile<BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, align_up(smem_raw, 1024), tmem);
+    if constexpr (BF && !TWO) return lanes::lane_tile<512>(g.a, g.la, tile, align_up(smem_raw, 128), tmem);
+    else return pair_tile<BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, align_up(smem_raw, 1024), tmem);
 }
 
 template <bool BF, bool TWO>
@@ -1654,15 +1660,23 @@ struct FusedPlan {
     float* w32 = nullptr;       // w_p with w_0 (FP32), for the mode-keyed epilogue
     float* zbuf = nullptr;      // mode-keyed noise of two steps [2][C][3][M]
     bool mz = false;            // mode-keyed noise on
-    uint8_t* lane_tab = nullptr;   // lane step (BF16, three passes, 64 .. 256 beads): table blocks
+    uint8_t* lane_tab = nullptr;   // lane step (BF16, three passes): table blocks
     float4* lane_c = nullptr;      // ... and per-mode constants
+    size_t lane_bytes = 0;
+    bool classic = false;          // tables of the other kernels exist
+    // what the tables of the other kernels are made of, until mode-keyed noise needs them
+    std::vector<double> chi, phi, h, w;
+    cudaStream_t stream = nullptr;
     CUtensorMap tmR, tmChiH, tmChiL, tmFH, tmFL;
 };
 
 // Chains per tile: a multiple of 4 (one share per TMEM lane quarter), 4..most.
 static int round_tile(int cpt, int most) { return std::min(most, std::max(4, (cpt + 3) / 4 * 4)); }
 // Most chains per tile of a plan's step.
-static int most_chains(const FusedPlan* p) { return p->lane_tab ? lanes::kMaxChains : kChains; }
+static int most_chains(const FusedPlan* p)
+{
+    return !p->lane_tab ? kChains : p->M == 512 ? lanes::Geo<512>::kMaxChains : lanes::Geo<256>::kMaxChains;
+}
 
 bool fused_supported(int M) { return M == 64 || M == 128 || M == 256 || M == 512; }
 
@@ -1670,8 +1684,7 @@ bool fused_supported(int M) { return M == 64 || M == 128 || M == 256 || M == 512
 static int grouped_smem(bool bf16, bool two)
 {
     if (bf16 && !two)
-        return std::max({FSmem<256, true, false>::kBytes, lanes::Geo<256>::kBytes, lanes::Geo<128>::kBytes,
-                         lanes::Geo<64>::kBytes});
+        return std::max({lanes::Geo<512>::kBytes, lanes::Geo<256>::kBytes, lanes::Geo<128>::kBytes, lanes::Geo<64>::kBytes});
     return bf16 ? std::max({FSmem<256, true, true>::kBytes, FSmem<128, true, true>::kBytes, FSmem<64, true, true>::kBytes,
                             FSmem<256, true, false>::kBytes})
                 : std::max({FSmem<256, false, false>::kBytes, FSmem<128, false, false>::kBytes,
@@ -1710,27 +1723,33 @@ static int lane_tables(FusedPlan* p, const double* chi, const double* phi, const
         }
         lc[q] = make_float4((float)dm[q], (float)g[q], (float)cs, (float)es[q]);
     }
-    auto table = [&](int t, int e, int row, int k) -> double {     // t: 0 inverse, 1 noise, 2 forward
+    // table t (0 inverse, 1 noise, 2 forward) of parity e: row and K index of the contraction
+    auto table = [&](int t, int e, int row, int k) -> double {
         const int r = M == 64 ? row & 63 : row;
         if (G::kScaled && t != 1) return std::sin(pi * (double)((r * k) % (2 * M)) / M);
-        const int mode = G::NP * (t == 0 ? k : r) + e, n = t == 0 ? r : k;
+        const int mode = (G::kFold ? 2 : 1) * (t == 0 ? k : r) + e, n = t == 0 ? r : k;
         if (t == 1) return w[mode] * phi[(size_t)n * M + mode];
         double c = chi[(size_t)n * M + mode];
         if (G::kFold && n == 0) c = e ? chi[(size_t)(M / 2) * M + mode] * (t == 2 ? 0.5 : 1.0) : 0.0;
         return t == 2 ? h[mode] * c : c;
     };
-    std::vector<uint16_t> img((size_t)G::BLK_TAB * lanes::kBlkBytes / 2);
-    for (int b = 0; b < G::BLK_TAB; ++b) {
-        const int t = b / G::BLK, k0 = 16 * ((b % G::BLK) / G::NP), e = (b % G::BLK) % G::NP;
+    // blocks of 16 K indices; for each, the parities' (a pair: one image per CTA, its
+    // parity's two row tiles)
+    constexpr int CTAS = G::kPair ? 2 : 1;
+    std::vector<uint16_t> img((size_t)CTAS * G::BLK_TAB * lanes::kBlkBytes / 2);
+    for (int b = 0; b < CTAS * G::BLK_TAB; ++b) {
+        const int c = b / G::BLK_TAB, bb = b % G::BLK_TAB, t = bb / G::BLK, k0 = 16 * ((bb % G::BLK) / G::NP);
+        const int s = (bb % G::BLK) % G::NP, e = G::kPair ? c : s, row0 = G::kPair ? 128 * s : 0;
         uint16_t* d = img.data() + (size_t)b * lanes::kBlkBytes / 2;
         for (int k = 0; k < 16; ++k)
             for (int row = 0; row < 128; ++row) {
-                const double x = table(t, e, row, k0 + k);
+                const double x = table(t, e, row0 + row, k0 + k);
                 const size_t o = (size_t)(k >> 3) * 1024 + (row >> 3) * 64 + (row & 7) * 8 + (k & 7);
                 d[o] = bf16_round_host((float)x);
                 d[lanes::kBlkBytes / 4 + o] = bf16_round_host((float)(x - (double)bf16_to_float_host(d[o])));
             }
     }
+    p->lane_bytes = img.size() * 2 + lc.size() * sizeof(float4);
     if (cudaMalloc((void**)&p->lane_tab, img.size() * 2) != cudaSuccess ||
         cudaMalloc((void**)&p->lane_c, lc.size() * sizeof(float4)) != cudaSuccess)
         return report(SFP_ENOMEM, "lane-step table allocation failed");
@@ -1748,37 +1767,13 @@ static cudaError_t set_smem_pair()
                                 FSmem<256, BF, false>::kBytes);
 }
 
-int fused_create(FusedPlan** out, int M, int C, const double* chi, const double* phi, const double* h,
-                 const double* w, const double* dm, const double* g, float* R, cudaStream_t stream, bool bf16, bool two)
+// Tables, maps and kernel attributes of k_fused_step, k_fused_pair and their grouped
+// launch (the caller frees the plan on failure).
+static int classic_tables(FusedPlan* p, const double* chi, const double* phi, const double* h, const double* w)
 {
-    *out = nullptr;
-    if (!fused_supported(M)) return report(SFP_ENOTSUP, "the fused step needs M in {64, 128, 256, 512}");
-    FusedPlan* p = new FusedPlan();
-    p->M = M;
-    p->C = C;
-    p->R = R;
-    p->bf16 = bf16;
-    p->two = bf16 && two;
-    // the fewest waves of tiles of at most 40 chains (a 512-bead tile takes two
-    // SMs), then the chains spread evenly over the tiles of those waves: chains
-    // per tile = ceil(C / (units x waves)) rounded up to a multiple of 4
-    // (fused_set_tile changes it)
-    if (bf16 && !two && M <= 256) {
-        const int rc = M == 256 ? lane_tables<256>(p, chi, phi, h, w, dm, g, stream)
-                     : M == 128 ? lane_tables<128>(p, chi, phi, h, w, dm, g, stream)
-                                : lane_tables<64>(p, chi, phi, h, w, dm, g, stream);
-        if (rc) {
-            fused_destroy(p);
-            return rc;
-        }
-    }
-    const int most = most_chains(p);
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        sms = 148;
-    const int units = M == 512 ? sms / 2 : sms;
-    const int waves = std::max(1, (C + units * most - 1) / (units * most));
-    p->cpt = round_tile((C + units * waves - 1) / (units * waves), most);
+    const int M = p->M;
+    const bool bf16 = p->bf16;
+    const cudaStream_t stream = p->stream;
     const size_t mm = (size_t)M * M;
     // chi [n][p] (row n = 0 and column p = 0 are zero) and F [2M][M]:
     // F[p][n] = h_p chi[n][p] (Eq. f2 weight on DeltaH = chi^T v, Eq. e11),
@@ -1808,24 +1803,16 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
             void*& d = p->tab[2 * t + k];
             const void* hsrc = bf16 ? (const void*)(k == 0 ? hb.data() : lb.data())
                                     : (const void*)(k == 0 ? hi.data() : lo.data());
-            if (cudaMalloc(&d, cnt[t] * el) != cudaSuccess) {
-                fused_destroy(p);
-                return report(SFP_ENOMEM, "fused-step table allocation failed");
-            }
+            if (cudaMalloc(&d, cnt[t] * el) != cudaSuccess) return report(SFP_ENOMEM, "fused-step table allocation failed");
             if (cudaMemcpyAsync(d, hsrc, cnt[t] * el, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
-                cudaStreamSynchronize(stream) != cudaSuccess) {
-                fused_destroy(p);
+                cudaStreamSynchronize(stream) != cudaSuccess)
                 return report(SFP_ECUDA, "fused-step table upload failed");
-            }
         }
     }
     int rc;
     // one box per lane quarter of the tile, 3 cpt / 4 rows: a tile never writes
     // the next tile's chains
-    if ((rc = make_map_2d(&p->tmR, R, 3 * C, M, 3 * (p->cpt / 4)))) {
-        fused_destroy(p);
-        return rc;
-    }
+    if ((rc = make_map_2d(&p->tmR, p->R, 3 * p->C, M, 3 * (p->cpt / 4)))) return rc;
     // B operand boxes: the rows of one CTA's TMEM half (all M, or 256 of 512)
     const int bx = std::min(M, 256);
     if (bf16)
@@ -1836,16 +1823,13 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
              make_map_2d(&p->tmChiL, (const float*)p->tab[1], M, M, bx) ? -1 :
              make_map_2d(&p->tmFH, (const float*)p->tab[2], 2 * M, M, bx) ? -1 :
              make_map_2d(&p->tmFL, (const float*)p->tab[3], 2 * M, M, bx);
-    if (rc) {
-        fused_destroy(p);
-        return SFP_ECUDA;
-    }
+    if (rc) return SFP_ECUDA;
     cudaError_t e;
     if (p->two)
         e = M == 512 ? set_smem_pair<true, true>() : M == 256 ? set_smem<256, true, true>() :
             M == 128 ? set_smem<128, true, true>() : set_smem<64, true, true>();
     else if (bf16)
-        e = M == 512 ? set_smem_pair<true>() : cudaSuccess;   // the lane step's own set-up: lane_tables
+        e = cudaSuccess;        // mode-keyed noise only, below
     else
         e = M == 512 ? set_smem_pair<false>() : M == 256 ? set_smem<256, false>() :
             M == 128 ? set_smem<128, false>() : set_smem<64, false>();
@@ -1862,13 +1846,64 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
         if (e == cudaSuccess) e = cudaMemcpyAsync(p->w32, wf.data(), (size_t)M * sizeof(float), cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     }
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(p->two ? k_fused_grouped<true, true> : bf16 ? k_fused_grouped<true, false>
-                                                                             : k_fused_grouped<false, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, grouped_smem(bf16, p->two));
-    if (e != cudaSuccess) {
+    if (e != cudaSuccess) return report(SFP_ECUDA, "cudaFuncSetAttribute (fused step) failed");
+    p->classic = true;
+    return SFP_OK;
+}
+
+int fused_create(FusedPlan** out, int M, int C, const double* chi, const double* phi, const double* h,
+                 const double* w, const double* dm, const double* g, float* R, cudaStream_t stream, bool bf16, bool two)
+{
+    *out = nullptr;
+    if (!fused_supported(M)) return report(SFP_ENOTSUP, "the fused step needs M in {64, 128, 256, 512}");
+    FusedPlan* p = new FusedPlan();
+    p->M = M;
+    p->C = C;
+    p->R = R;
+    p->bf16 = bf16;
+    p->two = bf16 && two;
+    p->stream = stream;
+    if (bf16 && !two) {
+        const int rc = M == 512 ? lane_tables<512>(p, chi, phi, h, w, dm, g, stream)
+                     : M == 256 ? lane_tables<256>(p, chi, phi, h, w, dm, g, stream)
+                     : M == 128 ? lane_tables<128>(p, chi, phi, h, w, dm, g, stream)
+                                : lane_tables<64>(p, chi, phi, h, w, dm, g, stream);
+        if (rc) {
+            fused_destroy(p);
+            return rc;
+        }
+    }
+    // the fewest waves of tiles of as many chains as the step takes (a 512-bead tile
+    // takes two SMs), then the chains spread evenly over the tiles of those waves:
+    // chains per tile = ceil(C / (units x waves)) rounded up to a multiple of 4
+    // (fused_set_tile changes it)
+    const int most = most_chains(p);
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 148;
+    const int units = M == 512 ? sms / 2 : sms;
+    const int waves = std::max(1, (C + units * most - 1) / (units * most));
+    p->cpt = round_tile((C + units * waves - 1) / (units * waves), most);
+    int rc = SFP_OK;
+    if (!p->lane_tab) {
+        rc = classic_tables(p, chi, phi, h, w);
+    } else if (M <= 256) {
+        // mode-keyed noise, if it is ever chosen, runs on the other kernels
+        const size_t mm = (size_t)M * M;
+        p->chi.assign(chi, chi + mm);
+        p->phi.assign(phi, phi + mm);
+        p->h.assign(h, h + M);
+        p->w.assign(w, w + M);
+    }
+    if (!rc)
+        rc = cudaFuncSetAttribute(p->two ? k_fused_grouped<true, true> : bf16 ? k_fused_grouped<true, false>
+                                                                              : k_fused_grouped<false, false>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, grouped_smem(bf16, p->two)) == cudaSuccess
+                 ? SFP_OK
+                 : report(SFP_ECUDA, "cudaFuncSetAttribute (fused step) failed");
+    if (rc) {
         fused_destroy(p);
-        return report(SFP_ECUDA, "cudaFuncSetAttribute (fused step) failed");
+        return rc;
     }
     *out = p;
     return SFP_OK;
@@ -1885,10 +1920,28 @@ int fused_step(FusedPlan* p, const FusedArgs& args, cudaStream_t stream)
     if (p->mz && (p->two || p->M > 256)) return report(SFP_ENOTSUP, "mode-keyed noise: M <= 256, three passes");
     if (p->lane_tab && !p->mz) {
         const lanes::LaneArgs la{p->lane_tab, p->lane_c};
-        if (p->M == 256) k_lane_step<256><<<grid, lanes::kThreads, lanes::Geo<256>::kBytes, stream>>>(a, la);
-        else if (p->M == 128) k_lane_step<128><<<grid, lanes::kThreads, lanes::Geo<128>::kBytes, stream>>>(a, la);
-        else k_lane_step<64><<<grid, lanes::kThreads, lanes::Geo<64>::kBytes, stream>>>(a, la);
-        const cudaError_t e = cudaGetLastError();
+        cudaError_t e;
+        if (p->M == 512) {
+            // two CTAs (a cluster) per tile
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(2u * grid.x);
+            cfg.blockDim = dim3(lanes::kThreads);
+            cfg.dynamicSmemBytes = lanes::Geo<512>::kBytes;
+            cfg.stream = stream;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = 2;
+            at[0].val.clusterDim.y = 1;
+            at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            e = cudaLaunchKernelEx(&cfg, k_lane_step<512>, a, la);
+        } else {
+            if (p->M == 256) k_lane_step<256><<<grid, lanes::kThreads, lanes::Geo<256>::kBytes, stream>>>(a, la);
+            else if (p->M == 128) k_lane_step<128><<<grid, lanes::kThreads, lanes::Geo<128>::kBytes, stream>>>(a, la);
+            else k_lane_step<64><<<grid, lanes::kThreads, lanes::Geo<64>::kBytes, stream>>>(a, la);
+            e = cudaGetLastError();
+        }
         return e == cudaSuccess ? SFP_OK : report(SFP_ECUDA, cudaGetErrorString(e));
     }
 #define SFP_FUSED_LAUNCH(NBV, BFV)                                                                   \
@@ -1920,8 +1973,6 @@ int fused_step(FusedPlan* p, const FusedArgs& args, cudaStream_t stream)
             cfg.numAttrs = 1;
             e = p->two ? cudaLaunchKernelEx(&cfg, k_fused_pair<true, true>, p->tmR, p->tmChiH, p->tmChiL, p->tmFH,
                                             p->tmFL, args)
-              : p->bf16 ? cudaLaunchKernelEx(&cfg, k_fused_pair<true>, p->tmR, p->tmChiH, p->tmChiL, p->tmFH,
-                                             p->tmFL, args)
                         : cudaLaunchKernelEx(&cfg, k_fused_pair<false>, p->tmR, p->tmChiH, p->tmChiL, p->tmFH,
                                              p->tmFL, args);
             break;
@@ -1989,11 +2040,8 @@ int fused_ctas_per_tile(const FusedPlan* p) { return p->M == 512 ? 2 : 1; }
 size_t fused_bytes(const FusedPlan* p)
 {
     if (!p) return 0;
-    return (size_t)6 * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float) +
-           (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0) +
-           (p->lane_tab ? (size_t)(p->M == 256 ? lanes::Geo<256>::BLK_TAB : p->M == 128 ? lanes::Geo<128>::BLK_TAB
-                                                                                     : lanes::Geo<64>::BLK_TAB) *
-                                  lanes::kBlkBytes + (size_t)p->M * sizeof(float4) : 0);
+    return (p->classic ? (size_t)6 * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float) : 0) +
+           (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0) + p->lane_bytes;
 }
 
 int fused_set_tile(FusedPlan* p, int cpt)
@@ -2014,6 +2062,10 @@ int fused_set_mode_noise(FusedPlan* p, bool on)
 {
     if (on && (!fused_mode_noise_supported(p->M) || p->two))
         return report(SFP_ENOTSUP, "mode-keyed noise on the fused step: 64, 128 or 256 beads, three passes");
+    if (on && !p->classic) {
+        const int rc = classic_tables(p, p->chi.data(), p->phi.data(), p->h.data(), p->w.data());
+        if (rc) return rc;
+    }
     if (on && !p->zbuf) {
         const size_t bytes = (size_t)2 * p->C * 3 * p->M * sizeof(float);
         if (cudaMalloc((void**)&p->zbuf, bytes) != cudaSuccess) return report(SFP_ENOMEM, "mode-noise buffer allocation failed");

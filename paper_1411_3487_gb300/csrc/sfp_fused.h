@@ -32,7 +32,7 @@ struct FusedArgs {
     const float* w;         // mode-keyed noise: w_p, w_0 of the centre of mass (set by fused_step)
 };
 
-// True when a group of M beads can take the fused step (M = 64, 128 or 256).
+// True when a group of M beads can take the fused step (M = 64, 128, 256 or 512).
 bool fused_supported(int M);
 
 // Tables of one group: chi [n][p] (row n = 0 and column p = 0 zero), phi [n][p],
@@ -45,10 +45,13 @@ bool fused_supported(int M);
 int fused_create(FusedPlan** out, int M, int C, const double* chi, const double* phi, const double* h,
                  const double* w, const double* dm, const double* g, float* R, cudaStream_t stream, bool bf16 = false,
                  bool two = false);
+// Three BF16 passes take the lane step (sfp_lanes.cuh) and hold its tables; those of
+// the other kernels are built when mode-keyed noise is first chosen.
 // args.n_steps steps of every chain of the group, in one launch.
 int fused_step(FusedPlan* plan, const FusedArgs& args, cudaStream_t stream);
 // Chains per tile of the plan, and a new value (1..40, rounded up to a multiple
-// of 4: one share per TMEM lane quarter; rebuilds the R map).
+// of 4 and limited to what the plan's step takes: 32 for the lane step, 24 at 512
+// beads; rebuilds the R map).
 int fused_tile(const FusedPlan* plan);
 // CTAs that run one tile: 2 at M = 512 (a cluster pair), else 1.
 int fused_ctas_per_tile(const FusedPlan* plan);

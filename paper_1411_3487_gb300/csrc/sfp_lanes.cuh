@@ -1,5 +1,6 @@
 // sfp_lanes.cuh -- the mode-space step (Sec. 4) of a tile of up to 32 chains of
-// 64, 128 or 256 beads on one CTA, BF16 hi/lo transforms, n_steps per launch.
+// 64, 128 or 256 beads on one CTA, or up to 24 of 512 beads on a cluster of two,
+// BF16 hi/lo transforms, n_steps per launch.
 //
 // The bonds and modes of a chain are the 128 TMEM lanes (the M dimension of the
 // MMA), the chains' axes its columns (N = 96: 32 chain slots of 3 axes):
@@ -39,9 +40,24 @@
 // per cycle, 168 warps' worth of Philox calls more than half of them; a chain of 5.3
 // us a step with one chain per tile (inverse and forward MMAs 3000 cycles each, force,
 // update and four hand-overs).  State and D live in 504 of the 512 TMEM columns.
+// 512 beads (a cluster of two CTAs): the parities of the mirror symmetry are 256 modes
+// each, two row tiles of 128, and CTA rank r takes parity r, so that its operand, its
+// share of the state and its table stream are what one CTA holds at 256 beads.  Bonds are
+// sums over both parities: after the inverse MMAs each CTA sends the other the parts of
+// D_u of that one's 128 bond lanes (32 KB a step each way), works out both parities' force
+// operand for its own lanes, keeps one and stores the other in its peer's operand X.  The
+// normals are drawn once: each CTA draws every second chunk and writes the sums to the
+// even modes' CTA and the differences to the other.  All of it goes by st.async, which
+// counts bytes on the reader's mbarrier, so that nobody waits for the stores (with plain
+// remote stores and remote arrivals: 197 us a step at 16384 chains instead of 175).  Half
+// of the noise chunks come after the forward MMAs, so that their way between the CTAs
+// passes behind those.  The step is bound by the table stream, 768 KB a CTA from L2, with
+// 64 KB under way in the ring: what both CTAs' operands and buffers leave.
+//
 // Measured (GB300, us a step in a 400-step call, the four-role kernel of sfp_fused.cu
 // before -> here): 4096 x 256 bp 22.7 -> 9.1, 8 x 256 bp 19.1 -> 5.3, 4096 x 128 bp
-// 10.3 -> 4.3, 50 x 128 bp 9.5 -> 2.7, 4096 x 64 bp 7.3 -> 2.3, 8 x 64 bp 5.9 -> 1.5.
+// 10.3 -> 4.3, 50 x 128 bp 9.5 -> 2.7, 4096 x 64 bp 7.3 -> 2.3, 8 x 64 bp 5.9 -> 1.5; 16384 x 512 bp 289 ->
+// 175 (here 1000 x 512 bp take 17.2, one chain 14.0).
 #pragma once
 #include <cstdint>
 #include <cuda_bf16.h>
@@ -55,47 +71,65 @@ namespace lanes {
 
 using namespace ptx;
 
-constexpr int kRowsN = 96;                      // MMA N: 32 chain slots x 3 axes
-constexpr int kMaxChains = 32;
+constexpr int kMaxSlots = 32;                   // chain slots of the shared-memory arrays
 constexpr int kWork = 8, kNoise = 8;            // force / update warps (2 .. 9), noise warps (10 .. 17)
 constexpr int kThreads = 32 * (4 + kWork + kNoise);
 constexpr int kBlkBytes = 8192;                 // a table block (one K step of 16): [hi, lo][2 k groups][16 row groups][8][8]
 constexpr int kALbo = 2048, kASbo = 128;        // table blocks: K-major core matrices
-constexpr int kXSbo = 2048;                     // operand X: rows-major (MN-major) core matrices, [12 row groups][16 k groups]
-constexpr int kXPart = 12 * kXSbo;              // one parity and part (hi or lo): 24 KB
-constexpr int kZLbo = 12 * 128 + 32;            // noise operand: K-major core matrices, k groups 32 bytes apart in the banks
-constexpr int kZPart = 4 * kZLbo;               // K = 32
 
 // Rows of N: four chains (batch b = chain / 4 of the tile) hold rows 24 (b / 2) +
 // 8 axis + 4 (b & 1) + chain % 4, so that a thread's four values of an axis are 8
 // contiguous bytes of operand X.
 template <int M>
 struct Geo {
-    static constexpr bool kFold = M == 256;
-    static constexpr int NP = kFold ? 2 : 1;            // parities
-    static constexpr int KP = M / NP;                   // K of one parity's contraction
-    static constexpr bool kStream = M == 256;           // tables through a ring, else resident
+    static constexpr bool kPair = M == 512;             // a tile on a cluster of two CTAs, a parity each
+    static constexpr bool kFold = M >= 256;             // mirror symmetry
+    static constexpr int NP = kFold ? 2 : 1;            // accumulators: the parities, or the two row tiles of this CTA's parity
+    static constexpr int KP = kFold ? M / 2 : M;        // K of a contraction
+    static constexpr int ROWS = kPair ? 80 : 96;        // MMA N at most: chain slots x 3 axes (72 of 80 used)
+    static constexpr int GROUPS = kPair ? 9 : 12;       // row groups of 8
+    static constexpr int kMaxChains = 8 * GROUPS / 3;
+    static constexpr bool kStream = M >= 256;           // tables through a ring, else resident
     static constexpr bool kScaled = M == 128;           // one symmetric table sin(pi n p / M) for both directions
-    static constexpr int NCH = KP / 32;                 // noise chunks (K = 32 per parity) of a step
+    static constexpr int ZK = kPair ? 64 : 32;          // K of a noise chunk
+    static constexpr int NCH = KP / ZK;                 // noise chunks of a step
     static constexpr int BLK = NP * KP / 16;            // table blocks of one contraction
     static constexpr int BLK_STEP = 3 * BLK;            // ... of a step (streamed)
-    static constexpr int BLK_TAB = kScaled ? 2 * BLK : 3 * BLK;   // ... in the table image
+    static constexpr int BLK_TAB = kScaled ? 2 * BLK : 3 * BLK;   // ... in the table image (of one CTA of a pair)
     // blocks in shared memory: all, or a ring; a ring slot always serves the same
-    // parity, whose MMA warp so sees every phase of its barrier
-    static constexpr int ST = kStream ? 10 : BLK_TAB;
-    static_assert(!kStream || ST % NP == 0, "ring slots per parity");
-    static constexpr int XB = NP * 2 * kXPart;
-    static constexpr int ZB = NP * 2 * kZPart;          // one buffer of the noise operand
+    // accumulator, whose MMA warp so sees every phase of its barrier
+    static constexpr int ST = kPair ? 8 : kStream ? 10 : BLK_TAB;
+    static_assert(!kStream || ST % NP == 0, "ring slots per accumulator");
+    static constexpr int PAR = kPair ? 1 : NP;          // parities whose operands this CTA holds
+    // operand X: rows-major (MN-major) core matrices, [GROUPS][KP / 8]
+    static constexpr int XSBO = KP * 16, XPART = GROUPS * XSBO, XB = PAR * 2 * XPART;
+    // a buffer of the noise operand: K-major core matrices, k groups 32 bytes apart in the banks
+    static constexpr int ZLBO = ROWS / 8 * 128 + 32, ZPART = ZK / 8 * ZLBO, ZB = PAR * 2 * ZPART;
+    static constexpr int UB = kPair ? 2 * GROUPS * 2048 : 0;   // bond vectors from the other CTA, [batch][axis][128 lanes][4 chains]
     static constexpr int kMisc = 1664;
-    static constexpr int kBytes = ST * kBlkBytes + XB + 2 * ZB + kMisc + 128;
-    // TMEM columns: D_u and D_inc, 96 each per parity; with the symmetric table, whose
-    // increment h_p c_p scales after the contraction, the noise in a third accumulator;
+    static constexpr int kBytes = ST * kBlkBytes + XB + 2 * ZB + UB + kMisc + 128;
+    // TMEM columns: D_u and D_inc, ROWS each per accumulator; with the symmetric table,
+    // whose increment h_p c_p scales after the contraction, the noise in a third one;
     // then the state R of the first TB batches
     static constexpr uint32_t kCols = 512;
-    static constexpr int kRCol = (2 * NP + (kScaled ? 1 : 0)) * kRowsN;
+    static constexpr int kRCol = (2 * NP + (kScaled ? 1 : 0)) * ROWS;
     static constexpr int TB = (512 - kRCol) / (12 * NP) < 8 ? (512 - kRCol) / (12 * NP) : 8;
     static_assert(kBytes <= 227 * 1024, "shared memory of one CTA");
+    static_assert(!kPair || 4 * TB >= kMaxChains, "a pair's whole state in TMEM");
 };
+
+// Stores to the other CTA's shared memory that count as transaction bytes of its
+// mbarrier `bar` (cluster addresses): the writer neither waits for them nor arrives.
+__device__ __forceinline__ void st_peer16(uint32_t addr, const float (&v)[4], uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1,%2,%3,%4}, [%5];"
+                 ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_peer8(uint32_t addr, uint2 v, uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1,%2}, [%3];"
+                 ::"r"(addr), "r"(v.x), "r"(v.y), "r"(bar) : "memory");
+}
 
 // One lane of the (converged) warp.
 __device__ __forceinline__ bool elect_one()
@@ -182,29 +216,34 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
     uint8_t* tabs = smem;
     uint8_t* X = smem + G::ST * kBlkBytes;
     uint8_t* Z = X + G::XB;
-    uint8_t* misc = Z + 2 * G::ZB;
+    uint8_t* U = Z + 2 * G::ZB;
+    uint8_t* misc = U + G::UB;
     int64_t* s_step = (int64_t*)misc;               // [32]
     double* s_shear = (double*)(misc + 256);        // [32]
     uint32_t* s_job = (uint32_t*)(misc + 512);      // [32]
     int* s_left = (int*)(misc + 640);               // [32] steps this chain still takes in this launch
     float* s_d0 = (float*)(misc + 768);             // [3][32] noise increments of the centre of mass
     uint64_t* bars = (uint64_t*)(misc + 1152);
-    float* s_shf = (float*)(misc + 1408);           // [32]
+    float* s_shf = (float*)(misc + 1456);           // [32]
     uint64_t* full = bars;              // ring slot: table block landed (1 + tx)
-    uint64_t* empty = bars + 10;        // ... MMAs done with it (commit)
-    uint64_t* tab_full = bars + 20;     // resident tables landed
-    uint64_t* r_ready = bars + 21;      // operand X holds the modes, D_inc has been read (every work warp)
-    uint64_t* v_ready = bars + 22;      // operand X holds the bond forces (every work warp; warp 19: s_d0 has been read)
-    uint64_t* n_ready = bars + 23;      // noise buffer b written (every noise warp)
-    uint64_t* n_free = bars + 25;       // MMAs done with noise buffer b (a commit per parity)
-    uint64_t* u_done = bars + 27;       // inverse MMAs done (a commit per parity)
-    uint64_t* inc_done = bars + 28;     // noise and forward MMAs done (a commit per parity)
-    uint64_t* never = bars + 29;        // nothing arrives here (the stall test)
-    volatile int* abort_flag = (volatile int*)(bars + 30);
+    uint64_t* empty = bars + 12;        // ... MMAs done with it (commit)
+    uint64_t* tab_full = bars + 24;     // resident tables landed
+    uint64_t* r_ready = bars + 25;      // operand X holds the modes, D_inc has been read (every work warp)
+    uint64_t* v_ready = bars + 26;      // operand X holds the bond forces (every work warp; warp 19: s_d0 has been read; pair: + tx)
+    uint64_t* n_ready = bars + 27;      // noise buffer b written (every noise warp)
+    uint64_t* n_free = bars + 29;       // MMAs done with noise buffer b (a commit per parity)
+    uint64_t* u_done = bars + 31;       // inverse MMAs done (a commit per parity)
+    uint64_t* inc_done = bars + 32;     // noise and forward MMAs done (a commit per parity)
+    uint64_t* never = bars + 33;        // nothing arrives here (the stall test)
+    uint64_t* u_in = bars + 34;         // pair: the other CTA's bond vectors are in U (1 + tx)
+    volatile int* abort_flag = (volatile int*)(bars + 35);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp: uniform
     const int c0 = tile * a.cpt;
     const int Ct = min(a.cpt, a.C - c0);
+    const uint32_t rank = G::kPair ? cluster_rank() : 0u;
+    // an address of this CTA's shared memory in the other CTA of the pair
+    auto peer = [&](const void* p) { return mapa(smem_u32(p), rank ^ 1u); };
 
     if (threadIdx.x == 0) {
         if constexpr (G::kStream)
@@ -215,9 +254,10 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         mbar_init(tab_full, 1);
         mbar_init(r_ready, kWork);
         mbar_init(v_ready, kWork + 1);
+        mbar_init(u_in, 1);
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&n_ready[b], kNoise);
-            mbar_init(&n_free[b], NP);
+            mbar_init(&n_ready[b], G::kPair && b != (int)rank ? 1 : kNoise);    // a pair's other buffer: transaction bytes
+            mbar_init(&n_free[b], (G::kPair ? 2 : 1) * NP);
         }
         mbar_init(u_done, NP);
         mbar_init(inc_done, NP);
@@ -225,7 +265,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < kMaxChains; i += blockDim.x) {
+    for (int i = threadIdx.x; i < kMaxSlots; i += blockDim.x) {
         const bool live = i < Ct;
         const int64_t st = live ? a.step[c0 + i] : 0;
         int64_t left = live ? (int64_t)a.n_steps : 0;
@@ -241,13 +281,15 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         reinterpret_cast<uint4*>(X)[i] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async();
     fence_before();
-    __syncthreads();
+    if constexpr (G::kPair) cluster_sync();     // both CTAs' barriers are initialised
+    else __syncthreads();
     fence_after();
     const bool has_shear = __syncthreads_or(threadIdx.x < Ct && s_shear[threadIdx.x] != 0.0) != 0;
     // no chain of the tile is sheared or reaches its stop step in this launch
     const bool steady = __syncthreads_and(!has_shear && (threadIdx.x >= Ct || s_left[threadIdx.x] == a.n_steps)) != 0;
 
     if (warp == 0) {
+        const uint8_t* tab = la.tab + (G::kPair ? rank * (uint32_t)(G::BLK_TAB * kBlkBytes) : 0u);
         // ---------------- table blocks (the whole warp runs the loop, one lane issues:
         // see the MMA issuer)
         const bool leader = elect_one();
@@ -262,7 +304,9 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 if (!ok) break;
                 if (leader) {
                     mbar_expect_tx(&full[s], kBlkBytes);
-                    bulk_load(tabs + s * kBlkBytes, la.tab + src * kBlkBytes, kBlkBytes, &full[s]);
+                    // a pair's step takes the second half of w phi after h chi
+                    const int k = !G::kPair || src < 3 * G::BLK / 2 ? src : src < 5 * G::BLK / 2 ? src + G::BLK / 2 : src - G::BLK;
+                    bulk_load(tabs + s * kBlkBytes, tab + k * kBlkBytes, kBlkBytes, &full[s]);
                 }
                 if (++src == G::BLK_STEP) src = 0;
                 if (++s == G::ST) {
@@ -279,12 +323,12 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             if (leader) {
                 mbar_expect_tx(tab_full, G::BLK_TAB * kBlkBytes);
                 for (int k = 0; k < G::BLK_TAB; ++k)
-                    bulk_load(tabs + k * kBlkBytes, la.tab + k * kBlkBytes, kBlkBytes, tab_full);
+                    bulk_load(tabs + k * kBlkBytes, tab + k * kBlkBytes, kBlkBytes, tab_full);
             }
             mbar_wait(tab_full, 0, a.err, abort_flag);
         }
     } else if (warp == 1 || (NP == 2 && warp == 18)) {
-        const int e = warp == 1 ? 0 : NP - 1;           // this warp's parity
+        const int e = warp == 1 ? 0 : NP - 1;           // this warp's accumulator
         // ---------------- MMA issuer.  The whole warp runs the loops and the waits,
         // one elected lane issues: with everything but the issue itself uniform over
         // the warp, descriptors live in uniform registers and an MMA costs a few
@@ -296,20 +340,30 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         const bool leader = elect_one();
         bool ok = true;
         auto wait = [&](uint64_t* bar, uint32_t parity) {
-            ok = __all_sync(0xffffffffu, ok && mbar_wait(bar, parity, a.err, abort_flag));
+            if constexpr (G::kPair) {
+                ok = __all_sync(0xffffffffu, ok && mbar_wait_cl(bar, parity, a.err, abort_flag));
+                fence_proxy_async_all();        // operands that the other CTA's threads wrote
+            } else {
+                ok = __all_sync(0xffffffffu, ok && mbar_wait(bar, parity, a.err, abort_flag));
+            }
             fence_after();
         };
         if (a.stall_test) wait(never, 0);
         if constexpr (!G::kStream) wait(tab_full, 0);
         const uint64_t tab0 = ndesc(smem_u32(tabs), kALbo, kASbo);
-        const uint64_t x0 = ndesc(smem_u32(X) + e * 2 * kXPart, 128, kXSbo), z0 = ndesc(smem_u32(Z) + e * 2 * kZPart, kZLbo, 128);
+        const int ep = G::kPair ? 0 : e;                // operands: of this parity, or of the CTA's
+        const uint32_t z_bytes = (uint32_t)(G::ZK * 12 * Ct);       // a chunk of the other CTA: K x 3 axes x (hi, lo)
+        const uint64_t x0 = ndesc(smem_u32(X) + ep * 2 * G::XPART, 128, G::XSBO), z0 = ndesc(smem_u32(Z) + ep * 2 * G::ZPART, G::ZLBO, 128);
         int slot = e;                                   // ring slot and phase of this parity's next streamed block
         uint32_t phase = 0;
         // the three MMAs of a block, table hi/lo x operand hi/lo; b: the operand's hi
         // part (the lo part b_lo further)
         auto block = [&](int resident, uint32_t d, uint64_t b, uint32_t b_lo, uint32_t idesc, bool first) {
             const int s = G::kStream ? slot : resident;
-            if constexpr (G::kStream) wait(&full[s], phase);
+            if constexpr (G::kStream) {
+                ok = __all_sync(0xffffffffu, ok && mbar_wait(&full[s], phase, a.err, abort_flag));
+                fence_after();
+            }
             if (leader && ok) {
                 const uint64_t ah = tab0 + (uint64_t)(s * (kBlkBytes / 16)), al = ah + kBlkBytes / 32, bl = b + b_lo / 16;
                 mma_bf16(d, al, b, idesc, first ? 0u : 1u);
@@ -332,27 +386,43 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         auto with_x = [&](int res0, uint32_t d, bool first) {
 #pragma unroll(kUnroll)
             for (int k = 0; k < G::KP / 16; ++k)
-                block(res0 + k, d, x0 + (uint64_t)(k * (2 * 128 / 16)), kXPart, id_x, first && k == 0);
+                block(res0 + k, d, x0 + (uint64_t)(k * (2 * 128 / 16)), G::XPART, id_x, first && k == 0);
         };
-        const uint32_t d_u = tmem + e * kRowsN, d_inc = d_u + NP * kRowsN, d_z = G::kScaled ? d_inc + kRowsN : d_inc;
-        int chunk = 0;
+        const uint32_t d_u = tmem + e * G::ROWS, d_inc = d_u + NP * G::ROWS, d_z = G::kScaled ? d_inc + G::ROWS : d_inc;
+        // a noise chunk: its turn of the buffer of its number mod 2
+        auto with_z = [&](int sp, int ch) {
+            const int b = ch & 1;
+            wait(&n_ready[b], (sp * (G::NCH / 2) + (ch >> 1)) & 1);
+            if constexpr (G::kPair) {
+                // the other CTA's next chunk (no byte of it comes before both CTAs' MMAs have read this one)
+                if (warp == 1 && leader && ok && b != (int)rank) mbar_expect_tx(&n_ready[b], z_bytes);
+            }
+#pragma unroll(G::kPair ? 1 : G::ZK / 16)
+            for (int k = 0; k < G::ZK / 16; ++k)
+                block(G::BLK + (G::ZK / 16) * ch + k, d_z, z0 + (uint64_t)(b * (G::ZB / 16) + k * (2 * G::ZLBO / 16)), G::ZPART,
+                      id_z, ch == 0 && k == 0);
+            if (leader && ok) {
+                if constexpr (G::kPair) mma_commit_mc(&n_free[b], (uint16_t)(1u << b));     // to the CTA that draws this buffer
+                else mma_commit(&n_free[b]);
+            }
+        };
+        if constexpr (G::kPair) {
+            if (warp == 1 && leader) mbar_expect_tx(&n_ready[rank ^ 1u], z_bytes);
+        }
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps && ok; ++sp) {
             wait(r_ready, sp & 1);
             with_x(0, d_u, true);
             if (leader && ok) mma_commit(u_done);
 #pragma unroll 1
-            for (int ch = 0; ch < G::NCH; ++ch, ++chunk) {
-                const int b = chunk & 1;
-                wait(&n_ready[b], (chunk >> 1) & 1);
-#pragma unroll
-                for (int k = 0; k < 2; ++k)
-                    block(G::BLK + 2 * ch + k, d_z, z0 + (uint64_t)(b * (G::ZB / 16) + k * (2 * kZLbo / 16)), kZPart, id_z,
-                          ch == 0 && k == 0);
-                if (leader && ok) mma_commit(&n_free[b]);
-            }
+            for (int ch = 0; ch < (G::kPair ? 2 : G::NCH); ++ch) with_z(sp, ch);
             wait(v_ready, sp & 1);
             with_x(G::kScaled ? 0 : 2 * G::BLK, d_inc, G::kScaled);
+            if constexpr (G::kPair) {
+                // the later chunks, whose way between the CTAs passes behind the forward MMAs
+#pragma unroll 1
+                for (int ch = 2; ch < G::NCH; ++ch) with_z(sp, ch);
+            }
             if (leader && ok) mma_commit(inc_done);
         }
     } else if (warp >= 2 && warp < 2 + kWork) {
@@ -362,14 +432,19 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         // the tile's batches of four chains: this warp takes b0, b0 + bs, ... of its lanes
         const int b0 = ((warp - 2) >> 2) + (M == 64 ? 2 * (q >> 1) : 0), bs = M == 64 ? 4 : 2;
         const int nb = (Ct + 3) >> 2;
-        const bool own0 = (32 * q & (M == 64 ? 63 : 127)) == 0 && lane == 0;   // this thread holds mode 0
-        const uint32_t d_u = tmem + ((uint32_t)(32 * q) << 16), d_inc = d_u + NP * kRowsN;
+        const bool own0 = (32 * q & (M == 64 ? 63 : 127)) == 0 && lane == 0 && rank == 0;   // this thread holds mode 0
+        // accumulator e's mode in this lane, and its K index in operand X past lane j's
+        auto mode = [&](int e) { return G::kPair ? 2 * (128 * e + j) + (int)rank : NP * j + e; };
+        auto xoff = [](int e) { return G::kPair ? e * 128 * 16 : e * 2 * G::XPART; };
+        const uint32_t d_u = tmem + ((uint32_t)(32 * q) << 16), d_inc = d_u + NP * G::ROWS;
         auto col = [](int b) { return 24 * (b >> 1) + 4 * (b & 1); };          // the batch's first row
         uint8_t* xw = X + j * 16;
+        const uint32_t xw_peer = G::kPair ? peer(xw) : 0u, u_peer = G::kPair ? peer(U) : 0u;
+        const uint32_t v_peer = G::kPair ? peer(v_ready) : 0u, uin_peer = G::kPair ? peer(u_in) : 0u;
         float dm[NP], gw[NP], cs[NP], es[NP];
 #pragma unroll
         for (int e = 0; e < NP; ++e) {
-            const float4 c = la.lane_c[NP * j + e];
+            const float4 c = la.lane_c[mode(e)];
             dm[e] = c.x; gw[e] = c.y; cs[e] = c.z; es[e] = c.w;
         }
         bool ok = true;
@@ -379,14 +454,14 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             __syncwarp();
             if (lane == 0 && ok) mbar_arrive(bar);
         };
-        auto store_x = [&](uint2 hi, uint2 lo, int e, int ax, int b) {
-            uint8_t* w = xw + e * 2 * kXPart + (3 * (b >> 1) + ax) * kXSbo + (b & 1) * 8;
+        auto store_x = [&](uint2 hi, uint2 lo, int off, int ax, int b) {
+            uint8_t* w = xw + off + (3 * (b >> 1) + ax) * G::XSBO + (b & 1) * 8;
             *reinterpret_cast<uint2*>(w) = hi;
-            *reinterpret_cast<uint2*>(w + kXPart) = lo;
+            *reinterpret_cast<uint2*>(w + G::XPART) = lo;
         };
         // the modes (2 j, 2 j + 1) or j of a batch in global memory and in TMEM,
         // [parity][axis][chain]; chains past the tile's last are zero
-        float* Rj = a.R + (size_t)3 * c0 * M + NP * j;
+        float* Rj = a.R + (size_t)3 * c0 * M + mode(0);
         auto load_r = [&](float (&r)[NP][3][4], int b) {
             const float* p = Rj + (size_t)(12 * b) * M;
 #pragma unroll
@@ -394,7 +469,10 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 const bool live = 4 * b + i < Ct;
 #pragma unroll
                 for (int ax = 0; ax < 3; ++ax) {
-                    if constexpr (NP == 2) {
+                    if constexpr (G::kPair) {
+                        r[0][ax][i] = live ? p[(3 * i + ax) * M] : 0.f;
+                        r[NP - 1][ax][i] = live ? p[(3 * i + ax) * M + 256] : 0.f;
+                    } else if constexpr (NP == 2) {
                         const float2 x = live ? *reinterpret_cast<const float2*>(p + (3 * i + ax) * M) : make_float2(0.f, 0.f);
                         r[0][ax][i] = x.x;
                         r[NP - 1][ax][i] = x.y;
@@ -411,7 +489,10 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 if (4 * b + i < Ct)
 #pragma unroll
                     for (int ax = 0; ax < 3; ++ax) {
-                        if constexpr (NP == 2)
+                        if constexpr (G::kPair) {
+                            p[(3 * i + ax) * M] = r[0][ax][i];
+                            p[(3 * i + ax) * M + 256] = r[NP - 1][ax][i];
+                        } else if constexpr (NP == 2)
                             *reinterpret_cast<float2*>(p + (3 * i + ax) * M) = make_float2(r[0][ax][i], r[NP - 1][ax][i]);
                         else
                             p[(3 * i + ax) * M] = r[0][ax][i];
@@ -442,19 +523,36 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                     } else {
                         split4(r[e][ax], h, l);
                     }
-                    store_x(h, l, e, ax, b);
+                    store_x(h, l, xoff(e), ax, b);
                 }
         };
         // bond vectors -> residual force v (Eq. e11) of a batch, two chains at a time
         // (packed FP32)
         auto force4 = [&](int b) {
-            float u[NP][3][4];
+            float u[NP][3][4];                  // even and odd part
+            if constexpr (G::kPair) {
+                float own[3][4];
 #pragma unroll
-            for (int e = 0; e < NP; ++e)
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + rank * G::ROWS + 8 * ax + col(b), own[ax]);
+                tmem_wait12(own);
 #pragma unroll
-                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + e * kRowsN + 8 * ax + col(b), u[e][ax]);
+                for (int ax = 0; ax < 3; ++ax) {
+                    const float4 o = *reinterpret_cast<const float4*>(U + ((3 * b + ax) * 128 + j) * 16);
+                    const float oth[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
-            for (int e = 0; e < NP; ++e) tmem_wait12(u[e]);
+                    for (int i = 0; i < 4; ++i) {
+                        u[0][ax][i] = rank ? oth[i] : own[ax][i];
+                        u[NP - 1][ax][i] = rank ? own[ax][i] : oth[i];
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < NP; ++e)
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + e * G::ROWS + 8 * ax + col(b), u[e][ax]);
+#pragma unroll
+                for (int e = 0; e < NP; ++e) tmem_wait12(u[e]);
+            }
             uint2 xh[NP][3], xl[NP][3];
 #pragma unroll
             for (int i = 0; i < 4; i += 2) {
@@ -492,10 +590,31 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                         else split2(w[e][ax], xh[e][ax].y, xl[e][ax].y);
                     }
             }
+            if constexpr (G::kPair) {
+                // K index 128 rank + j of both CTAs' operands: this CTA's parity here, the other there
+                const int off = (int)rank * 128 * 16;
 #pragma unroll
-            for (int e = 0; e < NP; ++e)
+                for (int ax = 0; ax < 3; ++ax) {
+                    store_x(rank ? xh[NP - 1][ax] : xh[0][ax], rank ? xl[NP - 1][ax] : xl[0][ax], off, ax, b);
+                    const uint32_t w = xw_peer + off + (3 * (b >> 1) + ax) * G::XSBO + (b & 1) * 8;
+                    st_peer8(w, rank ? xh[0][ax] : xh[NP - 1][ax], v_peer);
+                    st_peer8(w + G::XPART, rank ? xl[0][ax] : xl[NP - 1][ax], v_peer);
+                }
+            } else {
 #pragma unroll
-                for (int ax = 0; ax < 3; ++ax) store_x(xh[e][ax], xl[e][ax], e, ax, b);
+                for (int e = 0; e < NP; ++e)
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) store_x(xh[e][ax], xl[e][ax], xoff(e), ax, b);
+            }
+        };
+        // pair: the bond vectors of the other CTA's lanes, to that CTA
+        auto send4 = [&](int b) {
+            float v[3][4];
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + (rank ^ 1u) * G::ROWS + 8 * ax + col(b), v[ax]);
+            tmem_wait12(v);
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) st_peer16(u_peer + ((3 * b + ax) * 128 + j) * 16, v[ax], uin_peer);
         };
         // update (Eqs. d3, btum) of a batch whose modes are in r (tm: in TMEM)
         auto update4 = [&](float (&r)[NP][3][4], int b, int sp, bool tm, bool plain) {
@@ -504,11 +623,11 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
 #pragma unroll
             for (int e = 0; e < NP; ++e)
 #pragma unroll
-                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + e * kRowsN + 8 * ax + col(b), d[e][ax]);
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + e * G::ROWS + 8 * ax + col(b), d[e][ax]);
             if constexpr (G::kScaled) {
                 float dz[3][4];
 #pragma unroll
-                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + kRowsN + 8 * ax + col(b), dz[ax]);
+                for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_inc + G::ROWS + 8 * ax + col(b), dz[ax]);
                 tmem_wait12(d[0]);
                 tmem_wait12(dz);
 #pragma unroll
@@ -563,8 +682,13 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         for (int sp = 0; sp < a.n_steps; ++sp) {
             ok = ok && mbar_wait(u_done, sp & 1, a.err, abort_flag);
             fence_after();
+            if constexpr (G::kPair) {
 #pragma unroll 1
-            for (int b = b0; b < nb; b += bs) force4(b);
+                for (int b = b0; ok && b < nb; b += bs) send4(b);
+                ok = ok && mbar_wait_cl(u_in, sp & 1, a.err, abort_flag);
+            }
+#pragma unroll 1
+            for (int b = b0; ok && b < nb; b += bs) force4(b);
             arrive(v_ready);
             // a batch whose modes are in global memory is updated last; they come from L2
             // while the forward MMAs run
@@ -626,13 +750,18 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         const int nw = warp - 2 - kWork;
         const int t = lane & 7;
         bool ok = true;
-        const int chunks = a.n_steps * G::NCH;
+        const uint32_t nr_peer = G::kPair ? peer(&n_ready[rank]) : 0u;
+        // a pair's CTAs draw the chunks of a step in turn, each into its own buffer of
+        // both CTAs (the sums for the even modes' CTA, the differences for the other)
+        // (K = 32 at a time: half a chunk of a pair)
+        constexpr int NDR = G::kPair ? G::KP / 64 : G::NCH;     // drawn by this CTA per step
+        const int chunks = a.n_steps * NDR;
         static_assert(G::NCH % 2 == 0, "chunks in pairs");
         // Both chunks of a pair are drawn before either is written, so that the second
         // half of a step's normals waits in registers for the first half's MMAs.
 #pragma unroll 1
         for (int chunk = 0; chunk < chunks; chunk += 2) {
-            const int sp = chunk / G::NCH, ch = chunk - G::NCH * sp;
+            const int sp = chunk / NDR, ch = chunk - NDR * sp;
             uint2 hi[2][NP][3], lo[2][NP][3];
             // with fewer batches than warps, a chunk's batches go to other warps than the last one's
             const int cl[2] = {4 * ((nw + 5 * chunk) & (kNoise - 1)) + (lane >> 3),
@@ -642,7 +771,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 if (cl[k] >= Ct) continue;
                 const uint32_t job = s_job[cl[k]];
                 const int64_t st = s_step[cl[k]] + sp;
-                const uint32_t b4 = (uint32_t)(8 * (ch + k) + t);       // beads 4 b4 ...
+                const uint32_t b4 = (uint32_t)(8 * (G::kPair ? 2 * ch + 2 * (int)rank + k : ch + k) + t);       // beads 4 b4 ...
                 float z[3][4];
                 bead_quad_normals<float>(a.seed, job, st, b4, 0u, z);
                 if constexpr (NP == 2) {
@@ -667,34 +796,63 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 // the MMAs have read the chunk that this buffer held
-                if (chunk >= 2) ok = ok && mbar_wait(&n_free[k], ((chunk >> 1) - 1) & 1, a.err, abort_flag);
+                const int buf = G::kPair ? (int)rank : k;
+                if constexpr (G::kPair) {
+                    if (chunk > 0 && k == 0) ok = ok && mbar_wait_cl(&n_free[buf], ((chunk >> 1) - 1) & 1, a.err, abort_flag);
+                } else {
+                    if (chunk >= 2) ok = ok && mbar_wait(&n_free[buf], ((chunk >> 1) - 1) & 1, a.err, abort_flag);
+                }
                 if (cl[k] < Ct && ok) {
                     const int b = cl[k] >> 2;
-                    uint8_t* w = Z + k * G::ZB + (t >> 1) * kZLbo + 3 * (b >> 1) * 128 + (4 * (b & 1) + (cl[k] & 3)) * 16 + (t & 1) * 8;
-#pragma unroll
-                    for (int e = 0; e < NP; ++e)
+                    uint8_t* w = Z + buf * G::ZB + ((G::kPair ? 4 * k : 0) + (t >> 1)) * G::ZLBO + 3 * (b >> 1) * 128 + (4 * (b & 1) + (cl[k] & 3)) * 16 + (t & 1) * 8;
+                    if constexpr (G::kPair) {
+                        const uint32_t wp = peer(w);
 #pragma unroll
                         for (int ax = 0; ax < 3; ++ax) {
-                            *reinterpret_cast<uint2*>(w + e * 2 * kZPart + ax * 128) = hi[k][e][ax];
-                            *reinterpret_cast<uint2*>(w + e * 2 * kZPart + kZPart + ax * 128) = lo[k][e][ax];
+                            *reinterpret_cast<uint2*>(w + ax * 128) = rank ? hi[k][NP - 1][ax] : hi[k][0][ax];
+                            *reinterpret_cast<uint2*>(w + G::ZPART + ax * 128) = rank ? lo[k][NP - 1][ax] : lo[k][0][ax];
+                            st_peer8(wp + ax * 128, rank ? hi[k][0][ax] : hi[k][NP - 1][ax], nr_peer);
+                            st_peer8(wp + G::ZPART + ax * 128, rank ? lo[k][0][ax] : lo[k][NP - 1][ax], nr_peer);
                         }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < NP; ++e)
+#pragma unroll
+                            for (int ax = 0; ax < 3; ++ax) {
+                                *reinterpret_cast<uint2*>(w + e * 2 * G::ZPART + ax * 128) = hi[k][e][ax];
+                                *reinterpret_cast<uint2*>(w + e * 2 * G::ZPART + G::ZPART + ax * 128) = lo[k][e][ax];
+                            }
+                    }
                 }
+                if (G::kPair && k == 0) continue;       // the two halves arrive together
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0 && ok) mbar_arrive(&n_ready[k]);
+                if (lane == 0 && ok) mbar_arrive(&n_ready[buf]);
             }
         }
+        // a pair: the other CTA's last commits to this CTA's n_free have landed
+        if constexpr (G::kPair) ok = ok && mbar_wait_cl(&n_free[rank], ((chunks >> 1) - 1) & 1, a.err, abort_flag);
     } else if (warp == 19) {
         // ---------------- the centre of mass (p = 0 of Eq. d3 with zeta_0 = 0) in
         // FP64, a chain per lane, and the step counters
         bool ok = true;
-        const bool live = lane < Ct;
+        const bool live = lane < Ct && rank == 0;       // a pair: the even modes' CTA
         double cm[3] = {0.0, 0.0, 0.0};
         double* cg = a.com + 3 * (size_t)(c0 + lane);
         if (live)
             for (int ax = 0; ax < 3; ++ax) cm[ax] = cg[ax];
         const double sh = __dmul_rn(s_shear[lane], a.dtau);
-        if (lane == 0) mbar_arrive(v_ready);
+        // a pair: it also arms the barriers for the other CTA's stores of a step
+        const uint32_t nb = (uint32_t)(Ct + 3) >> 2;
+        auto arm = [&] {
+            if constexpr (G::kPair) {
+                mbar_expect_tx(u_in, nb * 128u * 48u);
+                mbar_expect_tx(v_ready, nb * 128u * 48u);
+            } else {
+                mbar_arrive(v_ready);
+            }
+        };
+        if (lane == 0) arm();
         ok = mbar_wait(r_ready, 0, a.err, abort_flag);      // every phase in turn
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps; ++sp) {
@@ -706,7 +864,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 if (has_shear) cm[0] = fma(sh, ycm, cm[0]);
             }
             __syncwarp();
-            if (lane == 0 && ok && sp + 1 < a.n_steps) mbar_arrive(v_ready);
+            if (lane == 0 && ok && sp + 1 < a.n_steps) arm();
         }
         if (ok && live) {
             for (int ax = 0; ax < 3; ++ax) cg[ax] = cm[ax];
@@ -714,7 +872,19 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         }
     }
     fence_before();
-    __syncthreads();
+    __syncwarp();
+    if constexpr (G::kPair) {
+        // neither CTA leaves while the other may still write into its shared memory; after
+        // a timeout, what this CTA has under way there lands first
+        if (*abort_flag) {
+            const uint64_t t0 = globaltimer();
+            while (globaltimer() - t0 < 1000000ull) __nanosleep(1000);
+        }
+        __syncwarp();
+        cluster_sync();
+    } else {
+        __syncthreads();
+    }
     const bool good = *abort_flag == 0;
     if (!good) {
         // a wait gave up: let copies and MMAs in flight land before the memory goes

@@ -1,5 +1,5 @@
 """The lane step (bonds and modes on the TMEM lanes; BF16 hi/lo transforms at 64,
-128 and 256 beads) against the FP64 path of the same library from the same
+128, 256 and 512 beads) against the FP64 path of the same library from the same
 equilibrium starts and noise keys: chain counts at the edges of its tiles and of
 the groups that share a tile's chains, one and several steps per launch, with and
 without shear.
@@ -15,7 +15,7 @@ import paper_1411_3487_gb300 as sfp
 
 pytestmark = pytest.mark.gpu
 
-DTAU = {64: 10.0, 128: 50.0, 256: 100.0}
+DTAU = {64: 10.0, 128: 50.0, 256: 100.0, 512: 100.0}
 
 
 def run(M, C, n, shear, precision):
@@ -37,3 +37,11 @@ def test_lane_step_matches_fp64(M, C, n, shear):
     assert err.max() < 1e-5, (err.max(), err.argmax())
     assert np.abs(com - rcom).max() < 2.0 ** -16 * np.abs(rcom).max()
     assert (steps == n).all()
+
+
+@pytest.mark.parametrize("C,n,shear", [(1, 1, 0.0), (2, 3, 1e8), (23, 4, 0.0), (24, 5, 1e8), (25, 40, 1e8), (77, 2, 0.0),
+                                       (1824, 3, 0.0), (1825, 2, 1e8)])
+def test_lane_step_of_512_beads_on_two_ctas_matches_fp64(C, n, shear):
+    """A tile of up to 24 chains on a cluster of two CTAs, one parity of the modes
+    each: bonds are sums over both, normals and forces are shared by both."""
+    test_lane_step_matches_fp64(512, C, n, shear)
