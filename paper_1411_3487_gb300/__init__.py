@@ -80,6 +80,11 @@ class Batch:
             arr[i].job_id = int(c.get("job_id", i))
             self.n_beads[i] = arr[i].n_beads
         self.offsets = np.concatenate([[0], np.cumsum(3 * self.n_beads)])
+        # where the chains of a batch of several lengths lie in a packed array (plain
+        # integers: indexing with NumPy's costs several times as much per chain)
+        offs = self.offsets.tolist()
+        self._views = None if n == 0 or np.all(self.n_beads == self.n_beads[0]) else [
+            (slice(a, b), (3, (b - a) // 3)) for a, b in zip(offs, offs[1:])]
         self.n_chains = n
         self.precision = precision
         self._n_lags = self._lags_next = 4
@@ -143,9 +148,9 @@ class Batch:
 
     # -- outputs ---------------------------------------------------------------
     def _unpack(self, flat: np.ndarray):
-        if np.all(self.n_beads == self.n_beads[0]):
+        if self._views is None:
             return flat.reshape(self.n_chains, 3, int(self.n_beads[0]))
-        return [flat[self.offsets[i]:self.offsets[i + 1]].reshape(3, -1) for i in range(self.n_chains)]
+        return [flat[s].reshape(t) for s, t in self._views]
 
     def set_path(self, path: int) -> None:
         """SFP_PATH_FUSED (one kernel per step) or SFP_PATH_STAGED (one per stage, probes kept)."""

@@ -1086,15 +1086,16 @@ __global__ void k_load_modes(const S* __restrict__ src, T* __restrict__ R,
     }
 }
 
-// state -> modes (D = FP64 or FP32, R_0 = sqrt(M) r_cm)
+// state -> modes (D = FP64 or FP32, R_0 = sqrt(M) r_cm), chain c at off[c] (NULL: 3 c M)
 template <typename T, typename D>
 __global__ void k_store_modes(const T* __restrict__ R, const double* __restrict__ com,
-                              D* __restrict__ dst, int C, int M, double sqrtM)
+                              D* __restrict__ dst, const int64_t* __restrict__ off, int C, int M, double sqrtM)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)C * 3 * M) return;
     const int p = (int)(t % M);
-    dst[t] = (p == 0) ? (D)(com[t / M] * sqrtM) : (D)R[t];
+    const int64_t o = off ? off[t / M / 3] + t % (3 * (int64_t)M) : t;
+    dst[o] = (p == 0) ? (D)(com[t / M] * sqrtM) : (D)R[t];
 }
 
 template <typename T>
