@@ -117,16 +117,31 @@ static_assert(2 + kComputeWarps == 10 && kComputeWarps == 8, "warp numbering of 
 // three stages stay faster: 24.0 against 24.5 us); the 512-bead kernel splits
 // in place.
 template <int NB, bool BF, bool MZ = false> constexpr bool kRS = BF && (NB != 256 || MZ);
-template <int NB, bool BF, bool RS>
+// Mirror symmetry (TF32, 128 and 256 beads): chi_{n,p} and phi_{n,p} are even or odd
+// under n -> M - n and n -> M - 1 - n with the parity of p, so each contraction splits
+// into two of half the rows and half the K, and the MMAs and the table bytes of a step
+// halve.  D_u and D_inc hold the even modes' half in their first NB / 2 columns and the
+// odd modes' in the rest; a K block holds 16 even indices, then the 16 odd ones: modes
+// (the split of R sorts them), or 16 bonds / beads n < NB / 2 as v_n - v_{M-n} and
+// z_n + z_{M-1-n}, then v_n + v_{M-n} and z_n - z_{M-1-n}.  Bond M / 2, its own mirror
+// image, takes n = 0, where there is no bond, with half its table column.  A step's MMAs
+// (12 of 128 columns a block, bound by their operands' way out of shared memory: about
+// 1100 cycles) take 14 us of it; the rest is the state's way through L2 at the step's end.
+// us a step in a 400-step call: 4096 x 256 bp 30.9 -> 22.4, one chain 25.9 -> 19.3, 4096 x
+// 128 bp 14.1 -> 11.6, 50 x 128 bp 11.7 -> 9.8.  At 64 beads, where the MMAs' A operand
+// sets their pace either way, the whole product stays.
+template <int NB, bool BF> constexpr bool kFold = !BF && NB >= 128;
+template <int NB, bool BF, bool RS, bool FOLD = false>
 struct FSmem {
     static constexpr int kEl = BF ? 2 : 4;
     static constexpr int kA = kRows * kKB * kEl;          // 16 KB (TF32) / 8 KB (BF16)
-    static constexpr int kB = NB * kKB * kEl;             // NB x 128 B / NB x 64 B
+    static constexpr int kN = FOLD ? NB / 2 : NB;         // B operand rows: the MMA's N
+    static constexpr int kB = kN * kKB * kEl;             // kN x 128 B / kN x 64 B
     static constexpr int kR = RS ? kRows * kKB * 4 : 0;   // FP32 R staging (BF16, RS)
     static constexpr int kStage = kR + 2 * kA + 2 * kB;
     static_assert(RS || kRows * kKB * 4 <= 2 * kA, "an FP32 R tile fits the A operand region");
     static constexpr int kStages = BF ? ((192 * 1024) / kStage < 4 ? (192 * 1024) / kStage : 4)
-                                      : (NB == 256 ? 2 : NB == 128 ? 3 : 4);
+                                      : (kN == 256 ? 2 : kN == 128 ? 3 : 4);
     static constexpr int kRT = kRows * kKB * 4;           // an FP32 R block of the epilogue, 16 KB
     static constexpr int kMisc = 5120;   // per-chain keys, steps, shear, stops; tables; barriers
     static constexpr int kBytes = kStages * kStage + kMisc + 1024;
@@ -165,6 +180,19 @@ __device__ __forceinline__ void put_hi_lo(uint8_t* hi, uint8_t* lo, int r, int k
         *reinterpret_cast<float*>(hi + o) = h;
         *reinterpret_cast<float*>(lo + o) = tf32_rna(x - h);
     }
+}
+
+// Four consecutive TF32 elements (r, k .. k + 3), k a multiple of 4.
+__device__ __forceinline__ void put4_hi_lo(uint8_t* hi, uint8_t* lo, int r, int k, const float (&x)[4])
+{
+    float4 h, l;
+    h.x = tf32_rna(x[0]); l.x = tf32_rna(x[0] - h.x);
+    h.y = tf32_rna(x[1]); l.y = tf32_rna(x[1] - h.y);
+    h.z = tf32_rna(x[2]); l.z = tf32_rna(x[2] - h.z);
+    h.w = tf32_rna(x[3]); l.w = tf32_rna(x[3] - h.w);
+    const uint32_t o = swz(r, k);
+    *reinterpret_cast<float4*>(hi + o) = h;
+    *reinterpret_cast<float4*>(lo + o) = l;
 }
 
 // Order of the 3 KB blocks of one step (KB = NB / 32 bead blocks, H = KB / 2).
@@ -319,7 +347,8 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
                                            const CUtensorMap& tmFL, const FusedArgs& a, int tile, uint8_t* smem,
                                            uint32_t tmem)
 {
-    using S = FSmem<NB, BF, kRS<NB, BF, MZ>>;
+    constexpr bool FOLD = kFold<NB, BF>;
+    using S = FSmem<NB, BF, kRS<NB, BF, MZ>, FOLD>;
     constexpr int ST = S::kStages;
     constexpr int KB = NB / kKB;        // inverse K blocks = forward bead blocks
     constexpr int NBLK = MZ ? 2 * KB : 3 * KB;   // blocks of one step, in the order of sched_decode (MZ: sched_mz)
@@ -402,6 +431,22 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
     const uint32_t t_u = tmem, t_inc = tmem + NB;
     const bool has_shear = __syncthreads_or(threadIdx.x < Ct && s_shear[threadIdx.x] != 0.0) != 0;
 
+    // D_inc of modes p0 .. p0 + 15 in lane quarter q
+    auto load_inc = [&](float (&d)[16], int q, int p0) {
+        const uint32_t t = t_inc + ((uint32_t)(32 * q) << 16);
+        if constexpr (FOLD) {
+            float ev[8], od[8];
+            tmem_ld8x2(t + p0 / 2, t + NB / 2 + p0 / 2, ev, od);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                d[2 * i] = ev[i];
+                d[2 * i + 1] = od[i];
+            }
+        } else {
+            tmem_ld16(t + (uint32_t)p0, d);
+        }
+    };
+
     // Epilogue of step sp (R += -dm R + D_inc (+ shear), Eqs. d3, btum) on the R
     // tile that the producer reloads into the stage memory (KB column blocks of
     // [128 rows][32], swizzled, each with its own barrier), in place.  The
@@ -443,11 +488,11 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
                         z[4 * k4] = x.x; z[4 * k4 + 1] = x.y; z[4 * k4 + 2] = x.z; z[4 * k4 + 3] = x.w;
                     }
-                    tmem_ld16(t_inc + ((uint32_t)(32 * q) << 16) + (uint32_t)p0, d);
+                    load_inc(d, q, p0);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) d[i] = fmaf(s_w[p0 + i], z[i], d[i]);
                 } else {
-                    tmem_ld16(t_inc + ((uint32_t)(32 * q) << 16) + (uint32_t)p0, d);
+                    load_inc(d, q, p0);
                 }
 #pragma unroll
                 for (int k4 = 0; k4 < 4; ++k4) {
@@ -537,8 +582,8 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
                     // noise block nb: rows w_p phi (t = 1); force block nb: rows h_p chi (t = 0)
                     const bool noise = kind == 1;
                     mbar_expect_tx(&full[s], 2 * S::kB);
-                    tma_load_2d(bh, &tmFH, &full[s], nb * kKB, noise ? NB : 0);
-                    tma_load_2d(bl, &tmFL, &full[s], nb * kKB, noise ? NB : 0);
+                    tma_load_2d(bh, &tmFH, &full[s], nb * kKB, noise ? S::kN : 0);
+                    tma_load_2d(bl, &tmFL, &full[s], nb * kKB, noise ? S::kN : 0);
                 }
             }
             // reload the R tile (KB column blocks of [128 rows][32]) into the stage
@@ -571,57 +616,69 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
           }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = BF ? idesc_bf16(kRows, NB) : idesc_tf32(kRows, NB);
-            bool ok = true;
-            // stall test: this wait runs out after its limit, raises the timeout bit
-            // and the abort flag, and every other wait of the CTA then gives up
-            if (a.stall_test) ok = mbar_wait(never, 0, a.err, abort_flag);
-            for (int sp = 0; sp < a.n_steps; ++sp) {
+        // ---------------- MMA issuer.  The whole warp runs the loop and the waits and one
+        // elected lane issues: with the rest uniform over the warp, descriptors live in
+        // uniform registers and an MMA costs a few instructions.
+        constexpr uint32_t idesc = BF ? idesc_bf16(kRows, S::kN) : idesc_tf32(kRows, S::kN);
+        const bool leader = lanes::elect_one();
+        const uint32_t a0 = smem_u32(stage0) + S::kR;
+        const uint64_t desc0 = BF ? sdesc64(a0) : sdesc(a0);
+        auto wait = [&](uint64_t* bar, uint32_t parity, bool ok) {
+            return __all_sync(0xffffffffu, ok && mbar_wait(bar, parity, a.err, abort_flag)) != 0;
+        };
+        bool ok = true;
+        // stall test: this wait runs out after its limit, raises the timeout bit
+        // and the abort flag, and every other wait of the CTA then gives up
+        if (a.stall_test) ok = wait(never, 0, ok);
+        int s = 0;
+        uint32_t ph = 0;
+#pragma unroll 1
+        for (int sp = 0; sp < a.n_steps; ++sp) {
+#pragma unroll 1
             for (int blk = 0; blk < NBLK; ++blk) {
-                const int gb = sp * NBLK + blk;
-                const int s = gb % ST;
-                const uint32_t ph = (gb / ST) & 1;
                 int kind, nb;
                 sched_decode_any<KB, BF ? 0 : 1, MZ>(blk, kind, nb);
-                ok = ok && mbar_wait(&full[s], ph, a.err, abort_flag);
-                ok = ok && mbar_wait(&ready[s], ph, a.err, abort_flag);
-                if (ok) {
-                    fence_after();
-                    const uint32_t st = smem_u32(stage0 + s * S::kStage);
-                    const uint32_t a_hi = st + S::kR, a_lo = a_hi + S::kA, b_hi = a_lo + S::kA, b_lo = b_hi + S::kB;
+                ok = wait(&full[s], ph, ok);
+                ok = wait(&ready[s], ph, ok);
+                fence_after();
+                if (leader && ok) {
+                    const uint64_t a_hi = desc0 + (uint64_t)(s * (S::kStage / 16)), a_lo = a_hi + S::kA / 16,
+                                   b_hi = a_lo + S::kA / 16, b_lo = b_hi + S::kB / 16;
                     const uint32_t d = kind == 0 ? t_u : t_inc;
                     // first inverse block, first forward (noise, or force with MZ) block
                     const bool first = MZ ? (blk == 0 || blk == KB) : blk <= 1;
                     if constexpr (BF) {
 #pragma unroll
                         for (int kk = 0; kk < kKB / 16; ++kk) {
-                            const uint32_t off = kk * 32;   // 16 BF16 = 32 bytes along K
+                            const uint64_t off = 2 * kk;    // 16 BF16 = 32 bytes along K
                             if constexpr (TWO) {
-                                mma_bf16(d, sdesc64(a_lo + off), sdesc64(b_hi + off), idesc, (first && kk == 0) ? 0u : 1u);
+                                mma_bf16(d, a_lo + off, b_hi + off, idesc, (first && kk == 0) ? 0u : 1u);
                             } else {
-                                mma_bf16(d, sdesc64(a_hi + off), sdesc64(b_lo + off), idesc, (first && kk == 0) ? 0u : 1u);
-                                mma_bf16(d, sdesc64(a_lo + off), sdesc64(b_hi + off), idesc, 1u);
+                                mma_bf16(d, a_hi + off, b_lo + off, idesc, (first && kk == 0) ? 0u : 1u);
+                                mma_bf16(d, a_lo + off, b_hi + off, idesc, 1u);
                             }
-                            mma_bf16(d, sdesc64(a_hi + off), sdesc64(b_hi + off), idesc, 1u);
+                            mma_bf16(d, a_hi + off, b_hi + off, idesc, 1u);
                         }
                     } else {
 #pragma unroll
                         for (int kk = 0; kk < kKB / 8; ++kk) {
-                            const uint32_t off = kk * 32;   // 8 TF32 = 32 bytes along K
-                            mma_tf32(d, sdesc(a_hi + off), sdesc(b_lo + off), idesc, (first && kk == 0) ? 0u : 1u);
-                            mma_tf32(d, sdesc(a_lo + off), sdesc(b_hi + off), idesc, 1u);
-                            mma_tf32(d, sdesc(a_hi + off), sdesc(b_hi + off), idesc, 1u);
+                            const uint64_t off = 2 * kk;    // 8 TF32 = 32 bytes along K
+                            // mirror symmetry: the even indices' half of D, then the odd ones'
+                            const uint32_t dk = FOLD && kk >= 2 ? d + NB / 2 : d;
+                            const bool zero = first && (kk == 0 || (FOLD && kk == 2));
+                            mma_tf32(dk, a_hi + off, b_lo + off, idesc, zero ? 0u : 1u);
+                            mma_tf32(dk, a_lo + off, b_hi + off, idesc, 1u);
+                            mma_tf32(dk, a_hi + off, b_hi + off, idesc, 1u);
                         }
                     }
-                }
-                if (ok) {
                     mma_commit(&empty[s]);
                     if (blk == (MZ ? KB - 1 : sched_inv<KB>(KB - 1))) mma_commit(u_done);
+                    if (blk == NBLK - 1) mma_commit(inc_done);
                 }
-            }
-            if (ok) mma_commit(inc_done);
+                if (++s == ST) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
         }
     } else if (MZ && warp >= 2 + kComputeWarps) {
@@ -666,6 +723,76 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps; ++sp) {
             if (sp + 1 < a.n_steps) draw_step(sp + 1);
+            epilogue(sp, eq, 2 + et, 2 + kNoiseInQ[(eq + 2) & 3], ok, finite, cm_unused[0], cm_unused[1], cm_unused[2]);
+        }
+        if (!finite) atomicOr(a.err, 1);
+    } else if (FOLD && warp >= 2 + kComputeWarps) {
+        // ---------------- noise warps, mirror symmetry: noise block j holds beads
+        // 16 j .. 16 j + 15 and their mirror images.  An item is four consecutive beads
+        // of a chain and their four images (six Philox calls, all that the sums and
+        // differences of those beads take: eight values for 16-byte stores); a block is
+        // cpt / 8 chunks of 32 items, chunk h of block qn drawn by warp (h + nch qn) mod
+        // kNoiseWarps, which alone arrives for it.  A warp so has blocks in between to
+        // draw its next chunk in, which it does right after it has written one.
+        const int nw = warp - 2 - kComputeWarps;
+        const int nch = (a.cpt + 7) >> 3;
+        const int eq = warp & 3, et = nw / 4;       // epilogue quarter, worker 2 + et
+        const int nq = a.n_steps * KB;
+        static_assert(kChains <= 8 * kNoiseWarps, "at most a chunk per warp and block");
+        bool ok = true, finite = true;
+        double cm_unused[3];
+        // this warp's chunk of block qn (none if not below nch)
+        auto chunk = [&](int qn) { return (nw + kNoiseWarps * nch - nch * (qn % kNoiseWarps)) % kNoiseWarps; };
+        auto next = [&](int qn) {
+            while (qn < nq && chunk(qn) >= nch) ++qn;
+            return qn;
+        };
+        float ev[3][4], od[3][4];       // [axis][bead]
+        auto draw = [&](int qn) {
+            const int f = 32 * chunk(qn) + lane, cl = f >> 2, sp = qn / KB, j = qn - KB * (qn / KB);
+            const bool live = cl < Ct;
+            const uint32_t job = live ? s_job[cl] : 0u;
+            const int64_t st = (live ? s_step[cl] : 0) + sp;
+            const uint32_t b4 = (uint32_t)(4 * j + (f & 3));
+            float z[3][4], y[3][4];
+            bead_quad_normals<float>(a.seed, job, st, b4, 0u, z);
+            bead_quad_normals<float>(a.seed, job, st, (uint32_t)(NB / 4 - 1) - b4, 0u, y);
+#pragma unroll
+            for (int ax2 = 0; ax2 < 3; ++ax2)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    ev[ax2][i] = live ? z[ax2][i] + y[ax2][3 - i] : 0.f;
+                    od[ax2][i] = live ? z[ax2][i] - y[ax2][3 - i] : 0.f;
+                }
+        };
+        int qn = next(0);
+        if (qn < nq) draw(qn);
+#pragma unroll 1
+        for (int sp = 0; sp < a.n_steps; ++sp) {
+#pragma unroll 1
+            while (qn < KB * (sp + 1)) {
+                const int blk = sp * NBLK + sched_noise<KB, BF ? 0 : 1>(qn - KB * sp), s = blk % ST;
+                const int h = chunk(qn), cl = (32 * h + lane) >> 2;
+                ok = ok && count_wait(s_freed, blk, a.err, abort_flag);     // see below
+                if (ok) {
+                    if (cl < a.cpt) {
+                        uint8_t* ah = stage0 + s * S::kStage;
+                        const int rb = s_rowb[cl];
+#pragma unroll
+                        for (int ax2 = 0; ax2 < 3; ++ax2) {
+                            put4_hi_lo(ah, ah + S::kA, rb + ax2, 4 * (lane & 3), ev[ax2]);
+                            put4_hi_lo(ah, ah + S::kA, rb + ax2, 16 + 4 * (lane & 3), od[ax2]);
+                        }
+                    }
+                    fence_proxy_async();
+                }
+                __syncwarp();
+                // the weights of a block's chunks add up to the count
+                if (lane == 0 && ok)
+                    mbar_arrive_cnt(&ready[s], kReadyCount / nch + (h < kReadyCount % nch ? 1 : 0));
+                qn = next(qn + 1);
+                if (qn < nq) draw(qn);
+            }
             epilogue(sp, eq, 2 + et, 2 + kNoiseInQ[(eq + 2) & 3], ok, finite, cm_unused[0], cm_unused[1], cm_unused[2]);
         }
         if (!finite) atomicOr(a.err, 1);
@@ -825,6 +952,28 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
                     *reinterpret_cast<uint4*>(al + o) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
                 }
                 fence_proxy_async();
+            } else if (FOLD) {
+                // two threads to a row, 16 modes each, sorted into even and odd ones: the
+                // warp reads its rows before it writes them
+                uint8_t* base = stage0 + s * S::kStage;
+                const int r = ct >> 1, k0 = 16 * (ct & 1);
+                const bool use = ok && (r & 31) < 3 * cpq;
+                float4 x[4];
+                if (use) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(base + swz(r, k0 + 4 * i));
+                }
+                __syncwarp();
+                if (use) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const float e4[4] = {x[2 * i].x, x[2 * i].z, x[2 * i + 1].x, x[2 * i + 1].z};
+                        const float o4[4] = {x[2 * i].y, x[2 * i].w, x[2 * i + 1].y, x[2 * i + 1].w};
+                        put4_hi_lo(base, base + S::kA, r, k0 / 2 + 4 * i, e4);
+                        put4_hi_lo(base, base + S::kA, r, 16 + k0 / 2 + 4 * i, o4);
+                    }
+                }
+                if (ok) fence_proxy_async();
             } else if (ok) {
                 float4* ah = (float4*)(stage0 + s * S::kStage);
                 float4* al = (float4*)(stage0 + s * S::kStage + S::kA);
@@ -852,15 +1001,35 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
         fence_after();
 #pragma unroll 1
         for (int nb = 0; nb < KB; ++nb) {
-            const int col = nb * kKB + 16 * half;       // first bead of this warp's 16
             float v[16];
-            tmem_ld16(t_u + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
+            if constexpr (FOLD) {
+                // bonds n and M - n from the even and odd modes' parts; their forces back
+                // to even (v[0 .. 7]) and odd operands (8 .. 15) of 8 n
+                const uint32_t t = t_u + ((uint32_t)(32 * q) << 16) + (uint32_t)(16 * nb + 8 * half);
+                float ev[8], od[8];
+                tmem_ld8x2(t, t + NB / 2, ev, od);
+                auto unit = [&](float x) {
+                    const float sq = x * x;
+                    const float t2 = sq + __shfl_down_sync(0xffffffffu, sq, 1) + __shfl_down_sync(0xffffffffu, sq, 2);
+                    return __shfl_sync(0xffffffffu, rsqrtf(t2) - a.c12nu, src0);
+                };
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float sq = v[i] * v[i];
-                const float t = sq + __shfl_down_sync(0xffffffffu, sq, 1) + __shfl_down_sync(0xffffffffu, sq, 2);
-                const float fac = __shfl_sync(0xffffffffu, rsqrtf(t) - a.c12nu, src0);
-                v[i] = (live && col + i >= 1) ? v[i] * fac : 0.f;
+                for (int i = 0; i < 8; ++i) {
+                    const float p = od[i] + ev[i], m = od[i] - ev[i];
+                    const float fp = unit(p), vm = m * unit(m);
+                    v[i] = live ? fmaf(p, fp, -vm) : 0.f;
+                    v[8 + i] = live ? fmaf(p, fp, vm) : 0.f;
+                }
+            } else {
+                const int col = nb * kKB + 16 * half;       // first bead of this warp's 16
+                tmem_ld16(t_u + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float sq = v[i] * v[i];
+                    const float t = sq + __shfl_down_sync(0xffffffffu, sq, 1) + __shfl_down_sync(0xffffffffu, sq, 2);
+                    const float fac = __shfl_sync(0xffffffffu, rsqrtf(t) - a.c12nu, src0);
+                    v[i] = (live && col + i >= 1) ? v[i] * fac : 0.f;
+                }
             }
             const int blk = g0 + (MZ ? KB + nb : sched_force<KB, BF ? 0 : 1>(nb)), s = blk % ST;
             const uint32_t ph = (blk / ST) & 1;
@@ -886,14 +1055,9 @@ __device__ __forceinline__ bool fused_tile(const CUtensorMap& tmR, const CUtenso
                 } else {
 #pragma unroll
                     for (int k4 = 0; k4 < 4; ++k4) {
-                        float4 h, l;
-                        h.x = tf32_rna(v[4 * k4]);     l.x = tf32_rna(v[4 * k4] - h.x);
-                        h.y = tf32_rna(v[4 * k4 + 1]); l.y = tf32_rna(v[4 * k4 + 1] - h.y);
-                        h.z = tf32_rna(v[4 * k4 + 2]); l.z = tf32_rna(v[4 * k4 + 2] - h.z);
-                        h.w = tf32_rna(v[4 * k4 + 3]); l.w = tf32_rna(v[4 * k4 + 3] - h.w);
-                        const uint32_t o = swz(row, 16 * half + 4 * k4);
-                        *reinterpret_cast<float4*>(ah + o) = h;
-                        *reinterpret_cast<float4*>(al + o) = l;
+                        const int k = FOLD ? 16 * (k4 >> 1) + 8 * half + 4 * (k4 & 1) : 16 * half + 4 * k4;
+                        const float x[4] = {v[4 * k4], v[4 * k4 + 1], v[4 * k4 + 2], v[4 * k4 + 3]};
+                        put4_hi_lo(ah, al, row, k, x);
                     }
                 }
             }
@@ -1664,6 +1828,7 @@ struct FusedPlan {
     float4* lane_c = nullptr;      // ... and per-mode constants
     size_t lane_bytes = 0;
     bool classic = false;          // tables of the other kernels exist
+    bool fold = false;             // ... in the halves of the mirror symmetry
     // what the tables of the other kernels are made of, until mode-keyed noise needs them
     std::vector<double> chi, phi, h, w;
     cudaStream_t stream = nullptr;
@@ -1687,15 +1852,15 @@ static int grouped_smem(bool bf16, bool two)
         return std::max({lanes::Geo<512>::kBytes, lanes::Geo<256>::kBytes, lanes::Geo<128>::kBytes, lanes::Geo<64>::kBytes});
     return bf16 ? std::max({FSmem<256, true, true>::kBytes, FSmem<128, true, true>::kBytes, FSmem<64, true, true>::kBytes,
                             FSmem<256, true, false>::kBytes})
-                : std::max({FSmem<256, false, false>::kBytes, FSmem<128, false, false>::kBytes,
-                            FSmem<64, false, false>::kBytes});
+                : std::max({FSmem<256, false, false>::kBytes, FSmem<256, false, false, kFold<256, false>>::kBytes,
+                            FSmem<128, false, false, kFold<128, false>>::kBytes, FSmem<64, false, false>::kBytes});
 }
 
 template <int NB, bool BF, bool TWO = false, bool MZ = false>
 static cudaError_t set_smem()
 {
     return cudaFuncSetAttribute(k_fused_step<NB, BF, TWO, MZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                FSmem<NB, BF, kRS<NB, BF, MZ>>::kBytes);
+                                FSmem<NB, BF, kRS<NB, BF, MZ>, kFold<NB, BF>>::kBytes);
 }
 template <int M>
 static cudaError_t set_smem_lane()
@@ -1778,14 +1943,33 @@ static int classic_tables(FusedPlan* p, const double* chi, const double* phi, co
     // chi [n][p] (row n = 0 and column p = 0 are zero) and F [2M][M]:
     // F[p][n] = h_p chi[n][p] (Eq. f2 weight on DeltaH = chi^T v, Eq. e11),
     // F[M + p][n] = w_p phi[n][p] (Eq. d6 weight on Z = phi^T z, Eq. c4).
-    std::vector<double> F(2 * mm);
-    for (int q = 0; q < M; ++q)
-        for (int n = 0; n < M; ++n) {
-            F[(size_t)q * M + n] = h[q] * chi[(size_t)n * M + q];
-            F[mm + (size_t)q * M + n] = w[q] * phi[(size_t)n * M + q];
-        }
-    const double* src[2] = {chi, F.data()};
-    const size_t cnt[2] = {mm, 2 * mm};
+    const bool fold = p->fold = !bf16 && (M == 256 ? kFold<256, false> : M == 128 ? kFold<128, false> : false);
+    const int half = M / 2;
+    std::vector<double> F(fold ? mm : 2 * mm), C(fold ? mm / 2 : 0);
+    if (fold) {
+        // rows: bonds n < M / 2, modes 2 i + e of column parity e; columns: per 32 the
+        // 16 even indices, then the 16 odd ones (modes of chi, bonds and beads of F)
+        for (int i = 0; i < half; ++i)
+            for (int c = 0; c < M; ++c) {
+                const int e = (c & 31) >> 4, k = c & 15;
+                const int pc = 32 * (c >> 5) + 2 * k + e, q = 2 * i + e, n = 16 * (c >> 5) + k;
+                // bond M / 2 in the place of n = 0
+                auto x = [&](int bond, int mode) {
+                    return bond ? chi[(size_t)bond * M + mode] : e ? chi[(size_t)half * M + mode] : 0.0;
+                };
+                C[(size_t)i * M + c] = x(i, pc);
+                F[(size_t)i * M + c] = h[q] * x(n, q) * (n ? 1.0 : 0.5);
+                F[mm / 2 + (size_t)i * M + c] = w[q] * phi[(size_t)n * M + q];
+            }
+    } else {
+        for (int q = 0; q < M; ++q)
+            for (int n = 0; n < M; ++n) {
+                F[(size_t)q * M + n] = h[q] * chi[(size_t)n * M + q];
+                F[mm + (size_t)q * M + n] = w[q] * phi[(size_t)n * M + q];
+            }
+    }
+    const double* src[2] = {fold ? C.data() : chi, F.data()};
+    const size_t cnt[2] = {fold ? mm / 2 : mm, F.size()};
     const size_t el = bf16 ? 2 : 4;
     for (int t = 0; t < 2; ++t) {
         std::vector<float> hi(cnt[t]), lo(cnt[t]);
@@ -1814,15 +1998,15 @@ static int classic_tables(FusedPlan* p, const double* chi, const double* phi, co
     // the next tile's chains
     if ((rc = make_map_2d(&p->tmR, p->R, 3 * p->C, M, 3 * (p->cpt / 4)))) return rc;
     // B operand boxes: the rows of one CTA's TMEM half (all M, or 256 of 512)
-    const int bx = std::min(M, 256);
+    const int rows = fold ? half : M, bx = std::min(rows, 256);
     if (bf16)
         rc = make_map_bf16(&p->tmChiH, p->tab[0], M, M, bx) ? -1 : make_map_bf16(&p->tmChiL, p->tab[1], M, M, bx) ? -1 :
              make_map_bf16(&p->tmFH, p->tab[2], 2 * M, M, bx) ? -1 : make_map_bf16(&p->tmFL, p->tab[3], 2 * M, M, bx);
     else
-        rc = make_map_2d(&p->tmChiH, (const float*)p->tab[0], M, M, bx) ? -1 :
-             make_map_2d(&p->tmChiL, (const float*)p->tab[1], M, M, bx) ? -1 :
-             make_map_2d(&p->tmFH, (const float*)p->tab[2], 2 * M, M, bx) ? -1 :
-             make_map_2d(&p->tmFL, (const float*)p->tab[3], 2 * M, M, bx);
+        rc = make_map_2d(&p->tmChiH, (const float*)p->tab[0], rows, M, bx) ? -1 :
+             make_map_2d(&p->tmChiL, (const float*)p->tab[1], rows, M, bx) ? -1 :
+             make_map_2d(&p->tmFH, (const float*)p->tab[2], 2 * rows, M, bx) ? -1 :
+             make_map_2d(&p->tmFL, (const float*)p->tab[3], 2 * rows, M, bx);
     if (rc) return SFP_ECUDA;
     cudaError_t e;
     if (p->two)
@@ -1946,13 +2130,13 @@ int fused_step(FusedPlan* p, const FusedArgs& args, cudaStream_t stream)
     }
 #define SFP_FUSED_LAUNCH(NBV, BFV)                                                                   \
     if (p->mz)                                                                                       \
-        k_fused_step<NBV, BFV, false, true><<<grid, kThreads, FSmem<NBV, BFV, kRS<NBV, BFV, true>>::kBytes, stream>>>( \
+        k_fused_step<NBV, BFV, false, true><<<grid, kThreads, FSmem<NBV, BFV, kRS<NBV, BFV, true>, kFold<NBV, BFV>>::kBytes, stream>>>( \
             p->tmR, p->tmChiH, p->tmChiL, p->tmFH, p->tmFL, a);                                      \
     else if (p->two)                                                                                 \
         k_fused_step<NBV, BFV, BFV><<<grid, kThreads, FSmem<NBV, BFV, kRS<NBV, BFV>>::kBytes, stream>>>(         \
             p->tmR, p->tmChiH, p->tmChiL, p->tmFH, p->tmFL, a);                                      \
     else if constexpr (!BFV)                                                                         \
-        k_fused_step<NBV, false><<<grid, kThreads, FSmem<NBV, false, false>::kBytes, stream>>>(                  \
+        k_fused_step<NBV, false><<<grid, kThreads, FSmem<NBV, false, false, kFold<NBV, false>>::kBytes, stream>>>(                  \
             p->tmR, p->tmChiH, p->tmChiL, p->tmFH, p->tmFL, a)
     cudaError_t e = cudaSuccess;
     switch (p->M * 2 + (p->bf16 ? 1 : 0)) {
@@ -2040,7 +2224,7 @@ int fused_ctas_per_tile(const FusedPlan* p) { return p->M == 512 ? 2 : 1; }
 size_t fused_bytes(const FusedPlan* p)
 {
     if (!p) return 0;
-    return (p->classic ? (size_t)6 * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float) : 0) +
+    return (p->classic ? (size_t)(p->fold ? 3 : 6) * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float) : 0) +
            (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0) + p->lane_bytes;
 }
 
