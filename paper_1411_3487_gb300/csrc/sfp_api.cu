@@ -547,28 +547,44 @@ bool one_launch(const sfp_batch* b, const Group& g)
 // The most bytes of pre-drawn bead normals the FP64 cluster path keeps.
 constexpr size_t kNoiseStepBytes = (size_t)32 << 20;
 
-// Launch k_chain_cluster<G> (clusters of G CTAs, one per chain) for k steps.
-template <int G>
-cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, size_t smem, double c12, double w0cm, int k)
+// The FP64 cluster kernel for clusters of G CTAs: the one with its tables in shared memory
+// where they fit (352 beads on 16 CTAs, 256 on 8).
+using ChainClusterFn = decltype(&sfp::k_chain_cluster<16>);
+ChainClusterFn chain_cluster_kernel(int M, int G, size_t* smem)
 {
+    const bool tab = sfp::chain_cluster_bytes(M, G) <= 224 * 1024;
+    *smem = tab ? sfp::chain_cluster_bytes(M, G) : (size_t)9 * M * sizeof(double);
+    return G == 16 ? (tab ? sfp::k_chain_cluster<16> : sfp::k_chain_cluster_wide<16>)
+                   : (tab ? sfp::k_chain_cluster<8> : sfp::k_chain_cluster_wide<8>);
+}
+void chain_cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int G, int C, size_t smem, cudaStream_t stream)
+{
+    *cfg = {};
+    cfg->gridDim = dim3((unsigned)(G * C));
+    cfg->blockDim = dim3(128);
+    cfg->dynamicSmemBytes = smem;
+    cfg->stream = stream;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = G;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+
+// Launch it (a cluster per chain) for k steps.
+cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, double w0cm, int k)
+{
+    size_t smem = 0;
+    const ChainClusterFn fn = chain_cluster_kernel(g.M, G, &smem);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(sfp::k_chain_cluster<G>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(G * g.C));
-    cfg.blockDim = dim3(128);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = b->cur;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = G;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, sfp::k_chain_cluster<G>, (double*)g.R, g.com, g.step,
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    chain_cluster_config(&cfg, &at, G, g.C, smem, b->cur);
+    return cudaLaunchKernelEx(&cfg, fn, (double*)g.R, g.com, g.step,
                               (const int64_t*)(g.limited ? g.stop : nullptr), (const double*)g.shear,
                               (const double*)g.chiT, (const double*)g.chi, (const double*)g.phi_d,
                               (const double*)g.dm, (const double*)g.h, (const double*)g.w, (const double*)g.g, g.C,
@@ -579,27 +595,19 @@ cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, size_t smem, double c12
 // CTAs per chain for the FP64 cluster path: 16 (a non-portable cluster size)
 // when the GPU can place such clusters for this shape, else 8; 0 when the
 // batch has too many chains for one cluster each.
-int chain_cluster_size(const Group& g, size_t smem, int sms)
+int chain_cluster_size(const Group& g, int sms)
 {
+    size_t smem = 0;
+    const ChainClusterFn fn = chain_cluster_kernel(g.M, 16, &smem);
     if ((int64_t)g.C * 16 <= sms &&
-        cudaFuncSetAttribute(sfp::k_chain_cluster<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-            cudaSuccess &&
-        (smem <= 48 * 1024 || cudaFuncSetAttribute(sfp::k_chain_cluster<16>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                                  cudaSuccess)) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(16u * (unsigned)g.C);
-        cfg.blockDim = dim3(128);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 16;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
+        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        (smem <= 48 * 1024 ||
+         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        chain_cluster_config(&cfg, &at, 16, g.C, smem, nullptr);
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, sfp::k_chain_cluster<16>, &cfg) == cudaSuccess && n >= 1) return 16;
+        if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) return 16;
         cudaGetLastError();
     }
     return (int64_t)g.C * 8 <= sms ? 8 : 0;
@@ -620,7 +628,7 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
     // few chains: a cluster of CTAs per chain, so that each chain uses several SMs;
     // the bead normals of up to kNoiseStepBytes of steps are drawn beforehand in
     // one kernel (the buffer is allocated on first use, outside stream capture)
-    if (g.chain_g < 0) g.chain_g = chain_cluster_size(g, smem, sms);
+    if (g.chain_g < 0) g.chain_g = chain_cluster_size(g, sms);
     const int G = g.chain_g;
     bool cluster = G > 0;
     if (cluster && !g.znoise) {
@@ -641,8 +649,7 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
             sfp::k_noise_steps<<<nblk((int64_t)k * g.C * K, 256), 256, 0, b->cur>>>(
                 g.znoise, g.C, g.M, b->seed, g.job, g.step, k, b->noise == SFP_NOISE_MODES ? 2u : 0u);
             CUDA_TRY(cudaGetLastError());
-            CUDA_TRY(G == 16 ? launch_chain_cluster<16>(b, g, smem, c12, w0cm, k)
-                             : launch_chain_cluster<8>(b, g, smem, c12, w0cm, k));
+            CUDA_TRY(launch_chain_cluster(b, g, G, c12, w0cm, k));
             b->launches += 2;
             done += k;
         }
@@ -1370,7 +1377,7 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
             e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) { destroy_impl(b); return fail(SFP_ECUDA, "create: %s", cudaGetErrorString(e)); }
-            g.chain_g = chain_cluster_size(g, (size_t)9 * M * sizeof(double), sms);
+            g.chain_g = chain_cluster_size(g, sms);
             if (g.chain_g > 0) {
                 const size_t per_step = (size_t)g.C * 3 * M * sizeof(double);
                 g.znoise_steps = (int)std::max<size_t>(1, std::min<size_t>(1024, kNoiseStepBytes / per_step));

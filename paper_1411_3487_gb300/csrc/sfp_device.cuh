@@ -183,6 +183,20 @@ __device__ __forceinline__ void bead_quad_normals(uint32_t seed, uint32_t job, i
 
 template <typename T> __device__ __forceinline__ T rsqrt_t(T x);
 template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
+// FP64: the FP32 approximation y (22 bits) and one cubic step, y + y e (1/2 + 3/8 e) with
+// e = 1 - x y^2 (the binomial series of (1 - e)^(-1/2), its next term below 2^-63): five
+// FP64 instructions, conversions by the bits.  Out of the range of an FP32 seed, and for
+// zeros, infinities and NaN, CUDA's own.
+template <> __device__ __forceinline__ double rsqrt_t<double>(double x)
+{
+    const int hi = __double2hiint(x);
+    if ((unsigned)(hi - 0x3C300000) >= 0x07800000u) return rsqrt(x);       // 2^-60 <= x < 2^60
+    float f = __uint_as_float(((unsigned)(hi - 0x38000000) << 3) | ((unsigned)__double2loint(x) >> 29));
+    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(f));
+    const unsigned b = __float_as_uint(f);
+    const double y = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
 }  // namespace sfp

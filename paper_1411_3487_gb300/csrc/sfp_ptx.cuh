@@ -306,7 +306,7 @@ __device__ __forceinline__ void mma_commit_mc(uint64_t* bar, uint16_t cta_mask)
 // the other CTA of the cluster arrives on.
 __device__ __forceinline__ bool mbar_wait_cl(uint64_t* bar, uint32_t parity, int* err, volatile int* abort_flag)
 {
-    const uint64_t t0 = globaltimer();
+    uint64_t t0 = 0;
     for (;;) {
         uint32_t done;
         asm volatile(
@@ -318,6 +318,7 @@ __device__ __forceinline__ bool mbar_wait_cl(uint64_t* bar, uint32_t parity, int
             : "memory");
         if (done) return true;
         if (*abort_flag) return false;
+        if (t0 == 0) t0 = globaltimer();
         if (globaltimer() - t0 > kTimeoutNs) {
             atomicOr(err, 2);
             *abort_flag = 1;

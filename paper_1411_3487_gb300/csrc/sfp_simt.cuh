@@ -4,6 +4,7 @@
 // rows of length M (beads n or modes p).  A "row" j = 3*chain + axis.
 #pragma once
 #include "sfp_device.cuh"
+#include "sfp_ptx.cuh"
 
 namespace sfp {
 
@@ -689,43 +690,61 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 // ---------------------------------------------------------------------------
 // The same FP64 step for a few chains, each on a cluster of G CTAs, so that a
 // chain uses the FP64 units of G SMs: CTA r of a chain's cluster owns bonds
-// and modes r S .. r S + S - 1 (S = ceil(M / G)) and keeps full copies of R,
-// v and z in its shared memory; each owner writes its slice into every CTA of
+// and modes r S .. r S + S - 1 (S = ceil(M / G)) and keeps full copies of R
+// and v in its shared memory; each owner writes its slice into every CTA of
 // the cluster (distributed shared memory).  Per step:
-//   owner r:  u_n, v_n of its bonds (Eqs. e5, e11), written to every CTA;
-//             every CTA copies the step's bead normals (Eq. b5), drawn for
-//             all the steps of the launch beforehand by k_noise_steps, from
-//             zpre[s] into its shared memory;
-//   cluster barrier;
-//   owner r:  DeltaH_p, Z_p of its modes (Eqs. e11, c4), the update of R_p
-//             (Eqs. d3, d6, f2, btum; rank 0 the FP64 centre of mass), R_p
-//             written to every CTA;
-//   cluster barrier.
-// Q threads share the sums of one bond or mode (Q a power of 2 within a warp),
-// and the groups are dealt round-robin over the four warps: GB300 issues FP64
-// arithmetic at a small fraction of the FP32 rate on each SM sub-partition, so
-// the work must reach all four of them.  The FP64 Box-Muller of a Philox call
-// is a long dependent chain there (~5 us), so the normals come from a separate
-// kernel that draws every call of every step at once.  Every CTA
-// of a cluster runs the same number of steps (one chain), so the hardware
-// cluster barriers always meet.
+//   owner r:  u_n, v_n of its bonds (Eqs. e5, e11) to every CTA; while they travel,
+//             Z_p of its modes (Eq. c4) from the step's bead normals (Eq. b5), drawn
+//             for all the steps of the launch beforehand by k_noise_steps;
+//   owner r:  DeltaH_p of its modes (Eq. e11), the update of R_p (Eqs. d3, d6,
+//             f2, btum; rank 0 the FP64 centre of mass), R_p to every CTA.
+// A value is an asynchronous store that counts its bytes on the reader's mbarrier, so
+// that a hand-over is one way through the cluster, without a fence or a barrier of all
+// its threads.  A CTA sends its part of one array only after all of the other has
+// arrived, which every warp of every CTA sends after its last read: neither array is
+// overwritten while it is read.
+// What bounds it is latency, and most of that FP64 issue: a sub-partition of the SM takes
+// about 60 cycles per FP64 warp instruction.  So a warp takes a bond or mode at a time, its
+// lanes 8 a + j the sums of axis a, every eighth term each: one addition per step of the
+// reduction instead of three, DeltaH_p and Z_p in one; the tables lie in shared memory,
+// and the normals of the next step come in beside this one.
+// The FP64 Box-Muller of a Philox call is a long dependent chain (~5 us), so the
+// normals come from a separate kernel that draws every call of every step at once.
+// One chain, us a step (cluster barriers, tables and normals from L2 before -> here): 64
+// beads 6.6 -> 3.1, 128 11.8 -> 7.5, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
+// Every wait is bounded; after a timeout the CTA raises bit 1 of the error word, and its
+// threads run through the remaining steps without sending anything.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_cta_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
 __device__ __forceinline__ void cluster_barrier()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// *p in the shared memory of CTA `rank` of the cluster (p: this CTA's own copy).
-__device__ __forceinline__ void st_peer(const double* p, uint32_t rank, double v)
+// *p in the shared memory of CTA `rank` of the cluster (p: this CTA's own copy), counted on
+// that CTA's mbarrier `bar`.
+__device__ __forceinline__ void st_peer(const double* p, uint32_t rank, double v, uint64_t* bar)
 {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+                 ::"r"(ptx::mapa(ptx::smem_u32(p), rank)), "l"(__double_as_longlong(v)),
+                 "r"(ptx::mapa(ptx::smem_u32(bar), rank)) : "memory");
+}
+__device__ __forceinline__ void copy_async8(double* dst, const double* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ptx::smem_u32(dst)), "l"(src) : "memory");
+}
+// Sum over the lanes 8 a .. 8 a + 7 of an axis.
+__device__ __forceinline__ double sum8(double x)
+{
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Shared memory of a CTA: R and v ([3][M + 8]: the axes in different banks), the normals
+// of two steps, the tables of the owned bonds and modes and their dm, g, h, w.
+constexpr size_t chain_cluster_bytes(int M, int G)
+{
+    const size_t S = (size_t)(M + G - 1) / G;
+    return 8 * (12 * (size_t)(M + 8) + S * (3 * (size_t)M + 4));
 }
 
 template <int G>
@@ -738,11 +757,179 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 int mode_noise, int* __restrict__ bad)
 {
     extern __shared__ unsigned char chain_smem[];
+    const int P = M + 8;
+    double* sR = reinterpret_cast<double*>(chain_smem);   // [3][P]
+    double* sv = sR + 3 * P;                              // [3][P]
+    double* sz = sv + 3 * P;                              // [2][3][P]
+    double* tab = sz + 6 * P;                             // [S][3][M] chi_n, chi_p, phi_p; [S] dm, g, h, w (w0_cm)
+    __shared__ uint64_t v_in, r_in;                       // v, R of every CTA have arrived (1 + tx)
+    __shared__ int s_abort;
+    const uint32_t rank = ptx::cluster_rank();
+    const int c = blockIdx.x / G;                         // the cluster's chain (c < C: grid = G C)
+    const int S = (M + G - 1) / G;
+    const int lo = min(M, (int)rank * S), hi = min(M, lo + S), nown = hi - lo;
+    const int nwarp = (int)blockDim.x / 32, wid = (int)threadIdx.x / 32, lane = (int)threadIdx.x % 32;
+    const int j = lane & 7, ax = min(lane >> 3, 2);
+    const bool sends = lane < 24;
+    // every warp runs the same passes over the owned bonds / modes
+    const int passes = (nown + nwarp - 1) / nwarp;
+    double* tdm = tab + (size_t)S * 3 * M;
+    double *tg = tdm + S, *th = tg + S, *tw = th + S;
+    double* Rc = Rg + (size_t)c * 3 * M;
+    for (int i = threadIdx.x; i < 3 * M; i += blockDim.x) sR[i / M * P + i % M] = Rc[i];
+    // all copies under way at once (a call of one step of 12 chains of 256 beads: 74 us, 86
+    // with loads through registers); phi by columns: a bead's owned modes lie side by side
+    for (int o = wid; o < nown; o += nwarp)
+        for (int k = lane; k < M; k += 32) {
+            copy_async8(tab + (size_t)o * 3 * M + k, chi + (size_t)(lo + o) * M + k);
+            copy_async8(tab + (size_t)(o * 3 + 1) * M + k, chiT + (size_t)(lo + o) * M + k);
+        }
+    for (int i = threadIdx.x, o = i % max(nown, 1), k = i / max(nown, 1); i < nown * M; i += blockDim.x) {
+        copy_async8(tab + (size_t)(o * 3 + 2) * M + k, phi + (size_t)k * M + lo + o);
+        o += (int)blockDim.x;
+        k += o / nown;
+        o %= nown;
+    }
+    for (int i = threadIdx.x; i < nown; i += blockDim.x) {
+        tdm[i] = dm[lo + i];
+        tg[i] = g[lo + i];
+        th[i] = h[lo + i];
+        tw[i] = lo + i ? w[lo + i] : w0_cm;
+    }
+    double cm = com[3 * c + ax];        // the centre of mass of this lane's axis (rank 0, warp 0)
+    const double sh = shear[c];
+    const int64_t st0 = step[c];
+    const int64_t lim = stop ? stop[c] : INT64_MAX;
+    bool fin = true, ok = true;
+    if (threadIdx.x == 0) {
+        ptx::mbar_init(&v_in, 1);
+        ptx::mbar_init(&r_in, 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));
+        ptx::mbar_expect_tx(&r_in, (uint32_t)(24 * (M - 1)));
+    }
+    auto fetch_z = [&](int s) {
+        if (s < n_steps) {
+            const double* src = zpre + ((size_t)s * C + c) * 3 * M;
+            for (int i = threadIdx.x; i < 3 * M; i += blockDim.x) copy_async8(sz + (s & 1) * 3 * P + i / M * P + i % M, src + i);
+        }
+    };
+    fetch_z(0);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // every CTA of the cluster runs (and has loaded R) before any remote write
+    cluster_barrier();
+    int s = 0;
+    for (; s < n_steps && st0 + s < lim; ++s) {
+        for (int pass = 0; pass < passes; ++pass) {
+            const int gi = pass * nwarp + wid;
+            if (gi >= nown) break;                      // the whole warp
+            const int n = lo + gi;
+            const double* t = tab + (size_t)gi * 3 * M;
+            double u = 0.0;
+#pragma unroll 8
+            for (int p = j; p < M; p += 8) u = fma(t[p], sR[ax * P + p], u);       // chi_{n,0} = 0
+            u = sum8(u);
+            const double u0 = __shfl_sync(0xffffffffu, u, 0), u1 = __shfl_sync(0xffffffffu, u, 8),
+                         u2 = __shfl_sync(0xffffffffu, u, 16);
+            const double l2 = fma(u0, u0, fma(u1, u1, u2 * u2));
+            const double v = n >= 1 ? u * (rsqrt_t<double>(l2) - c12nu) : 0.0;
+            if (sends && ok)
+#pragma unroll
+                for (int r = j; r < G; r += 8) st_peer(&sv[ax * P + n], (uint32_t)r, v, &v_in);
+        }
+        const double* z = sz + (s & 1) * 3 * P;
+        // this lane's part of w_p Z_p (w0_cm Z_0) of an owned mode
+        auto noise = [&](int gi) {
+            const int p = lo + gi;
+            double x = 0.0;
+            if (mode_noise) {
+                if (j == 0) x = z[ax * P + p];
+            } else {
+                const double* t = tab + ((size_t)gi * 3 + 2) * M;
+#pragma unroll 8
+                for (int n = j; n < M; n += 8) x = fma(t[n], z[ax * P + n], x);
+            }
+            return tw[gi] * x;
+        };
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();        // also: every warp is done with the normals of the last step
+        fetch_z(s + 1);
+        double x0 = wid < nown ? noise(wid) : 0.0;
+        ok = ok && ptx::mbar_wait_cl(&v_in, s & 1, bad, &s_abort);
+        if (threadIdx.x == 0) ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));
+        __syncwarp();
+        for (int pass = 0; pass < passes; ++pass) {
+            const int gi = pass * nwarp + wid;
+            if (gi >= nown) break;
+            const int p = lo + gi;
+            const double* t = tab + ((size_t)gi * 3 + 1) * M;
+            double d = 0.0;
+#pragma unroll 8
+            for (int n = j; n < M; n += 8) d = fma(t[n], sv[ax * P + n], d);
+            d = sum8(fma(th[gi], d, pass == 0 ? x0 : noise(gi)));
+            if (p == 0) {
+                // centre of mass (zeta_0 = 0, Eq. d6 limit; w0_cm = w_0 / sqrt(M)), shear on x
+                const double ycm = __shfl_sync(0xffffffffu, cm, 8);
+                cm += d;
+                if (ax == 0) cm = fma(sh * dtau, ycm, cm);
+            } else {
+                const double r = sR[ax * P + p];
+                double o = r + fma(-tdm[gi], r, d);
+                if (sh != 0.0 && ax == 0) o = fma(sh * tg[gi], sR[P + p], o);
+                fin = fin && isfinite(o);
+                if (sends && ok)
+#pragma unroll
+                    for (int q = j; q < G; q += 8) st_peer(&sR[ax * P + p], (uint32_t)q, o, &r_in);
+            }
+        }
+        ok = ok && ptx::mbar_wait_cl(&r_in, s & 1, bad, &s_abort);
+        if (threadIdx.x == 0) ptx::mbar_expect_tx(&r_in, (uint32_t)(24 * (M - 1)));
+        __syncwarp();
+    }
+    // each CTA writes back its own modes; rank 0 the centre of mass and the counter
+    for (int i = threadIdx.x; i < 3 * nown; i += blockDim.x) {
+        const int a = i / nown, p = lo + i % nown;
+        Rc[a * M + p] = p == 0 ? 0.0 : sR[a * P + p];
+    }
+    if (rank == 0 && wid == 0 && sends && j == 0) com[3 * c + ax] = cm;
+    if (rank == 0 && threadIdx.x == 0) step[c] = st0 + s;
+    if (!fin) atomicOr(bad, 1);
+    // nobody leaves while another CTA may still write into its shared memory
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    cluster_barrier();
+}
+
+// The cluster step of chains whose tables no CTA's shared memory holds (more than 352
+// beads on 16 CTAs): bound by FP64 issue and by the tables from L2 rather than by
+// latency.  Q threads share the sums of one bond or mode, all three axes (Q a power of 2
+// within a warp; neighbouring groups read neighbouring table entries), and the groups are
+// dealt round-robin over the four warps, so that all four sub-partitions have FP64 work;
+// plain stores to the other CTAs and a cluster barrier after each array.  (512 beads: 99
+// us a step; with the lanes and hand-overs of k_chain_cluster, tables from L2, 121.)
+// *p in the shared memory of CTA `rank` of the cluster (p: this CTA's own copy).
+__device__ __forceinline__ void st_peer_wait(const double* p, uint32_t rank, double v)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+template <int G>
+__global__ void __launch_bounds__(128)
+k_chain_cluster_wide(double* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict__ step,
+                const int64_t* __restrict__ stop, const double* __restrict__ shear, const double* __restrict__ chiT,
+                const double* __restrict__ chi, const double* __restrict__ phi, const double* __restrict__ dm,
+                const double* __restrict__ h, const double* __restrict__ w, const double* __restrict__ g, int C,
+                int M, double c12nu, double w0_cm, double dtau, int n_steps, const double* __restrict__ zpre,
+                int mode_noise, int* __restrict__ bad)
+{
+    extern __shared__ unsigned char chain_smem[];
     double* sR = reinterpret_cast<double*>(chain_smem);   // [3][M]
     double* sv = sR + 3 * M;                              // [3][M]
     double* sz = sv + 3 * M;                              // [3][M]
     __shared__ double s_cm[3];
-    const uint32_t rank = cluster_cta_rank();
+    const uint32_t rank = ptx::cluster_rank();
     const int c = blockIdx.x / G;                         // the cluster's chain (c < C: grid = G C)
     const int S = (M + G - 1) / G;
     const int lo = min(M, (int)rank * S), hi = min(M, lo + S), nown = hi - lo;
@@ -786,7 +973,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             double vv[3];
             residual_v<double>(uu, n >= 1, c12nu, vv);
             for (int r = j; act && r < G; r += Q)
-                for (int a = 0; a < 3; ++a) st_peer(&sv[a * M + n], (uint32_t)r, vv[a]);
+                for (int a = 0; a < 3; ++a) st_peer_wait(&sv[a * M + n], (uint32_t)r, vv[a]);
         }
         cluster_barrier();
         for (int pass = 0; pass < passes; ++pass) {
@@ -839,9 +1026,9 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 if (sh != 0.0) o0 += sh * g[p] * r1;
                 fin = fin && isfinite(o0) && isfinite(o1) && isfinite(o2);
                 for (int r = j; r < G; r += Q) {
-                    st_peer(&sR[p], (uint32_t)r, o0);
-                    st_peer(&sR[M + p], (uint32_t)r, o1);
-                    st_peer(&sR[2 * M + p], (uint32_t)r, o2);
+                    st_peer_wait(&sR[p], (uint32_t)r, o0);
+                    st_peer_wait(&sR[M + p], (uint32_t)r, o1);
+                    st_peer_wait(&sR[2 * M + p], (uint32_t)r, o2);
                 }
             }
         }
