@@ -1342,8 +1342,12 @@ namespace sfp {
 // so the windows of L and u_m give their time autocorrelations.  Windows and
 // snapshots are [c][kMaxLags][...] whatever lag.n is; win[v] and snp[v] hold
 // vector v = 0 (centre of mass), 1 (middle bead), 2 (L), 3 (u_m).
+// Bound by FP64 issue (about 60 cycles a warp instruction on a sub-partition), not by the
+// 48 bytes a mode: so the warp's sums are folded rather than each summed over all
+// lanes (12 additions, not 45) and a lane takes one vector and lag instead of lane 0 all of
+// them (4096 chains of 64 beads, 400 steps with 20 samples: 1.84 -> 1.48 ms).
 // ---------------------------------------------------------------------------
-constexpr int kMaxLags = 8;
+constexpr int kMaxLags = 8;         // lanes per vector of k_sample
 struct SampleLags {
     int n;
     int v[kMaxLags];
@@ -1362,10 +1366,10 @@ k_sample(const T* __restrict__ R, const double* __restrict__ com, const double* 
 {
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (c >= C) return;
+    if (c >= C) return;                 // the whole warp
     const T* Rc = R + (size_t)c * 3 * M;
     double* pw = power + (size_t)c * 3 * M;
-    double s[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    double s[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};      // L, u_m, r_m' - r_cm
     const double sqM = sqrt((double)M);
     for (int p = lane; p < M; p += 32) {
         const double cl = tab[p], cu = tab[M + p], cd = tab[2 * M + p];
@@ -1379,38 +1383,49 @@ k_sample(const T* __restrict__ R, const double* __restrict__ com, const double* 
             pw[(size_t)a * M + p] += xp * xp;
         }
     }
+    // sums over the warp: at each distance a lane keeps half of its values and hands the
+    // others over (5, 3, 2, 1 of 9, then the last pair): 12 additions
+    double k5[5], k3[3], k2[2];
+    auto fold = [&](bool hi, double lower, double upper, int o) {
+        return (hi ? upper : lower) + __shfl_xor_sync(0xffffffffu, hi ? lower : upper, o);
+    };
 #pragma unroll
-    for (int i = 0; i < 9; ++i)
+    for (int i = 0; i < 5; ++i) k5[i] = fold(lane & 16, s[i], i < 4 ? s[5 + i] : 0.0, 16);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
-    if (lane != 0) return;
-    double* sh = shape + 4 * (size_t)c;
-    sh[0] += s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
-    sh[1] += s[3] * s[3] + s[4] * s[4] + s[5] * s[5];
-    sh[2] += s[6] * s[6] + s[7] * s[7] + s[8] * s[8];
-    sh[3] += 1.0;
-    const double x[4][3] = {{com[3 * c], com[3 * c + 1], com[3 * c + 2]}, {s[6], s[7], s[8]},
-                            {s[0], s[1], s[2]}, {s[3], s[4], s[5]}};
-    for (int i = 0; i < lag.n && i < kMaxLags; ++i) {
-        if (lag.v[i] <= 0 || k % lag.v[i] != 0) continue;
-        const size_t w = (size_t)c * kMaxLags + i;
+    for (int i = 0; i < 3; ++i) k3[i] = fold(lane & 8, k5[i], i < 2 ? k5[3 + i] : 0.0, 8);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            double* sn = wv.snp[v] + w * 3;
-            if (k > 0) {
-                double d2 = 0.0;
+    for (int i = 0; i < 2; ++i) k2[i] = fold(lane & 4, k3[i], i < 1 ? k3[2] : 0.0, 4);
+    double t = fold(lane & 2, k2[0], k2[1], 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    // lane 8 v + i: vector v and lag i; the lanes that hold the sums of v
+    const int v = lane >> 3, i = lane & 7;
+    double x[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const double d = x[v][a] - sn[a];
-                    d2 += d * d;
-                }
-                wv.win[v][w * 2] += d2;
-                wv.win[v][w * 2 + 1] += 1.0;
-            }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) sn[a] = x[v][a];
-        }
+    for (int a = 0; a < 3; ++a) {
+        constexpr int kAt[9] = {0, 2, 4, 8, 10, 16, 18, 20, 24};
+        const int at = v == 1 ? kAt[6 + a] : v == 2 ? kAt[a] : kAt[3 + a];
+        x[a] = __shfl_sync(0xffffffffu, t, at);
+        if (v == 0) x[a] = com[3 * c + a];
     }
+    if (i == 0) {
+        double* sh = shape + 4 * (size_t)c + (v == 0 ? 3 : v == 1 ? 2 : v - 2);
+        *sh += v == 0 ? 1.0 : x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
+    }
+    if (i >= lag.n || lag.v[i] <= 0 || k % lag.v[i] != 0) return;
+    const size_t w = (size_t)c * kMaxLags + i;
+    double* sn = wv.snp[v] + w * 3;
+    if (k > 0) {
+        double d2 = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double d = x[a] - sn[a];
+            d2 += d * d;
+        }
+        wv.win[v][w * 2] += d2;
+        wv.win[v][w * 2 + 1] += 1.0;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) sn[a] = x[a];
 }
 
 }  // namespace sfp
