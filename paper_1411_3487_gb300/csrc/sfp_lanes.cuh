@@ -96,10 +96,11 @@ struct Geo {
     static constexpr int BLK = NP * KP / 16;            // table blocks of one contraction
     static constexpr int BLK_STEP = 3 * BLK;            // ... of a step (streamed)
     static constexpr int BLK_TAB = kScaled ? 2 * BLK : 3 * BLK;   // ... in the table image (of one CTA of a pair)
-    // blocks in shared memory: all, or a ring; a ring slot always serves the same
-    // accumulator, whose MMA warp so sees every phase of its barrier
+    // blocks in shared memory: all, or a ring, whose slots hold the blocks of both
+    // accumulators for the same K indices, one copy of 16 KB
     static constexpr int ST = kPair ? 8 : kStream ? 10 : BLK_TAB;
-    static_assert(!kStream || ST % NP == 0, "ring slots per accumulator");
+    static constexpr int SLOTS = ST / NP;
+    static_assert(!kStream || ST % NP == 0, "whole slots");
     static constexpr int PAR = kPair ? 1 : NP;          // parities whose operands this CTA holds
     // operand X: rows-major (MN-major) core matrices, [GROUPS][KP / 8]
     static constexpr int XSBO = KP * 16, XPART = GROUPS * XSBO, XB = PAR * 2 * XPART;
@@ -225,8 +226,8 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
     float* s_d0 = (float*)(misc + 768);             // [3][32] noise increments of the centre of mass
     uint64_t* bars = (uint64_t*)(misc + 1152);
     float* s_shf = (float*)(misc + 1456);           // [32]
-    uint64_t* full = bars;              // ring slot: table block landed (1 + tx)
-    uint64_t* empty = bars + 12;        // ... MMAs done with it (commit)
+    uint64_t* full = bars;              // ring slot: table blocks landed (1 + tx)
+    uint64_t* empty = bars + 12;        // ... MMAs done with it (a commit per accumulator)
     uint64_t* tab_full = bars + 24;     // resident tables landed
     uint64_t* r_ready = bars + 25;      // operand X holds the modes, D_inc has been read (every work warp)
     uint64_t* v_ready = bars + 26;      // operand X holds the bond forces (every work warp; warp 19: s_d0 has been read; pair: + tx)
@@ -247,9 +248,9 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
 
     if (threadIdx.x == 0) {
         if constexpr (G::kStream)
-            for (int s = 0; s < G::ST; ++s) {
+            for (int s = 0; s < G::SLOTS; ++s) {
                 mbar_init(&full[s], 1);
-                mbar_init(&empty[s], 1);
+                mbar_init(&empty[s], NP);
             }
         mbar_init(tab_full, 1);
         mbar_init(r_ready, kWork);
@@ -294,7 +295,8 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         // see the MMA issuer)
         const bool leader = elect_one();
         if constexpr (G::kStream) {
-            const int total = a.n_steps * G::BLK_STEP;
+            constexpr int STEP = G::BLK_STEP / NP, ONE = G::BLK / NP;     // slots of a step, of a contraction
+            const int total = a.n_steps * STEP;
             bool ok = true;
             int s = 0, src = 0;
             uint32_t phase = 1;
@@ -303,21 +305,21 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], phase, a.err, abort_flag));
                 if (!ok) break;
                 if (leader) {
-                    mbar_expect_tx(&full[s], kBlkBytes);
+                    mbar_expect_tx(&full[s], NP * kBlkBytes);
                     // a pair's step takes the second half of w phi after h chi
-                    const int k = !G::kPair || src < 3 * G::BLK / 2 ? src : src < 5 * G::BLK / 2 ? src + G::BLK / 2 : src - G::BLK;
-                    bulk_load(tabs + s * kBlkBytes, tab + k * kBlkBytes, kBlkBytes, &full[s]);
+                    const int k = !G::kPair || src < 3 * ONE / 2 ? src : src < 5 * ONE / 2 ? src + ONE / 2 : src - ONE;
+                    bulk_load(tabs + s * (NP * kBlkBytes), tab + k * (NP * kBlkBytes), NP * kBlkBytes, &full[s]);
                 }
-                if (++src == G::BLK_STEP) src = 0;
-                if (++s == G::ST) {
+                if (++src == STEP) src = 0;
+                if (++s == G::SLOTS) {
                     s = 0;
                     phase ^= 1u;
                 }
             }
             // the last commit of every ring slot has landed before the tile ends
-            for (int k = 0; k < G::ST && k < total && ok; ++k) {
-                const int last = k + G::ST * ((total - 1 - k) / G::ST);
-                ok = mbar_wait(&empty[k], (last / G::ST) & 1, a.err, abort_flag);
+            for (int k = 0; k < G::SLOTS && k < total && ok; ++k) {
+                const int last = k + G::SLOTS * ((total - 1 - k) / G::SLOTS);
+                ok = mbar_wait(&empty[k], (last / G::SLOTS) & 1, a.err, abort_flag);
             }
         } else {
             if (leader) {
@@ -354,14 +356,14 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         const int ep = G::kPair ? 0 : e;                // operands: of this parity, or of the CTA's
         const uint32_t z_bytes = (uint32_t)(G::ZK * 12 * Ct);       // a chunk of the other CTA: K x 3 axes x (hi, lo)
         const uint64_t x0 = ndesc(smem_u32(X) + ep * 2 * G::XPART, 128, G::XSBO), z0 = ndesc(smem_u32(Z) + ep * 2 * G::ZPART, G::ZLBO, 128);
-        int slot = e;                                   // ring slot and phase of this parity's next streamed block
+        int slot = 0;                                   // ring slot and phase of the next streamed block
         uint32_t phase = 0;
         // the three MMAs of a block, table hi/lo x operand hi/lo; b: the operand's hi
         // part (the lo part b_lo further)
         auto block = [&](int resident, uint32_t d, uint64_t b, uint32_t b_lo, uint32_t idesc, bool first) {
-            const int s = G::kStream ? slot : resident;
+            const int s = G::kStream ? NP * slot + e : resident;
             if constexpr (G::kStream) {
-                ok = __all_sync(0xffffffffu, ok && mbar_wait(&full[s], phase, a.err, abort_flag));
+                ok = __all_sync(0xffffffffu, ok && mbar_wait(&full[slot], phase, a.err, abort_flag));
                 fence_after();
             }
             if (leader && ok) {
@@ -369,12 +371,11 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 mma_bf16(d, al, b, idesc, first ? 0u : 1u);
                 mma_bf16(d, ah, bl, idesc, 1u);
                 mma_bf16(d, ah, b, idesc, 1u);
-                if constexpr (G::kStream) mma_commit(&empty[s]);
+                if constexpr (G::kStream) mma_commit(&empty[slot]);
             }
             if constexpr (G::kStream) {
-                slot += NP;                             // the other parity's block lies between
-                if (slot >= G::ST) {
-                    slot -= G::ST;
+                if (++slot == G::SLOTS) {
+                    slot = 0;
                     phase ^= 1u;
                 }
             }
