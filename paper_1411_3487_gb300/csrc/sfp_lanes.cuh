@@ -78,7 +78,7 @@ constexpr int kBlkBytes = 8192;                 // a table block (one K step of 
 constexpr int kALbo = 2048, kASbo = 128;        // table blocks: K-major core matrices
 
 // Rows of N: four chains (batch b = chain / 4 of the tile) hold rows 24 (b / 2) +
-// 8 axis + 4 (b & 1) + chain % 4, so that a thread's four values of an axis are 8
+// 8 axis + 4 (b & 1) + chain % 4 (Geo::pair, Geo::half), so that a thread's four values of an axis are 8
 // contiguous bytes of operand X.
 template <int M>
 struct Geo {
@@ -89,6 +89,13 @@ struct Geo {
     static constexpr int ROWS = kPair ? 80 : 96;        // MMA N at most: chain slots x 3 axes (72 of 80 used)
     static constexpr int GROUPS = kPair ? 9 : 12;       // row groups of 8
     static constexpr int kMaxChains = 8 * GROUPS / 3;
+    // Where batch b's rows lie: rows 24 pair + 8 axis + 4 half + chain.  A pair of CTAs puts
+    // batches 0 | 2 and 1 | 3 side by side, which one warp works on, so that what it
+    // stores in the other CTA is 16 bytes a lane.
+    __device__ static constexpr int pair(int b) { return kPair && b < 4 ? b & 1 : b >> 1; }
+    __device__ static constexpr int half(int b) { return kPair && b < 4 ? b >> 1 : b & 1; }
+    // pairs of batches that n batches take
+    __device__ static constexpr int pairs(int n) { return kPair ? (n <= 1 ? 1 : n <= 4 ? 2 : 3) : (n + 1) >> 1; }
     static constexpr bool kStream = M >= 256;           // tables through a ring, else resident
     static constexpr bool kScaled = M == 128;           // one symmetric table sin(pi n p / M) for both directions
     static constexpr int ZK = kPair ? 64 : 32;          // K of a noise chunk
@@ -121,10 +128,11 @@ struct Geo {
 
 // Stores to the other CTA's shared memory that count as transaction bytes of its
 // mbarrier `bar` (cluster addresses): the writer neither waits for them nor arrives.
-__device__ __forceinline__ void st_peer16(uint32_t addr, const float (&v)[4], uint32_t bar)
+// A warp's 16 bytes a lane side by side take 31 cycles, 8 bytes a lane 16 bytes apart 69.
+__device__ __forceinline__ void st_peer16(uint32_t addr, uint4 v, uint32_t bar)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1,%2,%3,%4}, [%5];"
-                 ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1,%2,%3,%4}, [%5];"
+                 ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void st_peer8(uint32_t addr, uint2 v, uint32_t bar)
 {
@@ -337,7 +345,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         // instructions (a single-lane loop took 740 cycles for the six MMAs of a
         // block, beside 16 busy warps; their run time is 288).
         // N: the rows of the batches in use (24 per two batches), a multiple of 16
-        const uint32_t id_z = idesc_bf16(128, (24 * ((Ct + 7) >> 3) + 15) & ~15);       // B K-major
+        const uint32_t id_z = idesc_bf16(128, (24 * G::pairs((Ct + 3) >> 2) + 15) & ~15);       // B K-major
         const uint32_t id_x = id_z | (1u << 16);                                        // B rows-major
         const bool leader = elect_one();
         bool ok = true;
@@ -438,7 +446,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         auto mode = [&](int e) { return G::kPair ? 2 * (128 * e + j) + (int)rank : NP * j + e; };
         auto xoff = [](int e) { return G::kPair ? e * 128 * 16 : e * 2 * G::XPART; };
         const uint32_t d_u = tmem + ((uint32_t)(32 * q) << 16), d_inc = d_u + NP * G::ROWS;
-        auto col = [](int b) { return 24 * (b >> 1) + 4 * (b & 1); };          // the batch's first row
+        auto col = [](int b) { return 24 * G::pair(b) + 4 * G::half(b); };     // the batch's first row
         uint8_t* xw = X + j * 16;
         const uint32_t xw_peer = G::kPair ? peer(xw) : 0u, u_peer = G::kPair ? peer(U) : 0u;
         const uint32_t v_peer = G::kPair ? peer(v_ready) : 0u, uin_peer = G::kPair ? peer(u_in) : 0u;
@@ -456,7 +464,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             if (lane == 0 && ok) mbar_arrive(bar);
         };
         auto store_x = [&](uint2 hi, uint2 lo, int off, int ax, int b) {
-            uint8_t* w = xw + off + (3 * (b >> 1) + ax) * G::XSBO + (b & 1) * 8;
+            uint8_t* w = xw + off + (3 * G::pair(b) + ax) * G::XSBO + G::half(b) * 8;
             *reinterpret_cast<uint2*>(w) = hi;
             *reinterpret_cast<uint2*>(w + G::XPART) = lo;
         };
@@ -529,7 +537,8 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         };
         // bond vectors -> residual force v (Eq. e11) of a batch, two chains at a time
         // (packed FP32)
-        auto force4 = [&](int b) {
+        // (a pair of CTAs: the other CTA's operand, [hi, lo][axis], into `there`)
+        auto force4 = [&](int b, uint2 (&there)[2][3]) {
             float u[NP][3][4];                  // even and odd part
             if constexpr (G::kPair) {
                 float own[3][4];
@@ -593,13 +602,11 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             }
             if constexpr (G::kPair) {
                 // K index 128 rank + j of both CTAs' operands: this CTA's parity here, the other there
-                const int off = (int)rank * 128 * 16;
 #pragma unroll
                 for (int ax = 0; ax < 3; ++ax) {
-                    store_x(rank ? xh[NP - 1][ax] : xh[0][ax], rank ? xl[NP - 1][ax] : xl[0][ax], off, ax, b);
-                    const uint32_t w = xw_peer + off + (3 * (b >> 1) + ax) * G::XSBO + (b & 1) * 8;
-                    st_peer8(w, rank ? xh[0][ax] : xh[NP - 1][ax], v_peer);
-                    st_peer8(w + G::XPART, rank ? xl[0][ax] : xl[NP - 1][ax], v_peer);
+                    store_x(rank ? xh[NP - 1][ax] : xh[0][ax], rank ? xl[NP - 1][ax] : xl[0][ax], (int)rank * 128 * 16, ax, b);
+                    there[0][ax] = rank ? xh[0][ax] : xh[NP - 1][ax];
+                    there[1][ax] = rank ? xl[0][ax] : xl[NP - 1][ax];
                 }
             } else {
 #pragma unroll
@@ -615,7 +622,10 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             for (int ax = 0; ax < 3; ++ax) tmem_ld4(d_u + (rank ^ 1u) * G::ROWS + 8 * ax + col(b), v[ax]);
             tmem_wait12(v);
 #pragma unroll
-            for (int ax = 0; ax < 3; ++ax) st_peer16(u_peer + ((3 * b + ax) * 128 + j) * 16, v[ax], uin_peer);
+            for (int ax = 0; ax < 3; ++ax)
+                st_peer16(u_peer + ((3 * b + ax) * 128 + j) * 16,
+                          make_uint4(__float_as_uint(v[ax][0]), __float_as_uint(v[ax][1]), __float_as_uint(v[ax][2]),
+                                     __float_as_uint(v[ax][3])), uin_peer);
         };
         // update (Eqs. d3, btum) of a batch whose modes are in r (tm: in TMEM)
         auto update4 = [&](float (&r)[NP][3][4], int b, int sp, bool tm, bool plain) {
@@ -688,8 +698,33 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 for (int b = b0; ok && b < nb; b += bs) send4(b);
                 ok = ok && mbar_wait_cl(u_in, sp & 1, a.err, abort_flag);
             }
+            uint2 there[2][3], held[2][3];
 #pragma unroll 1
-            for (int b = b0; ok && b < nb; b += bs) force4(b);
+            for (int b = b0; ok && b < nb; b += bs) {
+                force4(b, there);
+                if constexpr (G::kPair) {
+                    const uint32_t w = xw_peer + rank * (128 * 16) + 3 * G::pair(b) * G::XSBO;
+                    if (b == b0 && b + bs < nb) {
+                        // goes with the next batch
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int ax = 0; ax < 3; ++ax) held[i][ax] = there[i][ax];
+                    } else if (b == b0 + bs) {
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int ax = 0; ax < 3; ++ax)
+                                st_peer16(w + ax * G::XSBO + i * G::XPART, make_uint4(held[i][ax].x, held[i][ax].y, there[i][ax].x, there[i][ax].y), v_peer);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int ax = 0; ax < 3; ++ax)
+                                st_peer8(w + ax * G::XSBO + i * G::XPART + G::half(b) * 8, there[i][ax], v_peer);
+                    }
+                }
+            }
             arrive(v_ready);
             // a batch whose modes are in global memory is updated last; they come from L2
             // while the forward MMAs run
@@ -805,7 +840,8 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 }
                 if (cl[k] < Ct && ok) {
                     const int b = cl[k] >> 2;
-                    uint8_t* w = Z + buf * G::ZB + ((G::kPair ? 4 * k : 0) + (t >> 1)) * G::ZLBO + 3 * (b >> 1) * 128 + (4 * (b & 1) + (cl[k] & 3)) * 16 + (t & 1) * 8;
+                    uint8_t* w = Z + buf * G::ZB + ((G::kPair ? 4 * k : 0) + (t >> 1)) * G::ZLBO + 3 * G::pair(b) * 128 +
+                                 (4 * G::half(b) + (cl[k] & 3)) * 16 + (t & 1) * 8;
                     if constexpr (G::kPair) {
                         const uint32_t wp = peer(w);
 #pragma unroll
