@@ -24,7 +24,7 @@
 // themselves; at 64 beads lanes 64..127 repeat lanes 0..63, so that all four
 // TMEM lane quarters can work on the tile's chains.
 //
-// Roles (20 warps): warp 0 streams the tables (256 beads: 48 blocks of 8 KB a step
+// Roles (20 warps): warp 0 streams the tables (256 beads: 24 pairs of blocks, 16 KB each, a step
 // through a ring; 64 and 128 beads: resident, loaded once); warp 1 issues the MMAs
 // (256 beads: of the even modes, warp 18 of the odd ones, whose accumulators are
 // others); warps 2..9 (two per TMEM lane quarter) form the force, D_u -> v -> operand
@@ -49,15 +49,15 @@
 // normals are drawn once: each CTA draws every second chunk and writes the sums to the
 // even modes' CTA and the differences to the other.  All of it goes by st.async, which
 // counts bytes on the reader's mbarrier, so that nobody waits for the stores (with plain
-// remote stores and remote arrivals: 197 us a step at 16384 chains instead of 175).  Half
+// remote stores and remote arrivals: 197 us a step at 16384 chains instead of 175 then).  Half
 // of the noise chunks come after the forward MMAs, so that their way between the CTAs
 // passes behind those.  The step is bound by the table stream, 768 KB a CTA from L2, with
 // 64 KB under way in the ring: what both CTAs' operands and buffers leave.
 //
 // Measured (GB300, us a step in a 400-step call, the four-role kernel of sfp_fused.cu
-// before -> here): 4096 x 256 bp 22.7 -> 9.1, 8 x 256 bp 19.1 -> 5.3, 4096 x 128 bp
+// before -> here): 4096 x 256 bp 22.7 -> 8.9, 8 x 256 bp 19.1 -> 5.2, 4096 x 128 bp
 // 10.3 -> 4.3, 50 x 128 bp 9.5 -> 2.7, 4096 x 64 bp 7.3 -> 2.3, 8 x 64 bp 5.9 -> 1.5; 16384 x 512 bp 289 ->
-// 175 (here 1000 x 512 bp take 17.2, one chain 14.0).
+// 130 (here 1000 x 512 bp take 11.8, one chain 10.0).
 #pragma once
 #include <cstdint>
 #include <cuda_bf16.h>
@@ -349,17 +349,20 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         const uint32_t id_x = id_z | (1u << 16);                                        // B rows-major
         const bool leader = elect_one();
         bool ok = true;
-        auto wait = [&](uint64_t* bar, uint32_t parity) {
-            if constexpr (G::kPair) {
+        // peer: the barrier counts stores of the other CTA's threads into this CTA's shared
+        // memory; a proxy fence on this side, for this CTA's shared memory, orders the MMAs
+        // after them (one for every state space took 1200 cycles, six times a step)
+        auto wait = [&](uint64_t* bar, uint32_t parity, bool peer) {
+            if (G::kPair && peer) {
                 ok = __all_sync(0xffffffffu, ok && mbar_wait_cl(bar, parity, a.err, abort_flag));
-                fence_proxy_async_all();        // operands that the other CTA's threads wrote
+                fence_proxy_async();
             } else {
                 ok = __all_sync(0xffffffffu, ok && mbar_wait(bar, parity, a.err, abort_flag));
             }
             fence_after();
         };
-        if (a.stall_test) wait(never, 0);
-        if constexpr (!G::kStream) wait(tab_full, 0);
+        if (a.stall_test) wait(never, 0, false);
+        if constexpr (!G::kStream) wait(tab_full, 0, false);
         const uint64_t tab0 = ndesc(smem_u32(tabs), kALbo, kASbo);
         const int ep = G::kPair ? 0 : e;                // operands: of this parity, or of the CTA's
         const uint32_t z_bytes = (uint32_t)(G::ZK * 12 * Ct);       // a chunk of the other CTA: K x 3 axes x (hi, lo)
@@ -401,7 +404,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         // a noise chunk: its turn of the buffer of its number mod 2
         auto with_z = [&](int sp, int ch) {
             const int b = ch & 1;
-            wait(&n_ready[b], (sp * (G::NCH / 2) + (ch >> 1)) & 1);
+            wait(&n_ready[b], (sp * (G::NCH / 2) + (ch >> 1)) & 1, b != (int)rank);
             if constexpr (G::kPair) {
                 // the other CTA's next chunk (no byte of it comes before both CTAs' MMAs have read this one)
                 if (warp == 1 && leader && ok && b != (int)rank) mbar_expect_tx(&n_ready[b], z_bytes);
@@ -420,12 +423,12 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         }
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps && ok; ++sp) {
-            wait(r_ready, sp & 1);
+            wait(r_ready, sp & 1, false);
             with_x(0, d_u, true);
             if (leader && ok) mma_commit(u_done);
 #pragma unroll 1
             for (int ch = 0; ch < (G::kPair ? 2 : G::NCH); ++ch) with_z(sp, ch);
-            wait(v_ready, sp & 1);
+            wait(v_ready, sp & 1, true);
             with_x(G::kScaled ? 0 : 2 * G::BLK, d_inc, G::kScaled);
             if constexpr (G::kPair) {
                 // the later chunks, whose way between the CTAs passes behind the forward MMAs

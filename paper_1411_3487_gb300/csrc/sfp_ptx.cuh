@@ -243,9 +243,6 @@ __device__ __forceinline__ void tmem_ld8x2(uint32_t ta, uint32_t tb, float (&v)[
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// The same for every memory space (stores to another CTA's shared memory).
-__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
-
 // ---- two-CTA clusters (the fused step's 512-bead variant)
 
 __device__ __forceinline__ uint32_t cluster_rank()
