@@ -33,7 +33,7 @@
 // (kind::tf32) for SFP_FP32, BF16 parts (kind::f16) for SFP_MIXED_BF16.
 // Roles (640 threads):
 //   warp 0       TMA producer: R tiles and chi hi/lo (inverse), F hi/lo (forward)
-//   warp 1       TMEM allocation; one thread issues every MMA and commit
+//   warp 1       TMEM allocation; one elected lane issues every MMA and commit
 //   warps 2..9   compute: split the R tiles into hi/lo, read D_u (two warps per
 //                lane quarter) and write the force blocks, epilogue from D_inc
 //   warps 10..19 noise: Philox / Box-Muller normals written as the noise
@@ -1818,6 +1818,7 @@ k_fused_grouped(const __grid_constant__ GroupedArgs P)
 
 struct FusedPlan {
     int M = 0, C = 0, cpt = kChains;
+    int want = 0;               // chains per tile asked for (0: the default rule)
     bool bf16 = false, two = false;
     void* tab[4] = {nullptr, nullptr, nullptr, nullptr};    // chi_hi, chi_lo, F_hi, F_lo (TF32 or BF16)
     float* R = nullptr;
@@ -1840,7 +1841,21 @@ static int round_tile(int cpt, int most) { return std::min(most, std::max(4, (cp
 // Most chains per tile of a plan's step.
 static int most_chains(const FusedPlan* p)
 {
-    return !p->lane_tab ? kChains : p->M == 512 ? lanes::Geo<512>::kMaxChains : lanes::Geo<256>::kMaxChains;
+    return !p->lane_tab || p->mz ? kChains : p->M == 512 ? lanes::Geo<512>::kMaxChains : lanes::Geo<256>::kMaxChains;
+}
+
+// The fewest waves of tiles of as many chains as the step takes (a 512-bead tile takes
+// two SMs), then the chains spread evenly over the tiles of those waves: chains per tile
+// = ceil(C / (units x waves)) rounded up to a multiple of 4 (fused_set_tile changes it)
+static int default_tile(const FusedPlan* p)
+{
+    const int most = most_chains(p), C = p->C;
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 148;
+    const int units = p->M == 512 ? sms / 2 : sms;
+    const int waves = std::max(1, (C + units * most - 1) / (units * most));
+    return round_tile((C + units * waves - 1) / (units * waves), most);
 }
 
 bool fused_supported(int M) { return M == 64 || M == 128 || M == 256 || M == 512; }
@@ -1987,7 +2002,7 @@ static int classic_tables(FusedPlan* p, const double* chi, const double* phi, co
             void*& d = p->tab[2 * t + k];
             const void* hsrc = bf16 ? (const void*)(k == 0 ? hb.data() : lb.data())
                                     : (const void*)(k == 0 ? hi.data() : lo.data());
-            if (cudaMalloc(&d, cnt[t] * el) != cudaSuccess) return report(SFP_ENOMEM, "fused-step table allocation failed");
+            if (!d && cudaMalloc(&d, cnt[t] * el) != cudaSuccess) return report(SFP_ENOMEM, "fused-step table allocation failed");
             if (cudaMemcpyAsync(d, hsrc, cnt[t] * el, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
                 cudaStreamSynchronize(stream) != cudaSuccess)
                 return report(SFP_ECUDA, "fused-step table upload failed");
@@ -2026,7 +2041,7 @@ static int classic_tables(FusedPlan* p, const double* chi, const double* phi, co
         // w_p with w_0 (the centre of mass) in FP32, for the mode-keyed epilogue
         std::vector<float> wf(M);
         for (int q = 0; q < M; ++q) wf[q] = (float)w[q];
-        e = cudaMalloc((void**)&p->w32, (size_t)M * sizeof(float));
+        if (!p->w32) e = cudaMalloc((void**)&p->w32, (size_t)M * sizeof(float));
         if (e == cudaSuccess) e = cudaMemcpyAsync(p->w32, wf.data(), (size_t)M * sizeof(float), cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     }
@@ -2057,17 +2072,7 @@ int fused_create(FusedPlan** out, int M, int C, const double* chi, const double*
             return rc;
         }
     }
-    // the fewest waves of tiles of as many chains as the step takes (a 512-bead tile
-    // takes two SMs), then the chains spread evenly over the tiles of those waves:
-    // chains per tile = ceil(C / (units x waves)) rounded up to a multiple of 4
-    // (fused_set_tile changes it)
-    const int most = most_chains(p);
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        sms = 148;
-    const int units = M == 512 ? sms / 2 : sms;
-    const int waves = std::max(1, (C + units * most - 1) / (units * most));
-    p->cpt = round_tile((C + units * waves - 1) / (units * waves), most);
+    p->cpt = default_tile(p);
     int rc = SFP_OK;
     if (!p->lane_tab) {
         rc = classic_tables(p, chi, phi, h, w);
@@ -2228,16 +2233,23 @@ size_t fused_bytes(const FusedPlan* p)
            (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0) + p->lane_bytes;
 }
 
-int fused_set_tile(FusedPlan* p, int cpt)
+// The plan's tile and its R map.
+static int retile(FusedPlan* p, int cpt)
 {
-    if (cpt < 1 || cpt > kChains) return report(SFP_EINVAL, "chains per tile must be 1..40");
-    cpt = round_tile(cpt, most_chains(p));
     CUtensorMap m;
     const int rc = make_map_2d(&m, p->R, 3 * p->C, p->M, 3 * (cpt / 4));
     if (rc) return rc;
     p->tmR = m;
     p->cpt = cpt;
     return SFP_OK;
+}
+
+int fused_set_tile(FusedPlan* p, int cpt)
+{
+    if (cpt < 1 || cpt > kChains) return report(SFP_EINVAL, "chains per tile must be 1..40");
+    const int rc = retile(p, round_tile(cpt, most_chains(p)));
+    if (!rc) p->want = cpt;
+    return rc;
 }
 
 bool fused_mode_noise_supported(int M) { return M == 64 || M == 128 || M == 256; }
@@ -2254,8 +2266,12 @@ int fused_set_mode_noise(FusedPlan* p, bool on)
         const size_t bytes = (size_t)2 * p->C * 3 * p->M * sizeof(float);
         if (cudaMalloc((void**)&p->zbuf, bytes) != cudaSuccess) return report(SFP_ENOMEM, "mode-noise buffer allocation failed");
     }
+    if (p->mz == on) return SFP_OK;
+    // the kernels of the two keyings take tiles of different sizes
     p->mz = on;
-    return SFP_OK;
+    const int rc = p->lane_tab ? retile(p, p->want ? round_tile(p->want, most_chains(p)) : default_tile(p)) : SFP_OK;
+    if (rc) p->mz = !on;
+    return rc;
 }
 
 void fused_destroy(FusedPlan* p)

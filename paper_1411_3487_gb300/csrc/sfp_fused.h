@@ -59,7 +59,8 @@ int fused_ctas_per_tile(const FusedPlan* plan);
 size_t fused_bytes(const FusedPlan* plan);
 int fused_set_tile(FusedPlan* plan, int cpt);
 // Mode-keyed noise on (Z drawn per mode, Eq. c4 reading; M <= 256 only: the
-// 512-bead cluster kernel draws bead noise): allocates the plan's Z buffer.
+// 512-bead cluster kernel draws bead noise): allocates the plan's Z buffer and, for the
+// lane step's plans, the tables of the kernel that takes it; tiles are chosen anew.
 int fused_set_mode_noise(FusedPlan* plan, bool on);
 bool fused_mode_noise_supported(int M);
 // True for plans that the grouped launch takes (every fused plan).

@@ -45,3 +45,19 @@ def test_lane_step_of_512_beads_on_two_ctas_matches_fp64(C, n, shear):
     """A tile of up to 24 chains on a cluster of two CTAs, one parity of the modes
     each: bonds are sums over both, normals and forces are shared by both."""
     test_lane_step_matches_fp64(512, C, n, shear)
+
+
+@pytest.mark.parametrize("C", [33, 4865, 6080])
+def test_noise_keyings_by_turns(C):
+    """Bead-, mode- and bead-keyed steps of one batch: each keying's kernel takes tiles of
+    its own size, and the plan comes back to the lane step's."""
+    def steps(precision):
+        with sfp.Batch([{"n_beads": 64, "dtau": DTAU[64], "job_id": c} for c in range(C)], seed=5, precision=precision) as b:
+            b.init_equilibrium()
+            for keying in (sfp.SFP_NOISE_BEADS, sfp.SFP_NOISE_MODES, sfp.SFP_NOISE_BEADS):
+                b.set_noise(keying)
+                b.step(2)
+            return b.modes()
+    got, ref = steps(sfp.SFP_MIXED_BF16), steps(sfp.SFP_FP64)
+    err = np.linalg.norm((got - ref)[:, :, 1:], axis=(1, 2)) / np.linalg.norm(ref[:, :, 1:], axis=(1, 2))
+    assert err.max() < 1e-5, (err.max(), err.argmax())
