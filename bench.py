@@ -343,10 +343,12 @@ def run_native(args, rank, world, local):
             if us_m and precision in (sfp.SFP_MIXED_BF16, sfp.SFP_FP32):
                 peak_m = pk.get("bf16_tflops", 1900.0) if precision == sfp.SFP_MIXED_BF16 else (
                     pk.get("tf32_tflops") or pk.get("bf16_tflops", 1900.0) * 1.1 / 2.25)
-                fl = 3 * 12.0 * M_BEADS * beads      # inverse 2M x 3 + forward force half 2M x 3, three passes
+                # inverse 2M x 3 + forward force half 2M x 3, three passes (TF32: in halves)
+                per = 3 * (12 if precision == sfp.SFP_MIXED_BF16 else 6) * M_BEADS
+                fl = float(per) * beads
                 modes["roofline_tensor"] = {"achieved": fl / (us_m * 1e-6) / 1e12, "peak": peak_m,
                                             "frac": fl / (us_m * 1e-6) / 1e12 / peak_m, "kernel_us": us_m,
-                                            "flops_per_bead_step": 3 * 12 * M_BEADS}
+                                            "flops_per_bead_step": per}
 
     # the mixed-precision workload, 16384 chains x 512 bp at dt 15.9 ps: the fused
     # step (a tile per cluster of two CTAs) with each split, the staged
@@ -384,8 +386,10 @@ def run_native(args, rank, world, local):
             if pth == sfp.SFP_PATH_FUSED:
                 bf = prec in (sfp.SFP_MIXED_BF16, sfp.SFP_MIXED_BF16_2)
                 passes = 2 if prec == sfp.SFP_MIXED_BF16_2 else 3
-                big[name]["kernel"] = "k_fused_pair<%s>" % ({sfp.SFP_MIXED_BF16: "bf16", sfp.SFP_MIXED_BF16_2: "bf16, two passes"}.get(prec, "tf32"))
-                big[name]["roofline_tensor_frac"] = (passes * 18 * 512 * 16384 * 512 / (1e-3 * t_ms / n)) / 1e12 / (
+                big[name]["kernel"] = {sfp.SFP_MIXED_BF16: "k_lane_step<512>",
+                                       sfp.SFP_MIXED_BF16_2: "k_fused_pair<bf16, two passes>"}.get(prec, "k_fused_pair<tf32>")
+                work = 9 if prec == sfp.SFP_MIXED_BF16 else 18      # in the halves of the mirror symmetry, or whole
+                big[name]["roofline_tensor_frac"] = (passes * work * 512 * 16384 * 512 / (1e-3 * t_ms / n)) / 1e12 / (
                     pk["bf16_tflops"] if bf else pk.get("tf32_tflops") or pk["bf16_tflops"] * 1.1 / 2.25)
             elif prec == sfp.SFP_MIXED_BF16:
                 # per-kernel times of the staged step at this size (stage events, noise in line)
@@ -448,8 +452,8 @@ def run_native(args, rank, world, local):
         dist.destroy_process_group()
 
 
-KERNEL_SOURCES = ("paper_1411_3487_gb300/csrc/sfp_fused.cu", "paper_1411_3487_gb300/csrc/sfp_device.cuh",
-                  "paper_1411_3487_gb300/csrc/sfp_ptx.cuh")
+KERNEL_SOURCES = ("paper_1411_3487_gb300/csrc/sfp_fused.cu", "paper_1411_3487_gb300/csrc/sfp_lanes.cuh",
+                  "paper_1411_3487_gb300/csrc/sfp_device.cuh", "paper_1411_3487_gb300/csrc/sfp_ptx.cuh")
 
 
 def kernel_sha() -> str:
@@ -486,8 +490,10 @@ def roofline(kern, pk, how, precision, path, sfp):
     Algorithmic work of the transforms: 18 M flops per bead-step (inverse
     2 M x 3 rows, forward 2 M x 6 rows per chain); the tensor-core kernels
     execute each product as three MMAs (hi/lo split), so the tensor pipe does
-    54 M flops per bead-step, compared with the dense peak of the MMA type
-    (measured BF16; TF32 from it by the nominal 1.1/2.25 ratio)."""
+    54 M flops per bead-step, 27 M in the kernels that take the products in the
+    halves of the mirror symmetry (three-pass BF16 at 256 and 512 beads, TF32 at
+    128 and 256), compared with the dense peak of the MMA type (measured BF16;
+    TF32 from it by the nominal 1.1/2.25 ratio)."""
     if not kern:
         return None
     M, beads = M_BEADS, C_CHAINS * M_BEADS
@@ -507,17 +513,17 @@ def roofline(kern, pk, how, precision, path, sfp):
                 "algorithmic_bytes": 24 * beads, "kernel_us": us, "peak_source": f"{how} bf16 dense (burst)"}
     if precision == sfp.SFP_MIXED_BF16 and path == sfp.SFP_PATH_FUSED:
         us = kern.get("inverse_us")          # the fused kernel is recorded as the first stage
-        flops = 3 * 18.0 * M * beads
+        flops = 3 * 9.0 * M * beads
         peak = pk.get("bf16_tflops", 1900.0)
-        traffic = measured_traffic("fused_step_bf16_4096x256.md", "paper_1411_3487_gb300/csrc/sfp_fused.cu")
-        return {"bound": "tensor", "kernel": "k_fused_step<256, bf16> (whole step, bf16x3)",
+        traffic = measured_traffic("lane_step_bf16_4096x256.md", "paper_1411_3487_gb300/csrc/sfp_lanes.cuh")
+        return {"bound": "tensor", "kernel": "k_lane_step<256> (whole step, bf16x3)",
                 "achieved": flops / (us * 1e-6) / 1e12, "peak": peak, "unit": "TFLOP/s",
                 "frac": flops / (us * 1e-6) / 1e12 / peak, "traffic": traffic,
-                "traffic_unit": "DRAM bytes per launch (ncu, profiles/fused_step_bf16_4096x256.md)",
+                "traffic_unit": "DRAM bytes per launch (ncu, profiles/lane_step_bf16_4096x256.md)",
                 "algorithmic_bytes": 24 * beads, "kernel_us": us, "peak_source": f"{how} bf16 dense (burst)"}
     if precision == sfp.SFP_FP32 and path == sfp.SFP_PATH_FUSED:
         us = kern.get("inverse_us")          # the fused kernel is recorded as the first stage
-        flops = 3 * 18.0 * M * beads
+        flops = 3 * 9.0 * M * beads
         traffic = measured_traffic("fused_step_4096x256.md", "paper_1411_3487_gb300/csrc/sfp_fused.cu")
         return {"bound": "tensor", "kernel": "k_fused_step<256, tf32> (whole step, tf32x3)",
                 "achieved": flops / (us * 1e-6) / 1e12, "peak": tf32_peak, "unit": "TFLOP/s",
