@@ -51,8 +51,9 @@
 // counts bytes on the reader's mbarrier, so that nobody waits for the stores (with plain
 // remote stores and remote arrivals: 197 us a step at 16384 chains instead of 175 then).  Half
 // of the noise chunks come after the forward MMAs, so that their way between the CTAs
-// passes behind those.  The step is bound by the table stream, 768 KB a CTA from L2, with
-// 64 KB under way in the ring: what both CTAs' operands and buffers leave.
+// passes behind those.  The step is bound by its chain, 10 us of 14.5 at 24 chains: inverse
+// and forward MMAs 5 us with their waits for 768 KB of tables (64 KB under way in the
+// ring, what operands and buffers leave), two exchanges, force, update.
 //
 // Measured (GB300, us a step in a 400-step call, the four-role kernel of sfp_fused.cu
 // before -> here): 4096 x 256 bp 22.7 -> 8.9, 8 x 256 bp 19.1 -> 5.2, 4096 x 128 bp
