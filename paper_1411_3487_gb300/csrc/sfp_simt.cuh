@@ -700,9 +700,14 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 //             f2, btum; rank 0 the FP64 centre of mass), R_p to every CTA.
 // A value is an asynchronous store that counts its bytes on the reader's mbarrier, so
 // that a hand-over is one way through the cluster, without a fence or a barrier of all
-// its threads.  A CTA sends its part of one array only after all of the other has
-// arrived, which every warp of every CTA sends after its last read: neither array is
-// overwritten while it is read.
+// its threads.  A warp sends its part of one array only after all of the other has
+// arrived, and every warp that reads an array sends a part of the other after its last
+// read: neither array is overwritten while it is read, and no phase of a barrier begins
+// before the one before it is over for everyone who waits on it.  That needs all of them
+// to own something (M < G S leaves CTAs without bonds or modes, M <= 3 G warps): CTAs
+// that own nothing take no part and are sent nothing, warps that own nothing do not wait.
+// A CTA or warp that waits without being waited for can fall two phases behind, and the
+// bytes of the second then keep the count of the first from ever being zero.
 // What bounds it is latency, and most of that FP64 issue: a sub-partition of the SM takes
 // about 60 cycles per FP64 warp instruction.  So a warp takes a bond or mode at a time, its
 // lanes 8 a + j the sums of axis a, every eighth term each: one addition per step of the
@@ -771,6 +776,8 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     const int nwarp = (int)blockDim.x / 32, wid = (int)threadIdx.x / 32, lane = (int)threadIdx.x % 32;
     const int j = lane & 7, ax = min(lane >> 3, 2);
     const bool sends = lane < 24;
+    const int owners = (M + S - 1) / S;                   // CTAs 0 .. owners - 1 own something
+    const bool owns = wid < nown;                         // this warp does (uniform; warp 0 of every owner)
     // every warp runs the same passes over the owned bonds / modes
     const int passes = (nown + nwarp - 1) / nwarp;
     double* tdm = tab + (size_t)S * 3 * M;
@@ -820,7 +827,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     // every CTA of the cluster runs (and has loaded R) before any remote write
     cluster_barrier();
     int s = 0;
-    for (; s < n_steps && st0 + s < lim; ++s) {
+    for (; nown > 0 && s < n_steps && st0 + s < lim; ++s) {
         for (int pass = 0; pass < passes; ++pass) {
             const int gi = pass * nwarp + wid;
             if (gi >= nown) break;                      // the whole warp
@@ -836,7 +843,8 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             const double v = n >= 1 ? u * (rsqrt_t<double>(l2) - c12nu) : 0.0;
             if (sends && ok)
 #pragma unroll
-                for (int r = j; r < G; r += 8) st_peer(&sv[ax * P + n], (uint32_t)r, v, &v_in);
+                for (int r = j; r < G; r += 8)
+                    if (r < owners) st_peer(&sv[ax * P + n], (uint32_t)r, v, &v_in);
         }
         const double* z = sz + (s & 1) * 3 * P;
         // this lane's part of w_p Z_p (w0_cm Z_0) of an owned mode
@@ -855,8 +863,8 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();        // also: every warp is done with the normals of the last step
         fetch_z(s + 1);
-        double x0 = wid < nown ? noise(wid) : 0.0;
-        ok = ok && ptx::mbar_wait_cl(&v_in, s & 1, bad, &s_abort);
+        double x0 = owns ? noise(wid) : 0.0;
+        if (owns) ok = ok && ptx::mbar_wait_cl(&v_in, s & 1, bad, &s_abort);
         if (threadIdx.x == 0) ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));
         __syncwarp();
         for (int pass = 0; pass < passes; ++pass) {
@@ -865,8 +873,9 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             const int p = lo + gi;
             const double* t = tab + ((size_t)gi * 3 + 1) * M;
             double d = 0.0;
+            if (p > 0)                  // mode 0 takes no force, and nobody waits for its warp's read
 #pragma unroll 8
-            for (int n = j; n < M; n += 8) d = fma(t[n], sv[ax * P + n], d);
+                for (int n = j; n < M; n += 8) d = fma(t[n], sv[ax * P + n], d);
             d = sum8(fma(th[gi], d, pass == 0 ? x0 : noise(gi)));
             if (p == 0) {
                 // centre of mass (zeta_0 = 0, Eq. d6 limit; w0_cm = w_0 / sqrt(M)), shear on x
@@ -880,13 +889,15 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 fin = fin && isfinite(o);
                 if (sends && ok)
 #pragma unroll
-                    for (int q = j; q < G; q += 8) st_peer(&sR[ax * P + p], (uint32_t)q, o, &r_in);
+                    for (int q = j; q < G; q += 8)
+                        if (q < owners) st_peer(&sR[ax * P + p], (uint32_t)q, o, &r_in);
             }
         }
-        ok = ok && ptx::mbar_wait_cl(&r_in, s & 1, bad, &s_abort);
+        if (owns) ok = ok && ptx::mbar_wait_cl(&r_in, s & 1, bad, &s_abort);
         if (threadIdx.x == 0) ptx::mbar_expect_tx(&r_in, (uint32_t)(24 * (M - 1)));
         __syncwarp();
     }
+    __syncthreads();        // the modes that the waiting warps have seen, for the others too
     // each CTA writes back its own modes; rank 0 the centre of mass and the counter
     for (int i = threadIdx.x; i < 3 * nown; i += blockDim.x) {
         const int a = i / nown, p = lo + i % nown;
