@@ -883,10 +883,11 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 cm += d;
                 if (ax == 0) cm = fma(sh * dtau, ycm, cm);
             } else {
-                const double r = sR[ax * P + p];
+                const double r = sR[ax * P + p], ry = sR[P + p];
                 double o = r + fma(-tdm[gi], r, d);
-                if (sh != 0.0 && ax == 0) o = fma(sh * tg[gi], sR[P + p], o);
+                if (sh != 0.0 && ax == 0) o = fma(sh * tg[gi], ry, o);
                 fin = fin && isfinite(o);
+                __syncwarp();       // every lane has read the mode before one of them sends the new one here
                 if (sends && ok)
 #pragma unroll
                     for (int q = j; q < G; q += 8)

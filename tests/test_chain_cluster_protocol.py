@@ -186,3 +186,32 @@ def test_sending_to_ctas_that_own_nothing_is_caught(M, G):
 @pytest.mark.parametrize("M,G", [(3, 8), (20, 16)])
 def test_waits_of_warps_that_own_nothing_are_caught(M, G):
     assert caught(M, G, 40, idle_warps=True) > 0
+
+
+def update_lanes(rng, ordered, shear):
+    """The 24 lanes of a warp that update one mode: lane 8 a + j reads R of its axis (axis 0
+    with shear also that of axis 1); one lane of each axis then stores the new value in this
+    CTA's own copy.  Lanes run in any order after the last shuffle; `ordered`: a warp barrier
+    lies between the reads and the stores.  Returns the axes that a lane read too late."""
+    new, late, order = set(), set(), [(a, j) for a in range(3) for j in range(8)]
+    rng.shuffle(order)
+
+    def read(a):
+        late.update(({a, 1} if shear and a == 0 else {a}) & new)
+
+    if ordered:
+        for a, _ in order:
+            read(a)
+    for a, j in order:
+        if not ordered:
+            read(a)
+        if j == 3:
+            new.add(a)
+    return late
+
+
+@pytest.mark.parametrize("shear", [False, True])
+def test_a_mode_is_read_by_all_lanes_before_it_is_overwritten(shear):
+    for seed in range(20):
+        assert not update_lanes(random.Random(seed), True, shear)
+        assert update_lanes(random.Random(seed), False, shear)      # negative control
