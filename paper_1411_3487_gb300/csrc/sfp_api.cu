@@ -345,8 +345,8 @@ int launch_gemm(sfp_batch* b, const T* In, const T* B, T* Out, int J, int Nc, in
 // Chains on grid y of the mode update (4 modes per thread when M % 4 == 0).
 unsigned chains_y(int C) { return (unsigned)std::min(C, 65535); }
 
-// SFP_TEST_STALL=1 in the environment makes fused launches stall on purpose
-// (one bounded wait runs out), to test that a timeout is reported and the
+// SFP_TEST_STALL=1 in the environment makes fused launches and the FP64 cluster
+// step stall on purpose (one bounded wait runs out), to test that a timeout is reported and the
 // context stays usable.
 int stall_test()
 {
@@ -589,7 +589,7 @@ cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, doub
                               (const double*)g.chiT, (const double*)g.chi, (const double*)g.phi_d,
                               (const double*)g.dm, (const double*)g.h, (const double*)g.w, (const double*)g.g, g.C,
                               g.M, c12, w0cm, g.dtau, k, (const double*)g.znoise, b->noise == SFP_NOISE_MODES ? 1 : 0,
-                              b->bad);
+                              b->bad, stall_test());
 }
 
 // CTAs per chain for the FP64 cluster path: 16 (a non-portable cluster size)
@@ -1654,7 +1654,7 @@ int sfp_observe(sfp_batch* b, int32_t what, void* host_out, size_t bytes)
     CUDA_TRY(cudaMemcpyAsync(&bad, b->bad, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     if (bad & 4) return fail(SFP_ECUDA, "a 512-bead fused step ran without its two-CTA cluster");
-    if (bad & 2) return fail(SFP_ETIMEDOUT, "a tensor-core pipeline wait timed out");
+    if (bad & 2) return fail(SFP_ETIMEDOUT, "a bounded device wait timed out");
     if (bad & 1) return fail(SFP_ENONFINITE, "a chain's state became non-finite");
     return SFP_OK;
 }
@@ -2248,7 +2248,7 @@ int sfp::internal_slots_read(sfp_batch* b, const int32_t* slots, int32_t n, doub
     CUDA_TRY(cudaMemcpyAsync(&bad, b->bad, sizeof(int), cudaMemcpyDeviceToHost, st_r));
     CUDA_TRY(cudaStreamSynchronize(st_r));
     if (bad & 4) return fail(SFP_ECUDA, "a 512-bead fused step ran without its two-CTA cluster");
-    if (bad & 2) return fail(SFP_ETIMEDOUT, "a tensor-core pipeline wait timed out");
+    if (bad & 2) return fail(SFP_ETIMEDOUT, "a bounded device wait timed out");
     if (bad & 1) return fail(SFP_ENONFINITE, "a chain's state became non-finite");
     return SFP_OK;
 }

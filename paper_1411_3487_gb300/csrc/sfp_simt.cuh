@@ -717,8 +717,9 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 // normals come from a separate kernel that draws every call of every step at once.
 // One chain, us a step (cluster barriers, tables and normals from L2 before -> here): 64
 // beads 6.6 -> 3.1, 128 11.8 -> 7.5, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
-// Every wait is bounded; after a timeout the CTA raises bit 1 of the error word, and its
-// threads run through the remaining steps without sending anything.
+// Every wait is bounded; after a timeout the CTA raises bit 1 of the error word, its
+// threads run through the remaining steps without sending anything, and no CTA of the
+// cluster writes anything back: the chain is as it was before the launch.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cluster_barrier()
 {
@@ -759,7 +760,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 const double* __restrict__ chi, const double* __restrict__ phi, const double* __restrict__ dm,
                 const double* __restrict__ h, const double* __restrict__ w, const double* __restrict__ g, int C,
                 int M, double c12nu, double w0_cm, double dtau, int n_steps, const double* __restrict__ zpre,
-                int mode_noise, int* __restrict__ bad)
+                int mode_noise, int* __restrict__ bad, int stall_test)
 {
     extern __shared__ unsigned char chain_smem[];
     const int P = M + 8;
@@ -768,7 +769,9 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     double* sz = sv + 3 * P;                              // [2][3][P]
     double* tab = sz + 6 * P;                             // [S][3][M] chi_n, chi_p, phi_p; [S] dm, g, h, w (w0_cm)
     __shared__ uint64_t v_in, r_in;                       // v, R of every CTA have arrived (1 + tx)
+    __shared__ uint64_t never;                            // nothing arrives here (the stall test)
     __shared__ int s_abort;
+    volatile int* abort_flag = &s_abort;
     const uint32_t rank = ptx::cluster_rank();
     const int c = blockIdx.x / G;                         // the cluster's chain (c < C: grid = G C)
     const int S = (M + G - 1) / G;
@@ -811,6 +814,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     if (threadIdx.x == 0) {
         ptx::mbar_init(&v_in, 1);
         ptx::mbar_init(&r_in, 1);
+        ptx::mbar_init(&never, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));
@@ -826,6 +830,8 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     asm volatile("cp.async.wait_all;" ::: "memory");
     // every CTA of the cluster runs (and has loaded R) before any remote write
     cluster_barrier();
+    // stall test: the waits of one CTA run out here, and those of the others for its forces
+    if (stall_test && (int)rank == owners - 1) ok = ptx::mbar_wait_cl(&never, 0, bad, abort_flag);
     int s = 0;
     for (; nown > 0 && s < n_steps && st0 + s < lim; ++s) {
         for (int pass = 0; pass < passes; ++pass) {
@@ -864,7 +870,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
         __syncthreads();        // also: every warp is done with the normals of the last step
         fetch_z(s + 1);
         double x0 = owns ? noise(wid) : 0.0;
-        if (owns) ok = ok && ptx::mbar_wait_cl(&v_in, s & 1, bad, &s_abort);
+        if (owns) ok = ok && ptx::mbar_wait_cl(&v_in, s & 1, bad, abort_flag);
         if (threadIdx.x == 0) ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));
         __syncwarp();
         for (int pass = 0; pass < passes; ++pass) {
@@ -894,11 +900,22 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                         if (q < owners) st_peer(&sR[ax * P + p], (uint32_t)q, o, &r_in);
             }
         }
-        if (owns) ok = ok && ptx::mbar_wait_cl(&r_in, s & 1, bad, &s_abort);
+        if (owns) ok = ok && ptx::mbar_wait_cl(&r_in, s & 1, bad, abort_flag);
         if (threadIdx.x == 0) ptx::mbar_expect_tx(&r_in, (uint32_t)(24 * (M - 1)));
         __syncwarp();
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();        // the modes that the waiting warps have seen, for the others too
+    if (*abort_flag) {
+        // what is under way in the cluster lands first; the other CTAs learn of it
+        const uint64_t t0 = ptx::globaltimer();
+        while (ptx::globaltimer() - t0 < 1000000ull) __nanosleep(1000);
+        if (threadIdx.x < G)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ptx::mapa(ptx::smem_u32(&s_abort), threadIdx.x)), "r"(1) : "memory");
+    }
+    // nobody leaves while another CTA may still write into its shared memory
+    cluster_barrier();
+    if (*abort_flag) return;
     // each CTA writes back its own modes; rank 0 the centre of mass and the counter
     for (int i = threadIdx.x; i < 3 * nown; i += blockDim.x) {
         const int a = i / nown, p = lo + i % nown;
@@ -907,9 +924,6 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     if (rank == 0 && wid == 0 && sends && j == 0) com[3 * c + ax] = cm;
     if (rank == 0 && threadIdx.x == 0) step[c] = st0 + s;
     if (!fin) atomicOr(bad, 1);
-    // nobody leaves while another CTA may still write into its shared memory
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    cluster_barrier();
 }
 
 // The cluster step of chains whose tables no CTA's shared memory holds (more than 352
@@ -934,7 +948,7 @@ k_chain_cluster_wide(double* __restrict__ Rg, double* __restrict__ com, int64_t*
                 const double* __restrict__ chi, const double* __restrict__ phi, const double* __restrict__ dm,
                 const double* __restrict__ h, const double* __restrict__ w, const double* __restrict__ g, int C,
                 int M, double c12nu, double w0_cm, double dtau, int n_steps, const double* __restrict__ zpre,
-                int mode_noise, int* __restrict__ bad)
+                int mode_noise, int* __restrict__ bad, int)
 {
     extern __shared__ unsigned char chain_smem[];
     double* sR = reinterpret_cast<double*>(chain_smem);   // [3][M]
