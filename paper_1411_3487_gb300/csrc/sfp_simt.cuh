@@ -718,7 +718,7 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 // One chain, us a step (cluster barriers, tables and normals from L2 before -> here): 64
 // beads 6.6 -> 3.1, 128 11.8 -> 7.5, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
 // Every wait is bounded; after a timeout the CTA raises bit 1 of the error word, its
-// threads run through the remaining steps without sending anything, and no CTA of the
+// threads run through the remaining steps without sending or arming anything, and no CTA of the
 // cluster writes anything back: the chain is as it was before the launch.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cluster_barrier()
@@ -871,7 +871,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
         fetch_z(s + 1);
         double x0 = owns ? noise(wid) : 0.0;
         if (owns) ok = ok && ptx::mbar_wait_cl(&v_in, s & 1, bad, abort_flag);
-        if (threadIdx.x == 0) ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));
+        if (threadIdx.x == 0 && ok) ptx::mbar_expect_tx(&v_in, (uint32_t)(24 * M));    // only a phase that is over
         __syncwarp();
         for (int pass = 0; pass < passes; ++pass) {
             const int gi = pass * nwarp + wid;
@@ -901,7 +901,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             }
         }
         if (owns) ok = ok && ptx::mbar_wait_cl(&r_in, s & 1, bad, abort_flag);
-        if (threadIdx.x == 0) ptx::mbar_expect_tx(&r_in, (uint32_t)(24 * (M - 1)));
+        if (threadIdx.x == 0 && ok) ptx::mbar_expect_tx(&r_in, (uint32_t)(24 * (M - 1)));
         __syncwarp();
     }
     asm volatile("cp.async.wait_all;" ::: "memory");

@@ -12,9 +12,11 @@ order, and every run checks
   * no deadlock (a barrier whose bytes ran past its count never completes);
   * every parity wait is for the barrier's current phase or the one before it;
   * no value is overwritten before every warp of that CTA has read it, and every value
-    that a warp reads is this step's.
+    that a warp reads is this step's;
+  * after a timeout (one CTA sends nothing, every wait that can no longer be met gives up)
+    all warps come to the end and no barrier is armed in a phase that is not over.
 Negative controls: values sent to CTAs that own nothing, on which nobody waits, and warps
-that own nothing waiting on the barriers, must be caught."""
+that own nothing waiting on the barriers, and counts armed after a timeout must be caught."""
 import random
 
 import pytest
@@ -48,13 +50,15 @@ class Barrier:
 
 
 class Cluster:
-    def __init__(self, M, G, steps, seed, idle_ctas=False, idle_warps=False):
+    def __init__(self, M, G, steps, seed, idle_ctas=False, idle_warps=False, stall=None, arm_always=False):
         """idle_ctas: CTAs that own nothing receive every value and run the steps;
-        idle_warps: warps that own nothing wait on the barriers."""
+        idle_warps: warps that own nothing wait on the barriers; stall: a CTA that gave
+        up before its first step; arm_always: counts are armed after a timeout too."""
         self.M, self.G, self.steps = M, G, steps
         self.rng = random.Random(seed)
         self.lag = (None, 0.2, 0.05)[seed % 3]          # how eagerly stores arrive
         self.idle_ctas, self.idle_warps = idle_ctas, idle_warps
+        self.stall, self.arm_always = stall, arm_always
         S = (M + G - 1) // G
         self.own = [list(range(min(M, r * S), min(M, r * S + S))) for r in range(G)]
         self.ctas = [r for r in range(G) if self.own[r] or idle_ctas]
@@ -115,45 +119,53 @@ class Cluster:
         waits = bool(mine) or self.idle_warps or (self.idle_ctas and not self.own[r])
         if not self.own[r] and not self.idle_ctas:
             return
+        ok = r != self.stall
         for s in range(self.steps):
-            self.take(r, w, "R", s)
+            if ok:
+                self.take(r, w, "R", s)
             yield None
-            for n in mine:
+            for n in mine if ok else []:
                 self.send(r, "v", n, s)
             self.met[r][w] += 1
             yield lambda: min(self.met[r]) >= s + 1
-            if waits:
-                yield self.wait(r, "v", s)
-            if w == 0:
+            if waits and ok:
+                ok = yield self.wait(r, "v", s)
+            if w == 0 and (ok or self.arm_always):
                 self.bar[r, "v"].arm(self.M)
             yield None
-            self.take(r, w, "v", s)
-            for p in mine:
+            if ok:
+                self.take(r, w, "v", s)
+            for p in mine if ok else []:
                 if p:
                     self.send(r, "R", p, s + 1)
             yield None
-            if waits:
-                yield self.wait(r, "R", s)
-            if w == 0:
+            if waits and ok:
+                ok = yield self.wait(r, "R", s)
+            if w == 0 and (ok or self.arm_always):
                 self.bar[r, "R"].arm(self.M - 1)
             yield None
 
     def run(self):
-        roles = [[self.warp(r, w), None, False] for r in range(self.G) for w in range(WARPS)]
+        roles = [[self.warp(r, w), None, False, False] for r in range(self.G) for w in range(WARPS)]
         # some warps run more often than others, those that own nothing seldom
         weight = [self.rng.choice((1, 1, 8)) if self.mine(r, w) else 0.02 for r in range(self.G) for w in range(WARPS)]
         while True:
-            ready = [i for i, (g, cond, done) in enumerate(roles) if not done and (cond is None or cond())]
+            ready = [i for i, (g, cond, done, _) in enumerate(roles) if not done and (cond is None or cond())]
             if self.stores and (not ready or self.lag is None or self.rng.random() < self.lag):
                 self.land(self.rng.randrange(len(self.stores)))
                 continue
+            met = bool(ready)
             if not ready:
-                if not all(x[2] for x in roles):
+                if all(x[2] for x in roles):
+                    return
+                # the barriers of a block's warps are not bounded; what waits on the others gives up
+                ready = [i for i, (g, cond, done, _) in enumerate(roles) if not done and cond.__name__ == "done"]
+                if self.stall is None or not ready:
                     raise ProtocolError("deadlock")
-                return
             i = self.rng.choices(ready, [weight[k] for k in ready])[0]
             try:
-                roles[i][1] = next(roles[i][0])
+                roles[i][1] = roles[i][0].send(met if roles[i][3] else None)
+                roles[i][3] = True
             except StopIteration:
                 roles[i][2] = True
 
@@ -186,6 +198,14 @@ def test_sending_to_ctas_that_own_nothing_is_caught(M, G):
 @pytest.mark.parametrize("M,G", [(3, 8), (20, 16)])
 def test_waits_of_warps_that_own_nothing_are_caught(M, G):
     assert caught(M, G, 40, idle_warps=True) > 0
+
+
+@pytest.mark.parametrize("M,G", [(20, 16), (64, 16), (20, 8)])
+def test_every_warp_comes_to_the_end_after_a_timeout(M, G):
+    for seed in range(10):
+        Cluster(M, G, 4, seed, stall=(M - 1) // ((M + G - 1) // G)).run()
+        with pytest.raises(ProtocolError, match="armed twice"):
+            Cluster(M, G, 4, seed, stall=0, arm_always=True).run()
 
 
 def update_lanes(rng, ordered, shear):
