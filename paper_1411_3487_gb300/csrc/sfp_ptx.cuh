@@ -271,6 +271,7 @@ __device__ __forceinline__ uint32_t mapa(uint32_t saddr, uint32_t rank)
 // wait until all threads of the cluster have arrived.
 __device__ __forceinline__ void cluster_sync()
 {
+    __syncwarp();       // .aligned: the whole warp at once
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

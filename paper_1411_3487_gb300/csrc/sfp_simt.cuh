@@ -723,6 +723,7 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cluster_barrier()
 {
+    __syncwarp();       // .aligned: the whole warp at once
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // *p in the shared memory of CTA `rank` of the cluster (p: this CTA's own copy), counted on
