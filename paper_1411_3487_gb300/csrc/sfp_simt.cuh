@@ -879,6 +879,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             if (gi >= nown) break;
             const int p = lo + gi;
             const double* t = tab + ((size_t)gi * 3 + 1) * M;
+            const double r = sR[ax * P + p], ry = sR[P + p];
             double d = 0.0;
             if (p > 0)                  // mode 0 takes no force, and nobody waits for its warp's read
 #pragma unroll 8
@@ -890,7 +891,6 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 cm += d;
                 if (ax == 0) cm = fma(sh * dtau, ycm, cm);
             } else {
-                const double r = sR[ax * P + p], ry = sR[P + p];
                 double o = r + fma(-tdm[gi], r, d);
                 if (sh != 0.0 && ax == 0) o = fma(sh * tg[gi], ry, o);
                 fin = fin && isfinite(o);
