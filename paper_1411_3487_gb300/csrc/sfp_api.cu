@@ -306,6 +306,18 @@ int upload_typed(sfp_batch* b, void* dst, const std::vector<double>& src)
 
 unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+constexpr int kMaxBeads = 4096;     // of a chain
+// Dynamic shared memory of a launch.  What every kernel may take is 48 KB; a limit above
+// belongs to the kernel, for the whole process, so it is set to the most that any call
+// of the kernel takes: a limit of this call's size could be lowered by another thread's
+// call before the launch.
+template <typename Kernel>
+cudaError_t allow_shared(Kernel* fn, size_t bytes, size_t most)
+{
+    return bytes <= 48 * 1024 ? cudaSuccess
+                              : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // One or two FP32 products (n of them) of the same shape in one launch of k_gemm_f32.
 // 64 x 64 tiles, and 32 x 32 ones where 64 x 64 would not give every SM a block
 // (measured, us: 600 x 128 x 128, 20 blocks, 10.3 and 6.3; 150 x 1000 x 1000 51 and
@@ -550,10 +562,12 @@ constexpr size_t kNoiseStepBytes = (size_t)32 << 20;
 // The FP64 cluster kernel for clusters of G CTAs: the one with its tables in shared memory
 // where they fit (352 beads on 16 CTAs, 256 on 8).
 using ChainClusterFn = decltype(&sfp::k_chain_cluster<16>);
-ChainClusterFn chain_cluster_kernel(int M, int G, size_t* smem)
+constexpr size_t kChainClusterBytes = 224 * 1024, kChainBytes = (size_t)9 * kChainMaxBeads * sizeof(double);
+ChainClusterFn chain_cluster_kernel(int M, int G, size_t* smem, size_t* most)
 {
-    const bool tab = sfp::chain_cluster_bytes(M, G) <= 224 * 1024;
+    const bool tab = sfp::chain_cluster_bytes(M, G) <= kChainClusterBytes;
     *smem = tab ? sfp::chain_cluster_bytes(M, G) : (size_t)9 * M * sizeof(double);
+    *most = tab ? kChainClusterBytes : kChainBytes;
     return G == 16 ? (tab ? sfp::k_chain_cluster<16> : sfp::k_chain_cluster_wide<16>)
                    : (tab ? sfp::k_chain_cluster<8> : sfp::k_chain_cluster_wide<8>);
 }
@@ -575,12 +589,10 @@ void chain_cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int 
 // Launch it (a cluster per chain) for k steps.
 cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, double w0cm, int k)
 {
-    size_t smem = 0;
-    const ChainClusterFn fn = chain_cluster_kernel(g.M, G, &smem);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    size_t smem = 0, most = 0;
+    const ChainClusterFn fn = chain_cluster_kernel(g.M, G, &smem, &most);
+    const cudaError_t e = allow_shared(fn, smem, most);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     chain_cluster_config(&cfg, &at, G, g.C, smem, b->cur);
@@ -597,12 +609,11 @@ cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, doub
 // batch has too many chains for one cluster each.
 int chain_cluster_size(const Group& g, int sms)
 {
-    size_t smem = 0;
-    const ChainClusterFn fn = chain_cluster_kernel(g.M, 16, &smem);
+    size_t smem = 0, most = 0;
+    const ChainClusterFn fn = chain_cluster_kernel(g.M, 16, &smem, &most);
     if ((int64_t)g.C * 16 <= sms &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        (smem <= 48 * 1024 ||
-         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)) {
+        allow_shared(fn, smem, most) == cudaSuccess) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at;
         chain_cluster_config(&cfg, &at, 16, g.C, smem, nullptr);
@@ -619,8 +630,7 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
     if ((rc = mark(b, 0))) return rc;
     const size_t smem = (size_t)9 * g.M * sizeof(double);
     const auto chain_steps = g.M % 2 ? sfp::k_chain_steps<double, false> : sfp::k_chain_steps<double, true>;
-    if (smem > 48 * 1024)
-        CUDA_TRY(cudaFuncSetAttribute(chain_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(allow_shared(chain_steps, smem, kChainBytes));
     const double c12 = 1.0 - 2.0 * b->dv.nu, w0cm = g.tab.w0 / std::sqrt((double)g.M);
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
@@ -791,8 +801,7 @@ int step_group_euler(sfp_batch* b, Group& g, int64_t n_steps)
     const int threads = std::min(1024, (M + 31) / 32 * 32);
     if ((M + threads - 1) / threads > 4) return fail(SFP_ENOTSUP, "the Euler path supports up to 4096 beads");
     const size_t smem = (size_t)(6 * M + 3) * sizeof(T);
-    if (smem > 48 * 1024)
-        CUDA_TRY(cudaFuncSetAttribute(sfp::k_euler_bonds<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(allow_shared(sfp::k_euler_bonds<T>, smem, (6 * kMaxBeads + 3) * sizeof(T)));
     for (int64_t s0 = 0; s0 < n_steps; s0 += 1024) {
         const int k = (int)std::min<int64_t>(1024, n_steps - s0);
         sfp::k_euler_bonds<T><<<C, threads, smem, b->cur>>>((T*)g.r, g.com, g.step, g.job, g.shear, C, M,
@@ -1025,13 +1034,14 @@ int phi_transform(sfp_batch* b, Group& g, const double* in, double* out)
 // Equilibrium starts of a group into g.stage2 (positions; tabs: l0 | Ld | Lo).  Chains
 // per block: as many as give every SM one block, at most 32 (a warp takes their serial
 // parts), within the shared memory.
+constexpr size_t kStartBytes = 227 * 1024;
 cudaError_t launch_equilibrium(sfp_batch* b, Group& g, const double* tabs)
 {
     const int N = g.M - 1;
     const size_t per_chain = (size_t)sfp::eq_pitch(g.M) * sizeof(double);
-    const int per = (int)std::max<size_t>(1, std::min<size_t>({32, (size_t)(g.C + 151) / 152, (227 * 1024) / per_chain}));
+    const int per = (int)std::max<size_t>(1, std::min<size_t>({32, (size_t)(g.C + 151) / 152, kStartBytes / per_chain}));
     const size_t smem = per * per_chain;
-    const cudaError_t e = cudaFuncSetAttribute(sfp::k_equilibrium, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_shared(sfp::k_equilibrium, smem, kStartBytes);
     if (e != cudaSuccess) return e;
     sfp::k_equilibrium<<<nblk(g.C, per), 256, smem, b->stream>>>(g.stage2, tabs, tabs + N, tabs + 2 * N, g.C, g.M, per,
                                                                 b->dv.Tstar, b->dv.nu, b->seed, g.job);
@@ -1260,7 +1270,7 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
     int64_t acc = 0;
     for (int i = 0; i < n_chains; ++i) {
         const sfp_chain_desc& d = chains[i];
-        if (d.n_beads < 3 || d.n_beads > 4096) { delete b; return fail(SFP_EINVAL, "chain %d: n_beads %d outside 3..4096", i, d.n_beads); }
+        if (d.n_beads < 3 || d.n_beads > kMaxBeads) { delete b; return fail(SFP_EINVAL, "chain %d: n_beads %d outside 3..%d", i, d.n_beads, kMaxBeads); }
         if (d.reserved != 0) { delete b; return fail(SFP_EINVAL, "chain %d: reserved must be 0", i); }
         if (d.job_id >> 32) { delete b; return fail(SFP_EINVAL, "chain %d: job_id must be < 2^32", i); }
         const double dtau = d.dtau > 0.0 ? d.dtau : d.dt_ps / dv.c_ps;
@@ -2195,14 +2205,12 @@ int sfp::internal_slots_start(sfp_batch* b, const int32_t* slots, const uint32_t
     const int N = g.M - 1;
     const size_t smem = (size_t)sfp::eq_pitch(g.M) * 8;
     if (b->precision == SFP_FP64) {
-        if (smem > 48 * 1024)
-            CUDA_TRY(cudaFuncSetAttribute(sfp::k_init_slots<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CUDA_TRY(allow_shared(sfp::k_init_slots<double>, smem, (size_t)sfp::eq_pitch(kMaxBeads) * 8));
         sfp::k_init_slots<double><<<n, 128, smem, b->stream>>>((double*)g.R, g.com, g.step, g.stop, g.job, g.shear,
             g.slot_idx, g.slot_job, g.slot_stop, g.slot_shear, g.phi_d, g.rod, g.rod + N, g.rod + 2 * N,
             g.M, b->dv.Tstar, b->dv.nu, b->seed);
     } else {
-        if (smem > 48 * 1024)
-            CUDA_TRY(cudaFuncSetAttribute(sfp::k_init_slots<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CUDA_TRY(allow_shared(sfp::k_init_slots<float>, smem, (size_t)sfp::eq_pitch(kMaxBeads) * 8));
         sfp::k_init_slots<float><<<n, 128, smem, b->stream>>>((float*)g.R, g.com, g.step, g.stop, g.job, g.shear,
             g.slot_idx, g.slot_job, g.slot_stop, g.slot_shear, g.phi_d, g.rod, g.rod + N, g.rod + 2 * N,
             g.M, b->dv.Tstar, b->dv.nu, b->seed);
