@@ -279,8 +279,9 @@ int sfp_set_integrator(sfp_batch *b, int32_t integrator);
  *                    of the forward transform) is skipped.  The fused step takes
  *                    it at 64, 128 and 256 beads with three passes (the noise
  *                    warps draw Z one step ahead into a buffer of two steps,
- *                    8 C M bytes, allocated here and counted against the
- *                    budget); 512-bead and SFP_MIXED_BF16_2 groups then run on
+ *                    24 C M bytes, allocated here with the tables of the kernel
+ *                    that takes it, within the budget: SFP_ENOMEM, and nothing
+ *                    changed, where they exceed it); 512-bead and SFP_MIXED_BF16_2 groups then run on
  *                    the staged kernels, and the grouped launch is off.  The
  *                    Euler integrator and sfp_step_noalloc always draw bead
  *                    noise.  Host only; SFP_EINVAL for an unknown value. */

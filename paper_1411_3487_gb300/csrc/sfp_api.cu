@@ -1814,17 +1814,25 @@ int sfp_set_noise(sfp_batch* b, int32_t keying)
 {
     if (!b) return fail(SFP_EINVAL, "batch is NULL");
     if (keying != SFP_NOISE_BEADS && keying != SFP_NOISE_MODES) return fail(SFP_EINVAL, "unknown noise keying %d", keying);
-    if (keying == SFP_NOISE_MODES) {
-        for (auto& g : b->groups) {
-            if (!g.fused || !sfp::fused_mode_noise_supported(g.M) || b->precision == SFP_MIXED_BF16_2) continue;
-            const size_t before = sfp::fused_bytes(g.fused);
-            int rc = sfp::fused_set_mode_noise(g.fused, true);
-            if (rc) return fail(rc, "%s", sfp_last_error());
-            b->held += sfp::fused_bytes(g.fused) - before;
+    const bool on = keying == SFP_NOISE_MODES;
+    std::vector<sfp::FusedPlan*> plans;
+    size_t more = 0;
+    for (auto& g : b->groups)
+        if (g.fused && sfp::fused_mode_noise_supported(g.M) && b->precision != SFP_MIXED_BF16_2) {
+            plans.push_back(g.fused);
+            if (on) more += sfp::fused_mode_noise_bytes(g.fused);
         }
-    } else {
-        for (auto& g : b->groups)
-            if (g.fused) sfp::fused_set_mode_noise(g.fused, false);
+    if (more && b->budget && b->held + more > b->budget)
+        return fail(SFP_ENOMEM, "HBM budget of %zu bytes exceeded (%zu held, %zu for mode-keyed noise)", b->budget, b->held, more);
+    for (size_t i = 0; i < plans.size(); ++i) {
+        const size_t before = sfp::fused_bytes(plans[i]);
+        const int rc = sfp::fused_set_mode_noise(plans[i], on);
+        b->held += sfp::fused_bytes(plans[i]) - before;
+        if (rc) {
+            // the groups before it go back, so that all draw the noise that the batch records
+            while (i-- > 0) sfp::fused_set_mode_noise(plans[i], b->noise == SFP_NOISE_MODES);
+            return rc;
+        }
     }
     if (b->noise != keying) drop_graph(b);
     b->noise = keying;

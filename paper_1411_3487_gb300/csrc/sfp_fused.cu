@@ -2226,20 +2226,30 @@ int fused_tile(const FusedPlan* p) { return p->cpt; }
 
 int fused_ctas_per_tile(const FusedPlan* p) { return p->M == 512 ? 2 : 1; }
 
+static size_t classic_bytes(const FusedPlan* p)
+{
+    return (size_t)(p->fold ? 3 : 6) * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float);
+}
+static size_t zbuf_bytes(const FusedPlan* p) { return (size_t)2 * p->C * 3 * p->M * sizeof(float); }
+
 size_t fused_bytes(const FusedPlan* p)
 {
     if (!p) return 0;
-    return (p->classic ? (size_t)(p->fold ? 3 : 6) * p->M * p->M * (p->bf16 ? 2 : 4) + (size_t)p->M * sizeof(float) : 0) +
-           (p->zbuf ? (size_t)2 * p->C * 3 * p->M * sizeof(float) : 0) + p->lane_bytes;
+    return (p->classic ? classic_bytes(p) : 0) + (p->zbuf ? zbuf_bytes(p) : 0) + p->lane_bytes;
 }
 
-// The plan's tile and its R map.
+size_t fused_mode_noise_bytes(const FusedPlan* p) { return (p->classic ? 0 : classic_bytes(p)) + (p->zbuf ? 0 : zbuf_bytes(p)); }
+
+// The plan's tile and, for the kernels that load R by it, its R map (the lane step has
+// none, so that a return to it cannot fail).
 static int retile(FusedPlan* p, int cpt)
 {
-    CUtensorMap m;
-    const int rc = make_map_2d(&m, p->R, 3 * p->C, p->M, 3 * (cpt / 4));
-    if (rc) return rc;
-    p->tmR = m;
+    if (!p->lane_tab || p->mz) {
+        CUtensorMap m;
+        const int rc = make_map_2d(&m, p->R, 3 * p->C, p->M, 3 * (cpt / 4));
+        if (rc) return rc;
+        p->tmR = m;
+    }
     p->cpt = cpt;
     return SFP_OK;
 }
@@ -2260,11 +2270,19 @@ int fused_set_mode_noise(FusedPlan* p, bool on)
         return report(SFP_ENOTSUP, "mode-keyed noise on the fused step: 64, 128 or 256 beads, three passes");
     if (on && !p->classic) {
         const int rc = classic_tables(p, p->chi.data(), p->phi.data(), p->h.data(), p->w.data());
-        if (rc) return rc;
+        if (rc) {
+            for (void*& t : p->tab) {
+                cudaFree(t);
+                t = nullptr;
+            }
+            cudaFree(p->w32);
+            p->w32 = nullptr;
+            return rc;
+        }
     }
-    if (on && !p->zbuf) {
-        const size_t bytes = (size_t)2 * p->C * 3 * p->M * sizeof(float);
-        if (cudaMalloc((void**)&p->zbuf, bytes) != cudaSuccess) return report(SFP_ENOMEM, "mode-noise buffer allocation failed");
+    if (on && !p->zbuf && cudaMalloc((void**)&p->zbuf, zbuf_bytes(p)) != cudaSuccess) {
+        p->zbuf = nullptr;
+        return report(SFP_ENOMEM, "mode-noise buffer allocation failed");
     }
     if (p->mz == on) return SFP_OK;
     // the kernels of the two keyings take tiles of different sizes

@@ -61,7 +61,10 @@ int fused_set_tile(FusedPlan* plan, int cpt);
 // Mode-keyed noise on (Z drawn per mode, Eq. c4 reading; M <= 256 only: the
 // 512-bead cluster kernel draws bead noise): allocates the plan's Z buffer and, for the
 // lane step's plans, the tables of the kernel that takes it; tiles are chosen anew.
+// Fails only towards mode-keyed noise, and then changes nothing but the memory held.
 int fused_set_mode_noise(FusedPlan* plan, bool on);
+// Bytes that switching mode-keyed noise on would allocate.
+size_t fused_mode_noise_bytes(const FusedPlan* plan);
 bool fused_mode_noise_supported(int M);
 // True for plans that the grouped launch takes (every fused plan).
 bool fused_groupable(const FusedPlan* plan);
