@@ -323,15 +323,27 @@ cudaError_t allow_shared(Kernel* fn, size_t bytes, size_t most)
 // (measured, us: 600 x 128 x 128, 20 blocks, 10.3 and 6.3; 150 x 1000 x 1000 51 and
 // 31; 6003 x 100 x 100, 188 blocks, 10.4 both; 12288 x 256 x 256 45 and 64; 128 x 128
 // tiles of 8 x 8 outputs per thread: 59, and never ahead up to 49152 x 512 x 512).
-cudaError_t gemm_f32(cudaStream_t st, const sfp::GemmF32& g, int n, int J, int Nc, int K)
+// Row tiles are on grid y, which takes 65535: more rows (1.4 million chains) go in parts
+// (all tiles on grid x, with a division in the kernel: 57 -> 60 us a step of 1024 x 256
+// beads).
+cudaError_t gemm_f32(cudaStream_t st, sfp::GemmF32 g, int n, int J, int Nc, int K)
 {
     bool vec = K % 4 == 0;
     for (int z = 0; z < n; ++z)
         vec = vec && ((uintptr_t)g.in[z] | (uintptr_t)g.b[z] | (uintptr_t)g.out[z]) % 16 == 0;
     if ((int64_t)nblk(Nc, 64) * nblk(J, 64) * n >= 152) {
-        const dim3 grid(nblk(Nc, 64), nblk(J, 64), (unsigned)n);
-        if (vec) sfp::k_gemm_f32<64, 64, 8, 4, true><<<grid, 128, 0, st>>>(g, J, Nc, K);
-        else sfp::k_gemm_f32<64, 64, 8, 4, false><<<grid, 128, 0, st>>>(g, J, Nc, K);
+        constexpr int kRows = 64 * 65535;
+        for (;;) {
+            const int rows = std::min(J, kRows);
+            const dim3 grid(nblk(Nc, 64), nblk(rows, 64), (unsigned)n);
+            if (vec) sfp::k_gemm_f32<64, 64, 8, 4, true><<<grid, 128, 0, st>>>(g, rows, Nc, K);
+            else sfp::k_gemm_f32<64, 64, 8, 4, false><<<grid, 128, 0, st>>>(g, rows, Nc, K);
+            if ((J -= rows) == 0) break;
+            for (int z = 0; z < n; ++z) {
+                g.in[z] += (size_t)rows * K;
+                g.out[z] += (size_t)rows * Nc;
+            }
+        }
     } else {
         const dim3 grid(nblk(Nc, 32), nblk(J, 32), (unsigned)n);
         if (vec) sfp::k_gemm_f32<32, 32, 4, 4, true><<<grid, 64, 0, st>>>(g, J, Nc, K);
