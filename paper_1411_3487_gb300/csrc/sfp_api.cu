@@ -199,6 +199,7 @@ struct Group {
     double* znoise = nullptr;     // FP64 cluster path: bead normals of znoise_steps steps [s][C][3][M]
     int znoise_steps = 0;
     int chain_g = -1;             // FP64 path: CTAs per chain (16, 8, or 0: one CTA per chain); -1 not chosen yet
+    bool chain_tab = false;       // ... the cluster kernel with its tables in shared memory
     cudaStream_t ns = nullptr;    // the staged step's noise kernel, beside the inverse transform
     cudaEvent_t nfork = nullptr, njoin = nullptr;
     // observable sampling (allocated by the first sfp_set_sampling)
@@ -566,18 +567,15 @@ bool one_launch(const sfp_batch* b, const Group& g)
     return fused_ok(b, g) || (b->precision == SFP_FP64 && g.M <= kChainMaxBeads);
 }
 
-// n_steps FP64 steps of a group in one launch of k_chain_steps (a CTA per chain,
-// state in shared memory between steps); recorded as one fused stage.
 // The most bytes of pre-drawn bead normals the FP64 cluster path keeps.
 constexpr size_t kNoiseStepBytes = (size_t)32 << 20;
 
-// The FP64 cluster kernel for clusters of G CTAs: the one with its tables in shared memory
-// where they fit (352 beads on 16 CTAs, 256 on 8).
+// The FP64 cluster kernel for clusters of G CTAs, with its tables in shared memory (they
+// fit up to 352 beads on 16 CTAs and 256 on 8) or from L2.
 using ChainClusterFn = decltype(&sfp::k_chain_cluster<16>);
 constexpr size_t kChainClusterBytes = 224 * 1024, kChainBytes = (size_t)9 * kChainMaxBeads * sizeof(double);
-ChainClusterFn chain_cluster_kernel(int M, int G, size_t* smem, size_t* most)
+ChainClusterFn chain_cluster_kernel(int M, int G, bool tab, size_t* smem, size_t* most)
 {
-    const bool tab = sfp::chain_cluster_bytes(M, G) <= kChainClusterBytes;
     *smem = tab ? sfp::chain_cluster_bytes(M, G) : (size_t)9 * M * sizeof(double);
     *most = tab ? kChainClusterBytes : kChainBytes;
     return G == 16 ? (tab ? sfp::k_chain_cluster<16> : sfp::k_chain_cluster_wide<16>)
@@ -602,7 +600,7 @@ void chain_cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int 
 cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, double w0cm, int k)
 {
     size_t smem = 0, most = 0;
-    const ChainClusterFn fn = chain_cluster_kernel(g.M, G, &smem, &most);
+    const ChainClusterFn fn = chain_cluster_kernel(g.M, G, g.chain_tab, &smem, &most);
     const cudaError_t e = allow_shared(fn, smem, most);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
@@ -616,24 +614,44 @@ cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, doub
                               b->bad, stall_test());
 }
 
-// CTAs per chain for the FP64 cluster path: 16 (a non-portable cluster size)
-// when the GPU can place such clusters for this shape, else 8; 0 when the
-// batch has too many chains for one cluster each.
-int chain_cluster_size(const Group& g, int sms)
+// CTAs per chain and kernel of the FP64 cluster path: 16 (a non-portable cluster size)
+// when the GPU can place such clusters for this shape, else 8; 0 CTAs when the batch has
+// too many chains for one cluster each.  A CTA with tables of more than 112 KB fills its
+// SM, and of such clusters the GPU holds 7 of 16 CTAs and 15 of 8 at once (GB300); the
+// tables are left in L2 where the chains would then take turns (us a step, tables in
+// shared memory and in L2: 7 chains of 256 beads 22.6 and 30.0, 8 of them 44.5 and 36.3;
+// 15 of 184 beads 26.1 and 38.7, 16 of them 51.3 and 45.3).  From 257 beads a warp of the
+// kernel with L2 tables takes two bonds in turn on 16 CTAs, and up to 320 two rounds of
+// the other are still ahead (9 chains of 257 beads 56.4 and 61.8, of 320 65.2 and 77.6, of
+// 321 79.1 and 76.0).
+void choose_chain_cluster(Group& g, int sms)
 {
-    size_t smem = 0, most = 0;
-    const ChainClusterFn fn = chain_cluster_kernel(g.M, 16, &smem, &most);
-    if ((int64_t)g.C * 16 <= sms &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        allow_shared(fn, smem, most) == cudaSuccess) {
-        cudaLaunchConfig_t cfg;
-        cudaLaunchAttribute at;
-        chain_cluster_config(&cfg, &at, 16, g.C, smem, nullptr);
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) return 16;
-        cudaGetLastError();
+    g.chain_g = 0;
+    g.chain_tab = false;
+    for (const int G : {16, 8}) {
+        if ((int64_t)g.C * G > sms) continue;
+        for (const bool tab : {true, false}) {
+            if (tab && sfp::chain_cluster_bytes(g.M, G) > kChainClusterBytes) continue;
+            size_t smem = 0, most = 0;
+            const ChainClusterFn fn = chain_cluster_kernel(g.M, G, tab, &smem, &most);
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute at;
+            chain_cluster_config(&cfg, &at, G, g.C, smem, nullptr);
+            int n = 0;          // clusters that the GPU holds at once
+            if ((G == 16 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+                allow_shared(fn, smem, most) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            if (n >= (tab && !(g.M > 256 && g.M <= 320) ? g.C : 1)) {
+                g.chain_g = G;
+                g.chain_tab = tab;
+                return;
+            }
+        }
+        if (G == 8) g.chain_g = 8;
     }
-    return (int64_t)g.C * 8 <= sms ? 8 : 0;
 }
 
 int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
@@ -650,7 +668,7 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
     // few chains: a cluster of CTAs per chain, so that each chain uses several SMs;
     // the bead normals of up to kNoiseStepBytes of steps are drawn beforehand in
     // one kernel (the buffer is allocated on first use, outside stream capture)
-    if (g.chain_g < 0) g.chain_g = chain_cluster_size(g, sms);
+    if (g.chain_g < 0) choose_chain_cluster(g, sms);
     const int G = g.chain_g;
     bool cluster = G > 0;
     if (cluster && !g.znoise) {
@@ -1399,7 +1417,7 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
             e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) { destroy_impl(b); return fail(SFP_ECUDA, "create: %s", cudaGetErrorString(e)); }
-            g.chain_g = chain_cluster_size(g, sms);
+            choose_chain_cluster(g, sms);
             if (g.chain_g > 0) {
                 const size_t per_step = (size_t)g.C * 3 * M * sizeof(double);
                 g.znoise_steps = (int)std::max<size_t>(1, std::min<size_t>(1024, kNoiseStepBytes / per_step));
