@@ -1433,10 +1433,10 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
     }
     // Lengths that share one grouped launch (at most one group each of 64, 128,
     // 256 and 512 beads): chains per tile chosen for all of them together, not
-    // for each group as if it had the GPU to itself.  If tiles of 40 chains (the
-    // fewest MMAs per chain) take more than one wave of the SMs, 40 (the
-    // autotuner's choice on 8192 mixed chains); else the smallest tiles that
-    // still fit one wave.
+    // for each group as if it had the GPU to itself.  If the largest tiles that each
+    // group's step takes (the fewest MMAs per chain) need more than one wave of the
+    // SMs, those (the autotuner's choice on 8192 mixed chains); else the smallest
+    // tiles that still fit one wave.
     {
         std::vector<size_t> cand;
         bool seen[4] = {false, false, false, false};
@@ -1455,7 +1455,8 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
                 int64_t n = 0;
                 for (size_t i : cand) {
                     const Group& g = b->groups[i];
-                    n += (int64_t)((g.C + cpt - 1) / cpt) * (g.M == 512 ? 2 : 1);
+                    const int c = std::min(cpt, sfp::fused_most_chains(g.fused));
+                    n += (int64_t)((g.C + c - 1) / c) * sfp::fused_ctas_per_tile(g.fused);
                 }
                 return n;
             };
@@ -1956,11 +1957,12 @@ int sfp_autotune(sfp_batch* b, int32_t trial_steps, int32_t* chains_per_tile)
         Group& g = b->groups[fg[k]];
         std::vector<int> cs;
         const int units = sms / sfp::fused_ctas_per_tile(g.fused);   // tiles that fit one wave
+        const int most = sfp::fused_most_chains(g.fused);
         for (double f : {1.0, 0.75, 0.5, 1.0 / 3.0, 0.25}) {
             const int target = std::max(1, (int)(f * units));
-            cs.push_back(std::min(40, ((g.C + target - 1) / target + 3) / 4 * 4));
+            cs.push_back(std::min(most, ((g.C + target - 1) / target + 3) / 4 * 4));
         }
-        cs.push_back(40);
+        cs.push_back(most);
         std::sort(cs.begin(), cs.end());
         cs.erase(std::unique(cs.begin(), cs.end()), cs.end());
         for (int c : cs) {

@@ -2224,6 +2224,8 @@ int fused_step_grouped(FusedPlan* const* plans, const FusedArgs* args, int n, cu
 
 int fused_tile(const FusedPlan* p) { return p->cpt; }
 
+int fused_most_chains(const FusedPlan* p) { return most_chains(p); }
+
 int fused_ctas_per_tile(const FusedPlan* p) { return p->M == 512 ? 2 : 1; }
 
 static size_t classic_bytes(const FusedPlan* p)

@@ -53,6 +53,8 @@ int fused_step(FusedPlan* plan, const FusedArgs& args, cudaStream_t stream);
 // of 4 and limited to what the plan's step takes: 32 for the lane step, 24 at 512
 // beads; rebuilds the R map).
 int fused_tile(const FusedPlan* plan);
+// The most that the plan's step takes: 40, for the lane step 32, at 512 beads 24.
+int fused_most_chains(const FusedPlan* plan);
 // CTAs that run one tile: 2 at M = 512 (a cluster pair), else 1.
 int fused_ctas_per_tile(const FusedPlan* plan);
 // Device bytes the plan's tables hold.
