@@ -896,8 +896,11 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
                 mbar_arrive(v_ready);
             }
         };
-        if (lane == 0) arm();
-        ok = mbar_wait(r_ready, 0, a.err, abort_flag);      // every phase in turn
+        // every phase of r_ready in turn, and each before the arrival on v_ready that the
+        // next one needs: armed first, the step could pass while this warp still looks for
+        // phase 0, which then has the parity of phase 2
+        ok = __all_sync(0xffffffffu, mbar_wait(r_ready, 0, a.err, abort_flag)) != 0;
+        if (lane == 0 && ok) arm();
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps; ++sp) {
             ok = ok && mbar_wait(r_ready, (sp + 1) & 1, a.err, abort_flag);
