@@ -467,9 +467,9 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             __syncwarp();
             if (lane == 0 && ok) mbar_arrive(bar);
         };
-        // the lanes agree on whether a wait was met: the TMEM loads and stores after it are
-        // the whole warp's
-        auto agree = [&](bool met) { ok = __all_sync(0xffffffffu, ok && met) != 0; };
+        // the lanes agree on whether a wait was met, where TMEM loads, which are the whole
+        // warp's, depend on it (those of the update run either way)
+        auto agree = [&](bool met) { ok = __all_sync(0xffffffffu, met) != 0; };
         auto store_x = [&](uint2 hi, uint2 lo, int off, int ax, int b) {
             uint8_t* w = xw + off + (3 * G::pair(b) + ax) * G::XSBO + G::half(b) * 8;
             *reinterpret_cast<uint2*>(w) = hi;
@@ -679,7 +679,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             }
             put_r(r, b);
             if (tm) keep_r(r, b);
-            else store_r(r, b);
+            else if (ok) store_r(r, b);
         };
 
         // operand X of the first step
@@ -738,17 +738,17 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
             float rg[NP][3][4];
             const int bg = b0 + bs * ((G::TB - b0 + bs - 1) / bs);      // this warp's first one
             if (G::TB < 8 && bg < nb) load_r(rg, bg);
-            agree(ok && mbar_wait(inc_done, sp & 1, a.err, abort_flag));
+            ok = ok && mbar_wait(inc_done, sp & 1, a.err, abort_flag);
             fence_after();
 #pragma unroll 1
-            for (int b = b0; ok && b < min(nb, G::TB); b += bs) {
+            for (int b = b0; b < min(nb, G::TB); b += bs) {
                 float r[NP][3][4];
                 if (steady) update4(r, b, sp, true, true);
                 else update4(r, b, sp, true, false);
             }
             if constexpr (G::TB < 8) {
 #pragma unroll 1
-                for (int b = bg; ok && b < nb; b += bs) {
+                for (int b = bg; b < nb; b += bs) {
                     if (b != bg) load_r(rg, b);
                     update4(rg, b, sp, false, steady);
                 }
@@ -899,7 +899,7 @@ __device__ __forceinline__ bool lane_tile(const FusedArgs& a, const LaneArgs& la
         // every phase of r_ready in turn, and each before the arrival on v_ready that the
         // next one needs: armed first, the step could pass while this warp still looks for
         // phase 0, which then has the parity of phase 2
-        ok = __all_sync(0xffffffffu, mbar_wait(r_ready, 0, a.err, abort_flag)) != 0;
+        ok = mbar_wait(r_ready, 0, a.err, abort_flag);
         if (lane == 0 && ok) arm();
 #pragma unroll 1
         for (int sp = 0; sp < a.n_steps; ++sp) {
