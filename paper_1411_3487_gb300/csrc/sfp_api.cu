@@ -220,6 +220,7 @@ struct sfp_batch {
     Derived dv{};
     int precision = 0;
     uint32_t seed = 0;
+    int sms = 0;                       // multiprocessors of the device
     cudaStream_t stream = nullptr;
     size_t budget = 0, held = 0;
     int64_t launches = 0;
@@ -307,6 +308,14 @@ int upload_typed(sfp_batch* b, void* dst, const std::vector<double>& src)
 
 unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// Multiprocessors of the current device.
+cudaError_t multiprocessors(int* sms)
+{
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
 constexpr int kMaxBeads = 4096;     // of a chain
 // Dynamic shared memory of a launch.  What every kernel may take is 48 KB; a limit above
 // belongs to the kernel, for the whole process, so it is set to the most that any call
@@ -327,12 +336,12 @@ cudaError_t allow_shared(Kernel* fn, size_t bytes, size_t most)
 // Row tiles are on grid y, which takes 65535: more rows (1.4 million chains) go in parts
 // (all tiles on grid x, with a division in the kernel: 57 -> 60 us a step of 1024 x 256
 // beads).
-cudaError_t gemm_f32(cudaStream_t st, sfp::GemmF32 g, int n, int J, int Nc, int K)
+cudaError_t gemm_f32(cudaStream_t st, int sms, sfp::GemmF32 g, int n, int J, int Nc, int K)
 {
     bool vec = K % 4 == 0;
     for (int z = 0; z < n; ++z)
         vec = vec && ((uintptr_t)g.in[z] | (uintptr_t)g.b[z] | (uintptr_t)g.out[z]) % 16 == 0;
-    if ((int64_t)nblk(Nc, 64) * nblk(J, 64) * n >= 152) {
+    if ((int64_t)nblk(Nc, 64) * nblk(J, 64) * n >= sms) {
         constexpr int kRows = 64 * 65535;
         for (;;) {
             const int rows = std::min(J, kRows);
@@ -357,7 +366,7 @@ template <typename T>
 int launch_gemm(sfp_batch* b, const T* In, const T* B, T* Out, int J, int Nc, int K)
 {
     if constexpr (sizeof(T) == 4) {
-        CUDA_TRY(gemm_f32(b->cur, sfp::GemmF32{{In, nullptr}, {B, nullptr}, {Out, nullptr}}, 1, J, Nc, K));
+        CUDA_TRY(gemm_f32(b->cur, b->sms, sfp::GemmF32{{In, nullptr}, {B, nullptr}, {Out, nullptr}}, 1, J, Nc, K));
     } else {
         dim3 grid(nblk(Nc, 64), nblk(J, 64));
         sfp::k_gemm_nt<double, 64, 64, 8, 4, 4><<<grid, 256, 0, b->cur>>>(In, B, Out, J, Nc, K);
@@ -662,13 +671,10 @@ int step_group_chain(sfp_batch* b, Group& g, int64_t n_steps)
     const auto chain_steps = g.M % 2 ? sfp::k_chain_steps<double, false> : sfp::k_chain_steps<double, true>;
     CUDA_TRY(allow_shared(chain_steps, smem, kChainBytes));
     const double c12 = 1.0 - 2.0 * b->dv.nu, w0cm = g.tab.w0 / std::sqrt((double)g.M);
-    int dev = 0, sms = 0;
-    CUDA_TRY(cudaGetDevice(&dev));
-    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // few chains: a cluster of CTAs per chain, so that each chain uses several SMs;
     // the bead normals of up to kNoiseStepBytes of steps are drawn beforehand in
     // one kernel (the buffer is allocated on first use, outside stream capture)
-    if (g.chain_g < 0) choose_chain_cluster(g, sms);
+    if (g.chain_g < 0) choose_chain_cluster(g, b->sms);
     const int G = g.chain_g;
     bool cluster = G > 0;
     if (cluster && !g.znoise) {
@@ -758,7 +764,7 @@ int step_group(sfp_batch* b, Group& g)
     // a4: DeltaH = chi^T v (Eq. e11), Z = phi^T z (Eq. c4): the forward transform
     if (g.tc) rc = sfp::tc_transform(g.tc, mk ? 2 : 1, b->cur);
     else if constexpr (sizeof(T) == 4) {
-        CUDA_TRY(gemm_f32(b->cur, sfp::GemmF32{{fz, fz + n}, {(const T*)g.chiT, (const T*)g.phiT}, {yz, yz + n}}, mk ? 1 : 2,
+        CUDA_TRY(gemm_f32(b->cur, b->sms, sfp::GemmF32{{fz, fz + n}, {(const T*)g.chiT, (const T*)g.phiT}, {yz, yz + n}}, mk ? 1 : 2,
                           3 * C, M, M));
         b->launches++;
     } else if (!(rc = launch_gemm<T>(b, fz, (const T*)g.chiT, yz, 3 * C, M, M)) && !mk) {
@@ -1069,7 +1075,7 @@ cudaError_t launch_equilibrium(sfp_batch* b, Group& g, const double* tabs)
 {
     const int N = g.M - 1;
     const size_t per_chain = (size_t)sfp::eq_pitch(g.M) * sizeof(double);
-    const int per = (int)std::max<size_t>(1, std::min<size_t>({32, (size_t)(g.C + 151) / 152, kStartBytes / per_chain}));
+    const int per = (int)std::max<size_t>(1, std::min<size_t>({32, (size_t)(g.C + b->sms - 1) / b->sms, kStartBytes / per_chain}));
     const size_t smem = per * per_chain;
     const cudaError_t e = allow_shared(sfp::k_equilibrium, smem, kStartBytes);
     if (e != cudaSuccess) return e;
@@ -1327,6 +1333,8 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
     b->total_beads = acc / 3;
     const size_t es = (precision == SFP_FP64) ? 8 : 4;
     if ((rc = dalloc_t(b, &b->bad, sizeof(int)))) { destroy_impl(b); return rc; }
+    const cudaError_t de = multiprocessors(&b->sms);
+    if (de != cudaSuccess) { destroy_impl(b); return fail(SFP_ECUDA, "create: %s", cudaGetErrorString(de)); }
     size_t staging = 0;
     for (auto& g : b->groups) staging += align256(g.chains.size() * 3 * g.M * 8);
     if ((rc = dalloc_t(b, &b->stage, staging))) { destroy_impl(b); return rc; }
@@ -1413,11 +1421,7 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
         if (precision == SFP_FP64 && M <= kChainMaxBeads) {
             // the FP64 chain path: a cluster of CTAs per chain for few chains, with
             // its buffer of pre-drawn normals allocated here, outside any capture
-            int dev = 0, sms = 0;
-            e = cudaGetDevice(&dev);
-            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) { destroy_impl(b); return fail(SFP_ECUDA, "create: %s", cudaGetErrorString(e)); }
-            choose_chain_cluster(g, sms);
+            choose_chain_cluster(g, b->sms);
             if (g.chain_g > 0) {
                 const size_t per_step = (size_t)g.C * 3 * M * sizeof(double);
                 g.znoise_steps = (int)std::max<size_t>(1, std::min<size_t>(1024, kNoiseStepBytes / per_step));
@@ -1448,9 +1452,8 @@ int sfp_create(const sfp_params* params, const sfp_chain_desc* chains, int32_t n
             seen[slot] = true;
             cand.push_back(i);
         }
-        int dev = 0, sms = 0;
-        if (cand.size() >= 2 && cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
+        if (cand.size() >= 2) {
+            const int sms = b->sms;
             auto ctas = [&](int cpt) {
                 int64_t n = 0;
                 for (size_t i : cand) {
@@ -1898,9 +1901,7 @@ int sfp_autotune(sfp_batch* b, int32_t trial_steps, int32_t* chains_per_tile)
     for (size_t i = 0; i < G; ++i)
         if (fused_ok(b, b->groups[i])) fg.push_back(i);
     if (fg.empty()) return SFP_OK;
-    int dev = 0, sms = 148;
-    CUDA_TRY(cudaGetDevice(&dev));
-    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = b->sms;
     // save every group's dynamic state; each trial starts from it again
     struct Saved { void* R = nullptr; double* com = nullptr; int64_t* step = nullptr; };
     std::vector<Saved> sv(G);
@@ -2153,6 +2154,8 @@ int sfp_step_noalloc(const sfp_params* params, const sfp_chain_desc* chain, int3
                     C, M, off, (unsigned)SFP_NOALLOC_SCRATCH_BYTES);
     unsigned char* base = nullptr;
     if ((rc = noalloc_scratch(&base))) return rc;
+    int sms = 0;
+    CUDA_TRY(multiprocessors(&sms));
     cudaStream_t st = (cudaStream_t)cuda_stream;
     float* chi = (float*)(base + o_chi);
     float* chiT = (float*)(base + o_chiT);
@@ -2173,9 +2176,9 @@ int sfp_step_noalloc(const sfp_params* params, const sfp_chain_desc* chain, int3
     const double w0 = std::sqrt(2.0 * dv.Tstar * dtau);
     int* bad = (int*)(base + o_bad);   // written by the update kernel, not reported here
     for (int64_t s = 0; s < n_steps; ++s) {
-        CUDA_TRY(gemm_f32(st, sfp::GemmF32{{modes_dev, nullptr}, {chi, nullptr}, {r, nullptr}}, 1, 3 * C, M, M));
+        CUDA_TRY(gemm_f32(st, sms, sfp::GemmF32{{modes_dev, nullptr}, {chi, nullptr}, {r, nullptr}}, 1, 3 * C, M, M));
         CUDA_TRY(launch_force_noise<float>(st, r, fz, fz + n, C, M, c12, (uint32_t)seed, job, step));
-        CUDA_TRY(gemm_f32(st, sfp::GemmF32{{fz, fz + n}, {chiT, phiT}, {yz, yz + n}}, 2, 3 * C, M, M));
+        CUDA_TRY(gemm_f32(st, sms, sfp::GemmF32{{fz, fz + n}, {chiT, phiT}, {yz, yz + n}}, 2, 3 * C, M, M));
         CUDA_TRY(launch_mode_update<float>(st, modes_dev, yz, yz + n, com_dev, step, dm, h, w, g, shear, C, M, w0,
                                            dtau, bad, nullptr));
     }
