@@ -369,7 +369,7 @@ int launch_gemm(sfp_batch* b, const T* In, const T* B, T* Out, int J, int Nc, in
         CUDA_TRY(gemm_f32(b->cur, b->sms, sfp::GemmF32{{In, nullptr}, {B, nullptr}, {Out, nullptr}}, 1, J, Nc, K));
     } else {
         dim3 grid(nblk(Nc, 64), nblk(J, 64));
-        sfp::k_gemm_nt<double, 64, 64, 8, 4, 4><<<grid, 256, 0, b->cur>>>(In, B, Out, J, Nc, K);
+        sfp::k_gemm_nt<64, 64, 8, 4, 4><<<grid, 256, 0, b->cur>>>(In, B, Out, J, Nc, K);
         CUDA_TRY(cudaGetLastError());
     }
     b->launches++;

@@ -113,7 +113,7 @@ static_assert(2 + kComputeWarps == 10 && kComputeWarps == 8, "warp numbering of 
 // over it.  The single-CTA kernel stages R on its own at 64 and 128 beads
 // (four stages either way) and in place at 256 beads, where that gives four
 // stages of 48 KB instead of three of 64 KB (24.2 -> 23.1 us per step at
-// 4096 x 256 bp; with mode-keyed noise, whose steps have no noise blocks,
+// 4096 x 256 bp with three passes, which are the lane step's now; with mode-keyed noise, whose steps have no noise blocks,
 // three stages stay faster: 24.0 against 24.5 us); the 512-bead kernel splits
 // in place.
 template <int NB, bool BF, bool MZ = false> constexpr bool kRS = BF && (NB != 256 || MZ);
@@ -1144,9 +1144,9 @@ k_lane_step(const FusedArgs a, const lanes::LaneArgs la)
 // The 512-bead step: tile `tile` on a cluster of two CTAs, CTA h (its rank)
 // holding bonds and modes 256 h .. 256 h + 255 (see the file's header).  The
 // caller launches clusters of two and allocates the 512 TMEM columns at `tmem`;
-// the tile starts and ends with a cluster barrier.  Returns false if a wait
-// gave up.
-template <bool BF, bool TWO>
+// the tile starts and ends with a cluster barrier.  BF: two BF16 passes, else three of
+// TF32.  Returns false if a wait gave up.
+template <bool BF>
 __device__ __forceinline__ bool pair_tile(const CUtensorMap& tmR, const CUtensorMap& tmChiH,
                                           const CUtensorMap& tmChiL, const CUtensorMap& tmFH,
                                           const CUtensorMap& tmFL, const FusedArgs& a, int tile, uint8_t* smem,
@@ -1159,7 +1159,9 @@ __device__ __forceinline__ bool pair_tile(const CUtensorMap& tmR, const CUtensor
     constexpr int KB = 2 * KBL;         // inverse K blocks = forward bead blocks = M / 32
     constexpr int MB = KB * kKB;        // beads M
     constexpr int NBLK = 3 * KB;        // blocks of one step, in the order of sched_decode
-    constexpr int FILL = BF ? 4 : 1;   // noise blocks in phase 1's tail (measured: BF16 4, TF32 1)
+    // noise blocks in phase 1's tail (two BF16 passes, 16384 chains: 0 270 us a step, 2 266,
+    // 4 263.8, 6 264.1, 8 264.4; TF32: 1)
+    constexpr int FILL = BF ? 4 : 1;
     static_assert(KB % 2 == 0, "the block schedule pairs bead blocks");
 
     uint8_t* stage0 = smem;
@@ -1404,12 +1406,7 @@ __device__ __forceinline__ bool pair_tile(const CUtensorMap& tmR, const CUtensor
 #pragma unroll
                     for (int kk = 0; kk < kKB / 16; ++kk) {
                         const uint32_t off = kk * 32;   // 16 BF16 = 32 bytes along K
-                        if constexpr (TWO) {
-                            mma_bf16(d, sdesc64(a_lo + off), sdesc64(b_hi + off), idesc, (first && kk == 0) ? 0u : 1u);
-                        } else {
-                            mma_bf16(d, sdesc64(a_hi + off), sdesc64(b_lo + off), idesc, (first && kk == 0) ? 0u : 1u);
-                            mma_bf16(d, sdesc64(a_lo + off), sdesc64(b_hi + off), idesc, 1u);
-                        }
+                        mma_bf16(d, sdesc64(a_lo + off), sdesc64(b_hi + off), idesc, (first && kk == 0) ? 0u : 1u);
                         mma_bf16(d, sdesc64(a_hi + off), sdesc64(b_hi + off), idesc, 1u);
                     }
                 } else {
@@ -1723,7 +1720,7 @@ __device__ __forceinline__ void pair_abort_grace()
 }
 
 // One 512-bead tile per cluster of two CTAs (a launch of one length group).
-template <bool BF, bool TWO = false>
+template <bool BF>
 __global__ void __launch_bounds__(kThreads, 1)
 k_fused_pair(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmChiH,
              const __grid_constant__ CUtensorMap tmChiL, const __grid_constant__ CUtensorMap tmFH,
@@ -1739,7 +1736,7 @@ k_fused_pair(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CU
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     tmem_alloc<512>(&s_tmem);
     const uint32_t tmem = s_tmem;
-    const bool ok = pair_tile<BF, TWO>(tmR, tmChiH, tmChiL, tmFH, tmFL, a, (int)(blockIdx.x >> 1), smem, tmem);
+    const bool ok = pair_tile<BF>(tmR, tmChiH, tmChiL, tmFH, tmFL, a, (int)(blockIdx.x >> 1), smem, tmem);
     tmem_free<512>(tmem);
     if (!ok) pair_abort_grace();
 }
@@ -1781,7 +1778,7 @@ template <bool BF, bool TWO>
 __device__ __noinline__ bool grouped_pair(const GroupSlot& g, int tile, uint8_t* smem_raw, uint32_t tmem)
 {
     if constexpr (BF && !TWO) return lanes::lane_tile<512>(g.a, g.la, tile, align_up(smem_raw, 128), tmem);
-    else return pair_tile<BF, TWO>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, align_up(smem_raw, 1024), tmem);
+    else return pair_tile<BF>(g.tmR, g.tmChiH, g.tmChiL, g.tmFH, g.tmFL, g.a, tile, align_up(smem_raw, 1024), tmem);
 }
 
 template <bool BF, bool TWO>
@@ -1940,10 +1937,10 @@ static int lane_tables(FusedPlan* p, const double* chi, const double* phi, const
     return SFP_OK;
 }
 
-template <bool BF, bool TWO = false>
+template <bool BF>
 static cudaError_t set_smem_pair()
 {
-    return cudaFuncSetAttribute(k_fused_pair<BF, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(k_fused_pair<BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 FSmem<256, BF, false>::kBytes);
 }
 
@@ -2025,7 +2022,7 @@ static int classic_tables(FusedPlan* p, const double* chi, const double* phi, co
     if (rc) return SFP_ECUDA;
     cudaError_t e;
     if (p->two)
-        e = M == 512 ? set_smem_pair<true, true>() : M == 256 ? set_smem<256, true, true>() :
+        e = M == 512 ? set_smem_pair<true>() : M == 256 ? set_smem<256, true, true>() :
             M == 128 ? set_smem<128, true, true>() : set_smem<64, true, true>();
     else if (bf16)
         e = cudaSuccess;        // mode-keyed noise only, below
@@ -2160,7 +2157,7 @@ int fused_step(FusedPlan* p, const FusedArgs& args, cudaStream_t stream)
             at[0].val.clusterDim.z = 1;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            e = p->two ? cudaLaunchKernelEx(&cfg, k_fused_pair<true, true>, p->tmR, p->tmChiH, p->tmChiL, p->tmFH,
+            e = p->two ? cudaLaunchKernelEx(&cfg, k_fused_pair<true>, p->tmR, p->tmChiH, p->tmChiL, p->tmFH,
                                             p->tmFL, args)
                         : cudaLaunchKernelEx(&cfg, k_fused_pair<false>, p->tmR, p->tmChiH, p->tmChiL, p->tmFH,
                                              p->tmFL, args);

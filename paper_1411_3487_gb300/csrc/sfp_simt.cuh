@@ -9,44 +9,44 @@
 namespace sfp {
 
 // ---------------------------------------------------------------------------
-// Transform GEMM (NT):  Out[j][i] = sum_k In[j][k] * B[i][k]
+// FP64 transform GEMM (NT):  Out[j][i] = sum_k In[j][k] * B[i][k]
 //   inverse (Eq. e5):  In = R (k = p), B = chi  stored [n][p]  -> Out = u (bonds)
 //   forward (Eq. c4):  In = f|z (k = n), B = phi^T stored [p][n] -> Out = DeltaH|Z
 // Block tile BM rows x BN cols, K chunk BK; each thread owns TM x TN outputs.
 // Any J, Ncols, K (ragged tails are zero-filled).
 // ---------------------------------------------------------------------------
-template <typename T, int BM, int BN, int BK, int TM, int TN>
+template <int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
-k_gemm_nt(const T* __restrict__ In, const T* __restrict__ B, T* __restrict__ Out,
+k_gemm_nt(const double* __restrict__ In, const double* __restrict__ B, double* __restrict__ Out,
           int J, int Ncols, int K)
 {
     constexpr int NT = (BM / TM) * (BN / TN);
-    __shared__ T As[BK][BM + 1];
-    __shared__ T Bs[BK][BN + 1];
+    __shared__ double As[BK][BM + 1];
+    __shared__ double Bs[BK][BN + 1];
     const int tid = threadIdx.x;
     const int tx = tid % (BN / TN), ty = tid / (BN / TN);
     const int j0 = blockIdx.y * BM, i0 = blockIdx.x * BN;
-    T acc[TM][TN];
+    double acc[TM][TN];
 #pragma unroll
     for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < TN; ++b) acc[a][b] = T(0);
+        for (int b = 0; b < TN; ++b) acc[a][b] = 0.0;
 
     for (int k0 = 0; k0 < K; k0 += BK) {
         for (int e = tid; e < BM * BK; e += NT) {
             const int row = e / BK, kk = e % BK;
             const int gj = j0 + row, gk = k0 + kk;
-            As[kk][row] = (gj < J && gk < K) ? In[(size_t)gj * K + gk] : T(0);
+            As[kk][row] = (gj < J && gk < K) ? In[(size_t)gj * K + gk] : 0.0;
         }
         for (int e = tid; e < BN * BK; e += NT) {
             const int row = e / BK, kk = e % BK;
             const int gi = i0 + row, gk = k0 + kk;
-            Bs[kk][row] = (gi < Ncols && gk < K) ? B[(size_t)gi * K + gk] : T(0);
+            Bs[kk][row] = (gi < Ncols && gk < K) ? B[(size_t)gi * K + gk] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            T a[TM], b[TN];
+            double a[TM], b[TN];
 #pragma unroll
             for (int x = 0; x < TM; ++x) a[x] = As[kk][ty * TM + x];
 #pragma unroll
