@@ -40,10 +40,10 @@ extern "C" {
 #define SFP_ETIMEDOUT  -4   /* a bounded device wait gave up (every wait of the
                                tensor-core kernels and of the FP64 step of a few
                                chains is limited to 1 s; the kernel then returns
-                               without advancing the step counters and the
-                               context stays usable; with SFP_TEST_STALL=1 in
-                               the environment both stall on purpose, to test
-                               this) */
+                               and the context stays usable; the fused and the
+                               FP64 step leave the chain's step counter as it
+                               was; with SFP_TEST_STALL=1 in the environment both
+                               stall on purpose, to test this) */
 #define SFP_ENONFINITE -5   /* a chain's state became non-finite */
 #define SFP_ENOTSUP    -6   /* valid request that the library does not support */
 

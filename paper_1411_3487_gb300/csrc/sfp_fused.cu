@@ -113,9 +113,9 @@ static_assert(2 + kComputeWarps == 10 && kComputeWarps == 8, "warp numbering of 
 // over it.  The single-CTA kernel stages R on its own at 64 and 128 beads
 // (four stages either way) and in place at 256 beads, where that gives four
 // stages of 48 KB instead of three of 64 KB (24.2 -> 23.1 us per step at
-// 4096 x 256 bp with three passes, which are the lane step's now; with mode-keyed noise, whose steps have no noise blocks,
-// three stages stay faster: 24.0 against 24.5 us); the 512-bead kernel splits
-// in place.
+// 4096 x 256 bp with three passes, which are the lane step's now; with mode-keyed
+// noise, whose steps have no noise blocks, three stages stay faster: 24.0 against
+// 24.5 us); the 512-bead kernel splits in place.
 template <int NB, bool BF, bool MZ = false> constexpr bool kRS = BF && (NB != 256 || MZ);
 // Mirror symmetry (TF32, 128 and 256 beads): chi_{n,p} and phi_{n,p} are even or odd
 // under n -> M - n and n -> M - 1 - n with the parity of p, so each contraction splits

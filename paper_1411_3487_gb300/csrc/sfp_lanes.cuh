@@ -36,10 +36,12 @@
 // three of eight batches of chains find no room there and live in global memory (L2),
 // read and written by the thread that owns the modes.
 //
-// What bounds it (256 beads, 28 chains): about 38 K warp instructions a step at two
-// per cycle, 168 warps' worth of Philox calls more than half of them; a chain of 5.3
-// us a step with one chain per tile (inverse and forward MMAs 3000 cycles each, force,
-// update and four hand-overs).  State and D live in 504 of the 512 TMEM columns.
+// What bounds it (256 beads, 28 chains): the chain of a step, 5.3 us with one chain per
+// tile (inverse and forward MMAs 3000 cycles each, force, update and four hand-overs),
+// stretched by what shares the SM with it: 42.8 K warp instructions a step at 2.5 a
+// cycle, the normals' more than half.  Neither pipe is full: a capture of three steps
+// shows the issue slots 46 % busy and the tensor pipe 30 % active.  State and D live in
+// 504 of the 512 TMEM columns.
 // 512 beads (a cluster of two CTAs): the parities of the mirror symmetry are 256 modes
 // each, two row tiles of 128, and CTA rank r takes parity r, so that its operand, its
 // share of the state and its table stream are what one CTA holds at 256 beads.  Bonds are
@@ -57,8 +59,8 @@
 //
 // Measured (GB300, us a step in a 400-step call, the four-role kernel of sfp_fused.cu
 // before -> here): 4096 x 256 bp 22.7 -> 8.9, 8 x 256 bp 19.1 -> 5.2, 4096 x 128 bp
-// 10.3 -> 4.3, 50 x 128 bp 9.5 -> 2.7, 4096 x 64 bp 7.3 -> 2.3, 8 x 64 bp 5.9 -> 1.5; 16384 x 512 bp 289 ->
-// 130 (here 1000 x 512 bp take 11.8, one chain 10.0).
+// 10.3 -> 4.3, 50 x 128 bp 9.5 -> 2.7, 4096 x 64 bp 7.3 -> 2.4, 8 x 64 bp 5.9 -> 1.5; 16384 x 512 bp 289 ->
+// 132 (here 1000 x 512 bp take 11.9, one chain 10.0).
 #pragma once
 #include <cstdint>
 #include <cuda_bf16.h>

@@ -530,8 +530,9 @@ k_mode_update(T* __restrict__ R, const T* __restrict__ DH, const T* __restrict__
 // the parity of p, so every sum runs over half the indices: thread 2 i + e sums the
 // modes of parity e, its neighbour the others, and the two take bonds i and M - i (bond
 // M / 2 its own image, in the place of bond 0); the forces come back as v_i -+ v_{M-i},
-// the normals as z_n +- z_{M-1-n}.  FP64 issue bounds the kernel (64 FMA lanes per SM
-// and a few cycles): 512 chains of 128 beads 164 us a step without, 96 with; 200 of 256 beads 308 and 167.
+// the normals as z_n +- z_{M-1-n}.  FP64 issue bounds the kernel (about 60 cycles a warp
+// instruction on a sub-partition): 512 chains of 128 beads 164 us a step without, 96
+// with; 200 of 256 beads 308 and 167.
 // ---------------------------------------------------------------------------
 template <typename T, bool FOLD>
 __global__ void __launch_bounds__(256)
@@ -716,7 +717,7 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 // The FP64 Box-Muller of a Philox call is a long dependent chain (~5 us), so the
 // normals come from a separate kernel that draws every call of every step at once.
 // One chain, us a step (cluster barriers, tables and normals from L2 before -> here): 64
-// beads 6.6 -> 3.1, 128 11.8 -> 7.5, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
+// beads 6.6 -> 3.2, 128 11.8 -> 7.6, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
 // Every wait is bounded; after a timeout the CTA raises bit 1 of the error word, its
 // threads run through the remaining steps without sending or arming anything, and no CTA of the
 // cluster writes anything back: the chain is as it was before the launch.
@@ -928,7 +929,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
 }
 
 // The cluster step of chains whose tables no CTA's shared memory holds (more than 352
-// beads on 16 CTAs): bound by FP64 issue and by the tables from L2 rather than by
+// beads on 16 CTAs), or whose clusters would not all fit on the GPU with them: bound by FP64 issue and by the tables from L2 rather than by
 // latency.  Q threads share the sums of one bond or mode, all three axes (Q a power of 2
 // within a warp; neighbouring groups read neighbouring table entries), and the groups are
 // dealt round-robin over the four warps, so that all four sub-partitions have FP64 work;
