@@ -717,7 +717,7 @@ k_chain_steps(T* __restrict__ Rg, double* __restrict__ com, int64_t* __restrict_
 // The FP64 Box-Muller of a Philox call is a long dependent chain (~5 us), so the
 // normals come from a separate kernel that draws every call of every step at once.
 // One chain, us a step (cluster barriers, tables and normals from L2 before -> here): 64
-// beads 6.6 -> 3.2, 128 11.8 -> 7.6, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
+// beads 6.6 -> 3.2, 128 11.8 -> 7.5, 256 29.4 -> 22.0; 8 chains of 64 beads 9.1 -> 4.5.
 // Every wait is bounded; after a timeout the CTA raises bit 1 of the error word, its
 // threads run through the remaining steps without sending or arming anything, and no CTA of the
 // cluster writes anything back: the chain is as it was before the launch.
@@ -748,11 +748,15 @@ __device__ __forceinline__ double sum8(double x)
 }
 
 // Shared memory of a CTA: R and v ([3][M + 8]: the axes in different banks), the normals
-// of two steps, the tables of the owned bonds and modes and their dm, g, h, w.
+// of two steps, the tables of the owned bonds and modes and their dm, g, h, w.  Rows of
+// the tables are a multiple of 8 long, and all rows zero from M on, so that the eight
+// lanes of a sum take the same number of terms (with one more in some of them a warp runs
+// the loop's two forms in turn: one chain of 63 beads 3.8 us a step as it is, 4.7 then).
+__host__ __device__ constexpr int chain_cluster_pitch(int M) { return (M + 7) & ~7; }
 constexpr size_t chain_cluster_bytes(int M, int G)
 {
     const size_t S = (size_t)(M + G - 1) / G;
-    return 8 * (12 * (size_t)(M + 8) + S * (3 * (size_t)M + 4));
+    return 8 * (12 * (size_t)(M + 8) + S * (3 * (size_t)chain_cluster_pitch(M) + 4));
 }
 
 template <int G>
@@ -765,11 +769,11 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
                 int mode_noise, int* __restrict__ bad, int stall_test)
 {
     extern __shared__ unsigned char chain_smem[];
-    const int P = M + 8;
+    const int P = M + 8, MP = chain_cluster_pitch(M);
     double* sR = reinterpret_cast<double*>(chain_smem);   // [3][P]
     double* sv = sR + 3 * P;                              // [3][P]
     double* sz = sv + 3 * P;                              // [2][3][P]
-    double* tab = sz + 6 * P;                             // [S][3][M] chi_n, chi_p, phi_p; [S] dm, g, h, w (w0_cm)
+    double* tab = sz + 6 * P;                             // [S][3][MP] chi_n, chi_p, phi_p; [S] dm, g, h, w (w0_cm)
     __shared__ uint64_t v_in, r_in;                       // v, R of every CTA have arrived (1 + tx)
     __shared__ uint64_t never;                            // nothing arrives here (the stall test)
     __shared__ int s_abort;
@@ -785,7 +789,7 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     const bool owns = wid < nown;                         // this warp does (uniform; warp 0 of every owner)
     // every warp runs the same passes over the owned bonds / modes
     const int passes = (nown + nwarp - 1) / nwarp;
-    double* tdm = tab + (size_t)S * 3 * M;
+    double* tdm = tab + (size_t)S * 3 * MP;
     double *tg = tdm + S, *th = tg + S, *tw = th + S;
     double* Rc = Rg + (size_t)c * 3 * M;
     for (int i = threadIdx.x; i < 3 * M; i += blockDim.x) sR[i / M * P + i % M] = Rc[i];
@@ -793,15 +797,18 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
     // with loads through registers); phi by columns: a bead's owned modes lie side by side
     for (int o = wid; o < nown; o += nwarp)
         for (int k = lane; k < M; k += 32) {
-            copy_async8(tab + (size_t)o * 3 * M + k, chi + (size_t)(lo + o) * M + k);
-            copy_async8(tab + (size_t)(o * 3 + 1) * M + k, chiT + (size_t)(lo + o) * M + k);
+            copy_async8(tab + (size_t)o * 3 * MP + k, chi + (size_t)(lo + o) * M + k);
+            copy_async8(tab + (size_t)(o * 3 + 1) * MP + k, chiT + (size_t)(lo + o) * M + k);
         }
     for (int i = threadIdx.x, o = i % max(nown, 1), k = i / max(nown, 1); i < nown * M; i += blockDim.x) {
-        copy_async8(tab + (size_t)(o * 3 + 2) * M + k, phi + (size_t)k * M + lo + o);
+        copy_async8(tab + (size_t)(o * 3 + 2) * MP + k, phi + (size_t)k * M + lo + o);
         o += (int)blockDim.x;
         k += o / nown;
         o %= nown;
     }
+    for (int i = threadIdx.x; i < 12 * 8; i += blockDim.x) sR[(i >> 3) * P + M + (i & 7)] = 0.0;     // R, v, normals
+    for (int i = threadIdx.x; i < 3 * nown * 8; i += blockDim.x)
+        if (M + (i & 7) < MP) tab[(size_t)(i >> 3) * MP + M + (i & 7)] = 0.0;
     for (int i = threadIdx.x; i < nown; i += blockDim.x) {
         tdm[i] = dm[lo + i];
         tg[i] = g[lo + i];
@@ -840,10 +847,10 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             const int gi = pass * nwarp + wid;
             if (gi >= nown) break;                      // the whole warp
             const int n = lo + gi;
-            const double* t = tab + (size_t)gi * 3 * M;
+            const double* t = tab + (size_t)gi * 3 * MP;
             double u = 0.0;
 #pragma unroll 8
-            for (int p = j; p < M; p += 8) u = fma(t[p], sR[ax * P + p], u);       // chi_{n,0} = 0
+            for (int p = j; p < MP; p += 8) u = fma(t[p], sR[ax * P + p], u);       // chi_{n,0} = 0
             u = sum8(u);
             const double u0 = __shfl_sync(0xffffffffu, u, 0), u1 = __shfl_sync(0xffffffffu, u, 8),
                          u2 = __shfl_sync(0xffffffffu, u, 16);
@@ -862,9 +869,9 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             if (mode_noise) {
                 if (j == 0) x = z[ax * P + p];
             } else {
-                const double* t = tab + ((size_t)gi * 3 + 2) * M;
+                const double* t = tab + ((size_t)gi * 3 + 2) * MP;
 #pragma unroll 8
-                for (int n = j; n < M; n += 8) x = fma(t[n], z[ax * P + n], x);
+                for (int n = j; n < MP; n += 8) x = fma(t[n], z[ax * P + n], x);
             }
             return tw[gi] * x;
         };
@@ -879,12 +886,12 @@ k_chain_cluster(double* __restrict__ Rg, double* __restrict__ com, int64_t* __re
             const int gi = pass * nwarp + wid;
             if (gi >= nown) break;
             const int p = lo + gi;
-            const double* t = tab + ((size_t)gi * 3 + 1) * M;
+            const double* t = tab + ((size_t)gi * 3 + 1) * MP;
             const double r = sR[ax * P + p], ry = sR[P + p];
             double d = 0.0;
             if (p > 0)                  // mode 0 takes no force, and nobody waits for its warp's read
 #pragma unroll 8
-                for (int n = j; n < M; n += 8) d = fma(t[n], sv[ax * P + n], d);
+                for (int n = j; n < MP; n += 8) d = fma(t[n], sv[ax * P + n], d);
             d = sum8(fma(th[gi], d, pass == 0 ? x0 : noise(gi)));
             if (p == 0) {
                 // centre of mass (zeta_0 = 0, Eq. d6 limit; w0_cm = w_0 / sqrt(M)), shear on x
