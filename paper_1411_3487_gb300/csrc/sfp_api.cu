@@ -632,7 +632,9 @@ cudaError_t launch_chain_cluster(sfp_batch* b, Group& g, int G, double c12, doub
 // 15 of 184 beads 26.1 and 38.7, 16 of them 51.3 and 45.3).  From 257 beads a warp of the
 // kernel with L2 tables takes two bonds in turn on 16 CTAs, and up to 320 two rounds of
 // the other are still ahead (9 chains of 257 beads 56.4 and 61.8, of 320 65.2 and 77.6, of
-// 321 79.1 and 76.0).
+// 321 79.1 and 76.0).  Clusters of 8 that share SMs (from 16 chains) are a little behind at
+// 14 and 16 bonds a CTA (16 chains of 104 beads 16.7 and 17.2, of 105 18.3 and 17.7, of 113
+// 18.6 and 18.7, of 121 20.7 and 19.9, of 128 20.7 and 20.0, of 129 24.5 and 32.6).
 void choose_chain_cluster(Group& g, int sms)
 {
     g.chain_g = 0;
@@ -646,12 +648,19 @@ void choose_chain_cluster(Group& g, int sms)
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute at;
             chain_cluster_config(&cfg, &at, G, g.C, smem, nullptr);
-            int n = 0;          // clusters that the GPU holds at once
+            int n = 0, alone = 0;       // clusters that the GPU holds at once, and without sharing an SM
             if ((G == 16 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
                 allow_shared(fn, smem, most) != cudaSuccess ||
                 cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 n = 0;
+            }
+            const int S = (g.M + G - 1) / G;        // bonds of a CTA
+            if (tab && G == 8 && (S == 14 || S == 16)) {
+                cfg.dynamicSmemBytes = kChainClusterBytes;
+                if (allow_shared(fn, kChainClusterBytes, most) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&alone, fn, &cfg) == cudaSuccess && g.C > alone)
+                    continue;
             }
             if (n >= (tab && !(g.M > 256 && g.M <= 320) ? g.C : 1)) {
                 g.chain_g = G;

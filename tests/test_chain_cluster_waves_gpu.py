@@ -34,7 +34,7 @@ def test_one_chain_more_does_not_double_the_time(M, C):
     assert seconds(M, C + 1) < 1.8 * seconds(M, C)
 
 
-@pytest.mark.parametrize("M,C", [(256, 7), (256, 8), (184, 15), (184, 16), (320, 9), (321, 9)])
+@pytest.mark.parametrize("M,C", [(256, 7), (256, 8), (184, 15), (184, 16), (320, 9), (321, 9), (104, 16), (105, 16), (121, 15), (121, 16)])
 def test_each_form_matches_one_cta_per_chain(M, C, n=9):
     def run(C):
         with batch(M, C) as b:
